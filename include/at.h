@@ -12,10 +12,10 @@
  *
  * On the GPU the subdomains are processed by the CTAs of one persistent,
  * cooperatively launched kernel.  Halo values travel through a ring buffer of
- * past boundary values in device memory with one progress flag per
- * subdomain face (the device counterpart of the notified puts and circular
- * receive buffers of Algorithm 2), so CTAs run ahead of one another by up to
- * L steps without a grid-wide barrier.  AT_SYNC instead puts a grid barrier
+ * past boundary values in device memory whose entries carry their level (3D:
+ * with one progress flag per subdomain face; the device counterpart of the
+ * notified puts and circular receive buffers of Algorithm 2), so CTAs run
+ * ahead of one another by up to L steps without a grid-wide barrier.  AT_SYNC instead puts a grid barrier
  * after every step (Algorithm 1).
  *
  * Memory and ownership.  The library never allocates device memory.  The
@@ -71,9 +71,9 @@ extern "C" {
 /* at_grid.flags */
 #define AT_FLAG_PER_SUBDOMAIN_DELAY 1  /* SEEDED: one draw for both faces       */
 #define AT_FLAG_ALLOW_UNSTABLE      2  /* skip the stability check of at_create */
-#define AT_FLAG_TEST_SKIP_PUBLISH   4  /* test only: CTA 0 stops publishing its
-                                          progress flags after level test_skip_step,
-                                          so that its neighbours' waits time out
+#define AT_FLAG_TEST_SKIP_PUBLISH   4  /* test only: CTA 0 stops publishing to other
+                                          elements after level test_skip_step, so
+                                          that its neighbours' waits time out
                                           (1D: its first warp; 3D: its subdomains) */
 #define AT_FLAG_VISCOUS_FP64        8  /* FP32 state: form the viscous term nu dt D2 u
                                           and add it to u in FP64 (one rounding per
@@ -360,7 +360,7 @@ int at_step_levels(at_solver *h, int64_t n_steps, int delay_mode, int8_t *delays
 /* Restarts the solver at time level `level` from stored full fields: levels
  * + (l mod depth) * N words must hold level l for l = max(0, level-L-s+1) ..
  * level (s = 2 for order 2, 3 for order 4: the oldest level the next step's
- * halos read).  Sets the state, the ring buffers and every progress flag;
+ * halos read).  Sets the state and the ring buffers;
  * clears the device status.  Stream-ordered. */
 int at_set_history(at_solver *h, const void *levels, int64_t depth, int64_t level);
 
@@ -404,7 +404,7 @@ int at_adjoint(at_solver *h, int64_t n_steps, int delay_mode, const int8_t *dela
 int at_fma_peak(int dtype, int64_t trips, double *fma_per_s);
 
 /* Size in bytes of the fixed scratch array used by at_step_noalloc(). */
-#define AT_NOALLOC_SCRATCH_BYTES (8u * 1024u * 1024u)
+#define AT_NOALLOC_SCRATCH_BYTES (16u * 1024u * 1024u)
 
 /* at_step_noalloc -- the same run as at_create + at_set_state + at_step +
  * at_status, for callers that cannot allocate device memory (for example a
@@ -420,11 +420,11 @@ int at_fma_peak(int dtype, int64_t trips, double *fma_per_s);
  *
  * Memory.  Nothing is allocated, on the device or on the host: the ring
  * buffers, progress flags, status word and counters live in one array of
- * AT_NOALLOC_SCRATCH_BYTES (8 MiB) that this library places in the device
+ * AT_NOALLOC_SCRATCH_BYTES (16 MiB) that this library places in the device
  * memory of every GPU that loads it and keeps until the process exits.  A
- * problem whose scratch would not fit -- roughly 32 T + 16 bytes per
- * subdomain with T = 8 or 16 ring slots, i.e. up to about 15,000 subdomains at
- * order 4 and L = 3 -- is rejected with AT_ERR_ARG and a message giving both
+ * problem whose scratch would not fit -- 32 T bytes per
+ * subdomain (FP64 at order 4: 64 T) with T = 8 or 16 ring slots, i.e. up to
+ * about 32,000 (16,000) subdomains at order 4 and L = 3 -- is rejected with AT_ERR_ARG and a message giving both
  * sizes.
  *
  * Sharing.  All calls on a device share that one array, and it keeps what the

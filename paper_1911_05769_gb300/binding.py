@@ -42,7 +42,7 @@ AT_FLAG_VISCOUS_FP64 = 8
 AT_FLAG_VISCOUS_FP32 = 16
 AT_FLAG_COMPENSATED = 32
 
-AT_NOALLOC_SCRATCH_BYTES = 8 * 1024 * 1024
+AT_NOALLOC_SCRATCH_BYTES = 16 * 1024 * 1024
 
 
 class at_grid(ctypes.Structure):

@@ -82,18 +82,24 @@ struct Layout {
     size_t u, ring, flag, ctrl, hist, gbar, bsub, binst, ur, strip, tiles, order, total;
 };
 
-// Workspace: state, ring buffers [T][P][2], flags [P][2], control block,
-// delay counts, barrier counter; for an ensemble (n_inst > 0) also the
-// subdomain and instance records.
-Layout layout(int64_t N, int64_t P, int w, int L, int T, int64_t n_inst = 0, bool comp = false, bool strips = true)
+// 16-byte halves of a ring entry (atk::entry_halves): R words (a compensated
+// state: hi and lo words) at 8 bytes of payload each.
+int entry_halves(int w, int R, bool comp) { return w * R * (comp ? 2 : 1) > 8 ? 2 : 1; }
+
+// Workspace: state, ring buffers [T][P][2], control block, delay counts,
+// barrier counter; for an ensemble (n_inst > 0) also the subdomain and
+// instance records.
+Layout layout(int64_t N, int64_t P, int w, int R, int L, int T, int64_t n_inst = 0, bool comp = false,
+              bool strips = true)
 {
     Layout l{};
     size_t off = 0;
     l.u = off;    off = align_up(off + (size_t)N * w, 256);
     l.ur = off;   // compensated state: the rounding error of every point
     if (comp) off = align_up(off + (size_t)N * w, 256);
-    l.ring = off; off = align_up(off + (size_t)T * P * 2 * atk::kRingEntry, 256);
-    l.flag = off; off = align_up(off + (size_t)P * 2 * 8, 256);
+    l.ring = off;
+    off = align_up(off + (size_t)T * P * 2 * atk::kRingHalf * entry_halves(w, R, comp), 256);
+    l.flag = off;   // (3D only)
     l.ctrl = off; off = align_up(off + atk::kCtrlWords * 4, 256);
     l.hist = off; off = align_up(off + (size_t)(L + 1) * 8, 256);
     l.gbar = off; off = align_up(off + 8, 256);
@@ -211,6 +217,17 @@ int groups_per_lane(int64_t M)
     return g;
 }
 
+// Whether every lane of the stepper that holds points of a tile of M points
+// holds gw whole groups (then the run length is a compile-time constant); else
+// the lanes hold gpl = ceil(M / 128) groups and the last one fewer.
+bool full_runs(int64_t M, int gw) { return (M / 4) % gw == 0 && (M / 4 + 31) / 32 == gw; }
+
+int run_groups(int64_t M)
+{
+    const int gw = groups_per_lane(M);
+    return full_runs(M, gw) ? gw : (int)((M / 4 + 31) / 32);
+}
+
 // Whether an FP32-state solver accumulates the viscous term in FP64: forced
 // by the flags, else when nu dt / dx^2 reaches 0.8 of the stability limit.
 bool viscous_fp64(int w, int order, uint32_t flags, double D)
@@ -228,7 +245,7 @@ void pick_kernels(int w, int order, int64_t M, bool forced, bool v64, bool comp,
                   void **stepper_bs = nullptr)
 {
     const int gw = groups_per_lane(M);
-    const bool full = (M == 128LL * gw);
+    const bool full = full_runs(M, gw);
     void *bs = nullptr;
     if (w == 8) {
         *stepper = atk_stepper_kernel_f64(order, gw, forced, full);
@@ -260,15 +277,28 @@ struct TabSize {
 TabSize tab_size(int64_t M, int w, bool forced, bool batch, bool comp = false, int64_t ntk = 0, int k = 1)
 {
     if (batch) return {0, (long long)sizeof(atk::BatchSub), comp, 0, ntk, k};
-    if (forced) return {2LL * M * w, 2LL * w, comp, 2, 0, 1};
+    if (forced)
+        return {2LL * atk::tile_points(M, groups_per_lane(M), full_runs(M, groups_per_lane(M))) * w, 2LL * w, comp, 2, 0, 1};
     return {0, 0, comp, 0, 0, 1};
+}
+
+// Lets a kernel take all the dynamic shared memory its static one leaves.
+// (The limit belongs to the kernel, not to a solver: a smaller one set for one
+// solver would fail another's launches.)
+cudaError_t allow_smem(const void *kernel, int smem_optin)
+{
+    cudaFuncAttributes a{};
+    const cudaError_t e = cudaFuncGetAttributes(&a, kernel);
+    if (e != cudaSuccess) return e;
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                smem_optin - (int)a.sharedSizeBytes);
 }
 
 // Chooses the CTA count (all co-resident CTAs unless max_ctas is set, at most
 // one PE per subdomain) and the stages per PE that fit in shared memory, and
 // sets the kernel's dynamic shared-memory size.
-int launch_shape(int64_t M, int w, int64_t P, TabSize tsz, int max_ctas, int stages, int sms, int smem_optin,
-                 void *kernel, int *G_out, int *stages_out, atk::SmemLayout *sl_out, int *smem_out,
+int launch_shape(int64_t M, int w, int64_t P, TabSize tsz, int max_ctas, int stages, bool stages_given, int sms,
+                 int smem_optin, void *kernel, int *G_out, int *stages_out, atk::SmemLayout *sl_out, int *smem_out,
                  long long *smax_out)
 {
     if (M < 4 || M > atk::kMaxM) return fail(AT_ERR_ARG, "tile of %lld points (4..%d)", (long long)M, atk::kMaxM);
@@ -282,27 +312,64 @@ int launch_shape(int64_t M, int w, int64_t P, TabSize tsz, int max_ctas, int sta
             if (sk > *smax) *smax = sk;
         }
         const long long tab = tsz.fixed + (long long)atk::kWarps * (*smax + tsz.extra) * tsz.per_sub;
-        return atk::smem_layout(M, w, st, tab, tsz.comp);
+        const int gw = groups_per_lane(M);
+        return atk::smem_layout(atk::tile_points(M, gw, full_runs(M, gw)), w, st, tab, tsz.comp);
     };
-    // CTAs needed for one PE per subdomain at most
-    const int gmax = (int)((P + atk::kWarps - 1) / atk::kWarps);
+    // at most one CTA per subdomain: with few subdomains every CTA holds one
+    // (spread over the SMs, so that the subdomains share no SM's pipes) instead
+    // of kWarps (16 subdomains of 256 FP64 points: 0.5 us of FP64 pipe a step
+    // on 16 SMs, 2 us on 4).
+    const int gmax = (int)(P < (1LL << 30) ? P : (1LL << 30));
     int G = max_ctas > 0 ? max_ctas : sms;
     if (G > gmax) G = gmax;
     long long smax = 0;
     while (stages > atk::kMinStages && layout_for(G, stages, &smax).total > smem_optin) --stages;
     atk::SmemLayout sl = layout_for(G, stages, &smax);
     if (sl.total > smem_optin) return fail(AT_ERR_RESIDENCY, "shared memory %lld exceeds %d", sl.total, smem_optin);
-    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sl.total);
+    cudaError_t e = allow_smem(kernel, smem_optin);
     if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute");
     int occ = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kernel, atk::kThreads, (size_t)sl.total);
+    auto occupancy = [&](long long bytes, int *o) {
+        return cudaOccupancyMaxActiveBlocksPerMultiprocessor(o, kernel, atk::kThreads, (size_t)bytes);
+    };
+    e = occupancy(sl.total, &occ);
     if (e != cudaSuccess) return cuda_fail(e, "cudaOccupancyMaxActiveBlocksPerMultiprocessor");
-    if (max_ctas <= 0 && occ > 1) {
-        // all co-resident CTAs (fewer subdomains per PE only shrinks the tables)
-        int want = occ * sms;
-        if (want > gmax) want = gmax;
-        long long sm2 = 0;
-        if (layout_for(want, stages, &sm2).total <= sl.total) { G = want; sl = layout_for(G, stages, &smax); }
+    if (max_ctas <= 0) {
+        // all co-resident CTAs.  More CTAs hold fewer subdomains each, and so
+        // smaller tables: raise the count while the tables of that count fit
+        // one more per SM.  A third tile buffer is given up for a CTA more per
+        // SM (2048-instance ensemble: 2 CTAs of 3 buffers 4.36 ms,
+        // 3 CTAs of 2 buffers 3.41 ms for 100 steps)
+        auto fit = [&](int st, int from, int *G_fit) -> cudaError_t {
+            int per = from;
+            for (;;) {
+                const int64_t want = (int64_t)(per + 1) * sms;
+                long long sm2 = 0;
+                int o = 0;
+                const long long bytes = layout_for(want < gmax ? (int)want : gmax, st, &sm2).total;
+                if (bytes > smem_optin) break;
+                const cudaError_t r = occupancy(bytes, &o);
+                if (r != cudaSuccess) return r;
+                if (o < per + 1) break;
+                ++per;
+                if (want >= gmax) break;
+            }
+            const int64_t want = (int64_t)per * sms;
+            *G_fit = want < gmax ? (int)want : gmax;
+            return cudaSuccess;
+        };
+        int Gs = 0;
+        e = fit(stages, 0, &Gs);
+        if (e == cudaSuccess && !stages_given && stages > 2) {
+            int G2 = 0;
+            e = fit(2, 0, &G2);
+            if (e == cudaSuccess && G2 > Gs) { Gs = G2; stages = 2; }
+        }
+        if (e != cudaSuccess) return cuda_fail(e, "cudaOccupancyMaxActiveBlocksPerMultiprocessor");
+        if (Gs > 0) G = Gs;
+        sl = layout_for(G, stages, &smax);
+        e = occupancy(sl.total, &occ);
+        if (e != cudaSuccess) return cuda_fail(e, "cudaOccupancyMaxActiveBlocksPerMultiprocessor");
     }
     if (occ < 1 || (int64_t)occ * sms < G)
         return fail(AT_ERR_RESIDENCY, "%d CTAs cannot be co-resident (occupancy %d per SM)", G, occ);
@@ -326,10 +393,10 @@ struct at_solver {
     cudaStream_t stream;
     int device, sm_count, smem_optin;
     int G, stages, sb, smem;
+    int gpl;                   // 1D: groups of 4 points per lane of a tile
     long long smax;
     atk::SmemLayout sl;
     int64_t step;              // steps launched since at_set_state (host count)
-    int64_t flags_E;           // PEs of the launch that last released flags (0: none since the state was set)
     bool has_state;
     int dim;                   // 1 or 3
     Dims3 d3;                  // 3D: extents, subdomains, ring entry size
@@ -347,7 +414,6 @@ struct at_solver {
     int64_t ntiles_k;          // ensembles: tiles of that list
     std::vector<atk::BatchSub> bsub_host;   // ensembles: the subdomain records (tile planning)
     std::vector<at_instance> inst_host;     // ensembles: the instances
-    const void *flags_list;    // tile list of the launch that last released flags
     void *kernel;
     void *kernel_bs;           // the blocked synchronous mode's kernel (NULL: none)
     void *kernel_b3;           // 3D: the blocked free-running kernel (NULL: none)
@@ -358,35 +424,12 @@ struct at_solver {
 
 namespace {
 
-// Sets every progress flag to the level of the state.  A launch releases
-// only the flags of faces between processing elements; after a launch with
-// another partition of the subdomains (another CTA count) the flags of faces
-// that were inside a PE are stale, while every level up to the state's is
-// complete and its ring entries are written (entries go out on every face).
-__global__ void at_flags_to_level(unsigned long long *flag, const int *ctrl, long long nflags)
-{
-    const long long n0 = *reinterpret_cast<const long long *>(ctrl + atk::kCtrlN0);
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < nflags;
-         i += (long long)gridDim.x * blockDim.x)
-        flag[i] = (unsigned long long)n0;
-}
-
 // One launch of the persistent stepper: cooperative, so that every CTA is
 // resident; cudaLaunchKernelExC with the cooperative attribute may be
-// captured into a CUDA graph.  Brings the flags up to date first when the
-// partition into PEs differs from the previous launch's.
+// captured into a CUDA graph.  (Ring entries carry their levels, so a launch
+// may partition the subdomains into PEs differently from the one before.)
 cudaError_t launch_stepper(at_solver *h, atk::Params *p, void *kernel)
 {
-    const int64_t E = (int64_t)h->G * atk::kWarps;
-    if (h->flags_E != 0 && (h->flags_E != E || h->flags_list != (const void *)p->tiles)) {
-        const long long nflags = h->P * 2;
-        const int blocks = (int)((nflags + 255) / 256 < 1024 ? (nflags + 255) / 256 : 1024);
-        at_flags_to_level<<<blocks, 256, 0, h->stream>>>(p->flag, p->ctrl, nflags);
-        const cudaError_t e = cudaGetLastError();
-        if (e != cudaSuccess) return e;
-    }
-    h->flags_E = E;
-    h->flags_list = p->tiles;
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(h->G);
     cfg.blockDim = dim3(atk::kThreads);
@@ -408,7 +451,7 @@ void prepare_bs(at_solver *h)
 {
     h->bs_ok = false;
     if (!h->kernel_bs) return;
-    if (cudaFuncSetAttribute(h->kernel_bs, cudaFuncAttributeMaxDynamicSharedMemorySize, h->smem) != cudaSuccess) {
+    if (allow_smem(h->kernel_bs, h->smem_optin) != cudaSuccess) {
         cudaGetLastError();
         return;
     }
@@ -493,8 +536,11 @@ int set_tile_plan(at_solver *h, int K)
     if (e != cudaSuccess) return cuda_fail(e, "copying the tile lists");
     h->K = K;
     h->ntiles_k = (int64_t)tp.listk.size();
+    // (tiles of K > 1 subdomains: M is a multiple of a lane's 4 gw points, so
+    // the runs are full also where a tile holds fewer than K)
     const int gw = groups_per_lane((int64_t)K * h->M);
-    const bool full = K == 1 && h->M == 128LL * gw;
+    const bool full = K > 1 || full_runs(h->M, gw);
+    h->gpl = full ? gw : (int)((h->M / 4 + 31) / 32);
     const int order = h->order;
     h->kernel = h->w == 8 ? atk_batch_kernel_f64(order, gw, full)
                 : h->comp ? atk_batch_kernel_f32c(order, gw, full)
@@ -502,7 +548,6 @@ int set_tile_plan(at_solver *h, int K)
     h->kernel_bs = h->w == 8 ? atk_sync_batch_kernel_f64(order, gw, full)
                    : h->comp ? nullptr
                              : atk_sync_batch_kernel_f32(order, gw, full);
-    h->flags_list = nullptr;
     return AT_OK;
 }
 
@@ -522,7 +567,7 @@ size_t at_workspace_bytes(const at_grid *grid, int64_t P, int scheme_order, int 
         check_args3(grid, P, scheme_order, L, &d);
         return layout3(d, P, w, L, ring_slots(L, s), 1).total;
     }
-    return layout(grid->n[0], P, w, L, ring_slots(L, s), 0, (grid->flags & AT_FLAG_COMPENSATED) != 0).total;
+    return layout(grid->n[0], P, w, s - 1, L, ring_slots(L, s), 0, (grid->flags & AT_FLAG_COMPENSATED) != 0).total;
 }
 
 // nf = 1: the scalar equation with viscosity kappa[0]; nf = 3..5: the system
@@ -735,7 +780,7 @@ int at_create(const at_grid *grid, int64_t P, int scheme_order, int L, double nu
     const bool comp = (grid->flags & AT_FLAG_COMPENSATED) != 0;
     if (comp && (w != 4 || (grid->flags & AT_FLAG_VISCOUS_FP64)))
         return fail(AT_ERR_ARG, "AT_FLAG_COMPENSATED needs FP32 state and excludes AT_FLAG_VISCOUS_FP64");
-    const Layout lay = layout(N, P, w, L, T, 0, comp);
+    const Layout lay = layout(N, P, w, scheme_order / 2, L, T, 0, comp);
     if (!grid->workspace) return fail(AT_ERR_ARG, "workspace is NULL");
     if (grid->workspace_bytes < lay.total)
         return fail(AT_ERR_ARG, "workspace too small: %zu < %zu", grid->workspace_bytes, lay.total);
@@ -767,6 +812,7 @@ int at_create(const at_grid *grid, int64_t P, int scheme_order, int L, double nu
 
     pick_kernels(w, scheme_order, h->M, grid->forcing_amp != 0.0, h->v64, h->comp, &h->kernel, &h->init_kernel,
                  &h->kernel_bs);
+    h->gpl = run_groups(h->M);
 
     // launch shape: by default as many CTAs of kWarps processing elements
     // (warps) as can be resident, at most one PE per subdomain; `stages`
@@ -775,7 +821,7 @@ int at_create(const at_grid *grid, int64_t P, int scheme_order, int L, double nu
     int stages = grid->stages > 0 ? grid->stages : 3;
     if (stages < atk::kMinStages) stages = atk::kMinStages;
     int rc2 = launch_shape(h->M, w, P, tab_size(h->M, w, grid->forcing_amp != 0.0, false, comp), grid->max_ctas,
-                           stages, sms, smem_optin, h->kernel, &h->G, &h->stages, &h->sl, &h->smem, &h->smax);
+                           stages, grid->stages > 0, sms, smem_optin, h->kernel, &h->G, &h->stages, &h->sl, &h->smem, &h->smax);
     if (rc2 != AT_OK) { delete h; return rc2; }
     prepare_bs(h);
     h->sb = sb;
@@ -790,7 +836,7 @@ static atk::Params make_params(const at_solver *h)
     atk::Params p{};
     p.u = h->ws + h->lay.u;
     p.ring = h->ws + h->lay.ring;
-    p.flag = reinterpret_cast<unsigned long long *>(h->ws + h->lay.flag);
+    p.nh = entry_halves(h->w, h->R, h->comp);
     p.ctrl = reinterpret_cast<int *>(h->ws + h->lay.ctrl);
     p.hist = reinterpret_cast<unsigned long long *>(h->ws + h->lay.hist);
     p.gbar = reinterpret_cast<unsigned long long *>(h->ws + h->lay.gbar);
@@ -816,18 +862,29 @@ static atk::Params make_params(const at_solver *h)
         p.cA = h->dt / (12.0 * h->dx);
         p.cB = h->nu * h->dt / (12.0 * h->dx * h->dx);
     }
-    p.dtA = h->dt * h->g.forcing_amp;
+    p.cr = (h->order == 2 ? 2.0 : 1.0) * h->nu / h->dx;
+    const bool dtA = h->v64 || h->comp;
+    p.fX = dtA ? h->dt * h->g.forcing_amp : (h->order == 2 ? 2.0 : 12.0) * h->dx * h->g.forcing_amp;
+    p.cA32 = (float)p.cA;
+    p.cB32 = (float)p.cB;
+    // (the factors of the rounded cA: their products with it are rounded once)
+    p.cr32 = (float)(p.cB / (double)p.cA32);
+    p.fX32 = (float)(dtA ? p.fX : h->dt * h->g.forcing_amp / (double)p.cA32);
+    p.gpl = h->gpl;
+    const atk::Swizzle swz = atk::Swizzle::of(h->gpl * h->w / 4);
+    p.swz_shift = swz.shift;
+    p.swz_mask = swz.mask;
     p.x0 = h->g.origin[0];
     p.dx = h->dx;
     p.G = h->G;
     p.E = h->G * atk::kWarps;
     p.stages = h->stages;
     p.smax = h->smax;
-    p.bar_off = h->sl.bar_off;
-    p.hist_off = h->sl.hist_off;
     p.raw_off = h->sl.raw_off;
     p.stage_off = h->sl.stage_off;
-    p.stage_bytes = h->sl.stage_bytes;
+    p.stage_bytes = (int)h->sl.stage_bytes;
+    const int gw = groups_per_lane(h->M);
+    p.tab_words = (int)atk::tile_points(h->M, gw, full_runs(h->M, gw));
     p.tab_off = h->sl.tab_off;
     p.sb = 1;
     p.alt = 0;
@@ -851,11 +908,10 @@ int at_set_state(at_solver *h, const void *u)
         e = cudaLaunchKernel(h->init_kernel, dim3(blocks), dim3(256), args, 0, h->stream);
         if (e != cudaSuccess) return cuda_fail(e, "launch at_init3d");
         h->step = 0;
-        h->flags_E = 0;
-        h->has_state = true;
+            h->has_state = true;
         return AT_OK;
     }
-    e = cudaMemsetAsync(h->ws + h->lay.ring, 0, (size_t)h->T * h->P * 2 * atk::kRingEntry, h->stream);
+    e = cudaMemsetAsync(h->ws + h->lay.ring, 0, h->lay.ctrl - h->lay.ring, h->stream);
     if (e != cudaSuccess) return cuda_fail(e, "cudaMemsetAsync(ring)");
     if (h->comp) {
         e = cudaMemsetAsync(h->ws + h->lay.ur, 0, (size_t)h->N * h->w, h->stream);
@@ -867,7 +923,6 @@ int at_set_state(at_solver *h, const void *u)
     e = cudaLaunchKernel(h->init_kernel, dim3(blocks), dim3(256), args, 0, h->stream);
     if (e != cudaSuccess) return cuda_fail(e, "launch at_init");
     h->step = 0;
-    h->flags_E = 0;
     h->has_state = true;
     return AT_OK;
 }
@@ -941,9 +996,14 @@ static int step_impl(at_solver *h, int64_t n_steps, int delay_mode, int8_t *dela
     }
     p.levels = levels;
     p.levels_depth = depth;
-    const cudaError_t e = launch_stepper(h, &p, (delay_mode == AT_SYNC && p.sb > 1) ? h->kernel_bs : h->kernel);
-    if (e != cudaSuccess) return cuda_fail(e, "cooperative launch of at_stepper");
-    h->step += n_steps;
+    // (the kernel counts the levels of a launch in 32 bits)
+    for (int64_t done = 0; done < n_steps; done += p.n_steps) {
+        p.n_steps = n_steps - done < (1LL << 29) ? n_steps - done : (1LL << 29);
+        p.delays = delays ? delays + (size_t)done * h->P * 2 : nullptr;
+        const cudaError_t e = launch_stepper(h, &p, (delay_mode == AT_SYNC && p.sb > 1) ? h->kernel_bs : h->kernel);
+        if (e != cudaSuccess) return cuda_fail(e, "cooperative launch of at_stepper");
+        h->step += p.n_steps;
+    }
     return AT_OK;
 }
 
@@ -974,6 +1034,9 @@ int at_set_history(at_solver *h, const void *levels, int64_t depth, int64_t leve
     cudaError_t e = cudaMemcpyAsync(h->ws + h->lay.u, lv + (size_t)(level % depth) * h->N * h->w, (size_t)h->N * h->w,
                                     cudaMemcpyDeviceToDevice, h->stream);
     if (e != cudaSuccess) return cuda_fail(e, "cudaMemcpyAsync(level)");
+    // (entries of the levels after `level` would pass for the coming run's)
+    e = cudaMemsetAsync(h->ws + h->lay.ring, 0, h->lay.ctrl - h->lay.ring, h->stream);
+    if (e != cudaSuccess) return cuda_fail(e, "cudaMemsetAsync(ring)");
     atk::Params p = make_params(h);
     const long long lo = level - need + 1;
     void *kern = h->w == 8 ? atk_restore_kernel_f64(h->order) : atk_restore_kernel_f32(h->order);
@@ -985,7 +1048,6 @@ int at_set_history(at_solver *h, const void *levels, int64_t depth, int64_t leve
     e = cudaLaunchKernel(kern, dim3(blocks), dim3(256), args, 0, h->stream);
     if (e != cudaSuccess) return cuda_fail(e, "launch at_restore");
     h->step = level;
-    h->flags_E = 0;
     h->has_state = true;
     return AT_OK;
 }
@@ -1164,7 +1226,7 @@ size_t at_batch_workspace_bytes(const at_grid *grid, int64_t n_inst, const at_in
     if (check_batch(grid, n_inst, inst, M, scheme_order, &d) != AT_OK) return 0;
     const int w = grid->dtype == AT_F64 ? 8 : 4;
     const int s = scheme_order / 2 + 1;
-    return layout(d.N, d.P, w, d.Lmax, ring_slots(d.Lmax, s), n_inst, (grid->flags & AT_FLAG_COMPENSATED) != 0).total;
+    return layout(d.N, d.P, w, s - 1, d.Lmax, ring_slots(d.Lmax, s), n_inst, (grid->flags & AT_FLAG_COMPENSATED) != 0).total;
 }
 
 int at_create_batch(const at_grid *grid, int64_t n_inst, const at_instance *inst, int64_t M, int scheme_order,
@@ -1181,7 +1243,7 @@ int at_create_batch(const at_grid *grid, int64_t n_inst, const at_instance *inst
     const int T = ring_slots(d.Lmax, s);
     const bool comp = (grid->flags & AT_FLAG_COMPENSATED) != 0;
     if (comp && w != 4) return fail(AT_ERR_ARG, "AT_FLAG_COMPENSATED needs FP32 state");
-    const Layout lay = layout(d.N, d.P, w, d.Lmax, T, n_inst, comp);
+    const Layout lay = layout(d.N, d.P, w, s - 1, d.Lmax, T, n_inst, comp);
     if (!grid->workspace) return fail(AT_ERR_ARG, "workspace is NULL");
     if (grid->workspace_bytes < lay.total)
         return fail(AT_ERR_ARG, "workspace too small: %zu < %zu", grid->workspace_bytes, lay.total);
@@ -1212,13 +1274,11 @@ int at_create_batch(const at_grid *grid, int64_t n_inst, const at_instance *inst
         for (int64_t lp = 0; lp < Pi; ++lp) {
             atk::BatchSub &b = sub[(size_t)(p0 + lp)];
             b = atk::BatchSub{};
-            if (scheme_order == 2) {
-                b.cA = a.dt / (2.0 * dx);
-                b.cB = a.nu * a.dt / (dx * dx);
-            } else {
-                b.cA = a.dt / (12.0 * dx);
-                b.cB = a.nu * a.dt / (12.0 * dx * dx);
-            }
+            const double cB = a.nu * a.dt / ((scheme_order == 2 ? 1.0 : 12.0) * dx * dx);
+            b.cA = a.dt / ((scheme_order == 2 ? 2.0 : 12.0) * dx);
+            b.cr = comp ? cB : (scheme_order == 2 ? 2.0 : 1.0) * a.nu / dx;
+            b.cA32 = (float)b.cA;
+            b.cr32 = (float)(comp ? cB : cB / (double)b.cA32);
             b.seed = a.seed;
             b.L = a.L;
             b.lp = (int)lp;
@@ -1259,7 +1319,7 @@ int at_create_batch(const at_grid *grid, int64_t n_inst, const at_instance *inst
     int stages = grid->stages > 0 ? grid->stages : 3;
     if (stages < atk::kMinStages) stages = atk::kMinStages;
     rc = launch_shape((int64_t)h->K * M, w, d.P, tab_size(M, w, false, true, comp, h->ntiles_k, h->K), grid->max_ctas,
-                      stages, sms, smem_optin, h->kernel, &h->G, &h->stages, &h->sl, &h->smem, &h->smax);
+                      stages, grid->stages > 0, sms, smem_optin, h->kernel, &h->G, &h->stages, &h->sl, &h->smem, &h->smax);
     if (rc != AT_OK) { delete h; return rc; }
     prepare_bs(h);
     h->sb = grid->steps_per_pass > 0 ? grid->steps_per_pass : 1;
@@ -1285,7 +1345,7 @@ int at_tune(at_solver *h, int64_t n_steps, int delay_mode, at_tune_result *res)
     if (cudaStreamIsCapturing(h->stream, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone)
         return fail(AT_ERR_STATE, "at_tune under stream capture");
     std::memset(res, 0, sizeof(*res));
-    const int gmax = (int)((h->P + atk::kWarps - 1) / atk::kWarps);
+    const int gmax = (int)(h->P < (1LL << 30) ? h->P : (1LL << 30));
 
     cudaEvent_t ev[3];
     for (int i = 0; i < 3; ++i) {
@@ -1309,7 +1369,7 @@ int at_tune(at_solver *h, int64_t n_steps, int delay_mode, at_tune_result *res)
         int G = 0, st = 0, smem = 0;
         long long smax = 0;
         atk::SmemLayout sl{};
-        const int r = launch_shape((int64_t)kt * h->M, h->w, h->P, tsz, sh.G, sh.stages, h->sm_count,
+        const int r = launch_shape((int64_t)kt * h->M, h->w, h->P, tsz, sh.G, sh.stages, true, h->sm_count,
                                    h->smem_optin, h->kernel, &G, &st, &sl, &smem, &smax);
         if (r != AT_OK) return r;
         if (st != sh.stages) return AT_ERR_RESIDENCY;   // did not fit as asked
@@ -1668,7 +1728,7 @@ extern "C" int at_step_noalloc(const at_grid *grid, int64_t P, int scheme_order,
     const int w = grid->dtype == AT_F64 ? 8 : 4;
     const int s = scheme_order / 2 + 1;
     const int T = ring_slots(L, s);
-    const Layout lay = layout(0, P, w, L, T, 0, false, false);   // scratch only: the state is the caller's
+    const Layout lay = layout(0, P, w, s - 1, L, T, 0, false, false);   // scratch only: the state is the caller's
     if (lay.total > (size_t)AT_NOALLOC_SCRATCH_BYTES)
         return fail(AT_ERR_ARG,
                     "at_step_noalloc: P=%lld, L=%d, order %d need %zu bytes of scratch, more than the "
@@ -1700,10 +1760,11 @@ extern "C" int at_step_noalloc(const at_grid *grid, int64_t P, int scheme_order,
     h.comp = false;
     h.v64 = viscous_fp64(w, scheme_order, (uint32_t)grid->flags, nu * dt / (dx * dx));
     pick_kernels(w, scheme_order, h.M, grid->forcing_amp != 0.0, h.v64, false, &h.kernel, &h.init_kernel);
+    h.gpl = run_groups(h.M);
     int stages = grid->stages > 0 ? grid->stages : 3;
     if (stages < atk::kMinStages) stages = atk::kMinStages;
-    rc = launch_shape(h.M, w, P, tab_size(h.M, w, grid->forcing_amp != 0.0, false), grid->max_ctas, stages, sms,
-                      smem_optin, h.kernel, &h.G, &h.stages, &h.sl, &h.smem, &h.smax);
+    rc = launch_shape(h.M, w, P, tab_size(h.M, w, grid->forcing_amp != 0.0, false), grid->max_ctas, stages,
+                      grid->stages > 0, sms, smem_optin, h.kernel, &h.G, &h.stages, &h.sl, &h.smem, &h.smax);
     if (rc != AT_OK) return rc;
     h.sb = 1;
 
@@ -1719,11 +1780,13 @@ extern "C" int at_step_noalloc(const at_grid *grid, int64_t P, int scheme_order,
     if (e != cudaSuccess) return cuda_fail(e, "launch at_init");
     if (n_steps > 0) {
         p.mode = delay_mode;
-        p.delays = delays;
-        p.n_steps = n_steps;
         p.sb = 1;
-        e = launch_stepper(&h, &p, h.kernel);
-        if (e != cudaSuccess) return cuda_fail(e, "cooperative launch of at_stepper");
+        for (int64_t done = 0; done < n_steps; done += p.n_steps) {
+            p.n_steps = n_steps - done < (1LL << 29) ? n_steps - done : (1LL << 29);
+            p.delays = delays ? delays + (size_t)done * P * 2 : nullptr;
+            e = launch_stepper(&h, &p, h.kernel);
+            if (e != cudaSuccess) return cuda_fail(e, "cooperative launch of at_stepper");
+        }
     }
     return read_status(&h);
 }

@@ -122,6 +122,27 @@ __device__ __forceinline__ void fence_proxy_async_global()
     asm volatile("fence.proxy.async.global;" ::: "memory");
 }
 
+__device__ __forceinline__ void cp_async_commit()
+{
+    asm volatile("cp.async.commit_group;" ::: "memory");
+}
+
+// Waits until at most n of this thread's committed groups are in flight (at
+// most 7: a larger n waits for more than it has to).
+__device__ __forceinline__ void cp_async_wait(int n)
+{
+    switch (n) {
+    case 0: asm volatile("cp.async.wait_group 0;" ::: "memory"); break;
+    case 1: asm volatile("cp.async.wait_group 1;" ::: "memory"); break;
+    case 2: asm volatile("cp.async.wait_group 2;" ::: "memory"); break;
+    case 3: asm volatile("cp.async.wait_group 3;" ::: "memory"); break;
+    case 4: asm volatile("cp.async.wait_group 4;" ::: "memory"); break;
+    case 5: asm volatile("cp.async.wait_group 5;" ::: "memory"); break;
+    case 6: asm volatile("cp.async.wait_group 6;" ::: "memory"); break;
+    default: asm volatile("cp.async.wait_group 7;" ::: "memory"); break;
+    }
+}
+
 __device__ __forceinline__ void cp_async_wait_all()
 {
     asm volatile("cp.async.wait_all;" ::: "memory");
@@ -153,6 +174,34 @@ __device__ __forceinline__ long long ld_acquire_cta_shared(const volatile long l
     return v;
 }
 
+// ---- words with their level tag ---------------------------------------------
+// 8 bytes of payload and 8 of tag as one 16-byte access (single-copy atomic at
+// gpu scope), so that a reader that sees the tag has the payload: no fence, no
+// flag, one trip to the L2 cache.  Predicated (no branch around one access).
+__device__ __forceinline__ void st_tagged(bool on, void *e, unsigned long long payload, unsigned long long tag)
+{
+    asm volatile("{\n\t.reg .b128 q;\n\t.reg .pred p;\n\tsetp.ne.b32 p, %3, 0;\n\tmov.b128 q, {%1, %2};\n\t"
+                 "@p st.relaxed.gpu.global.b128 [%0], q;\n\t}"
+                 ::"l"(e), "l"(payload), "l"(tag), "r"((int)on) : "memory");
+}
+
+// (off: payload and tag 0, no level's)
+template <int NH>
+__device__ __forceinline__ void ld_tagged(bool on, const unsigned char *e, unsigned long long *payload,
+                                          unsigned long long *tag)
+{
+#pragma unroll
+    for (int h = 0; h < NH; ++h)
+        asm volatile("{\n\t.reg .b128 q;\n\t.reg .pred p;\n\tsetp.ne.b32 p, %3, 0;\n\t"
+                     "mov.b128 q, {%4, %4};\n\t@p ld.relaxed.gpu.global.b128 q, [%2];\n\t"
+                     "mov.b128 {%0, %1}, q;\n\t}"
+                     : "=l"(payload[h]), "=l"(tag[h]) : "l"(e + 16 * h), "r"((int)on), "l"(0ull) : "memory");
+}
+
+// a word from the L2 cache
+__device__ __forceinline__ float ld_cg(const float *p) { return __ldcg(p); }
+__device__ __forceinline__ double ld_cg(const double *p) { return __ldcg(p); }
+
 __device__ __forceinline__ int ld_relaxed(const int *p)
 {
     int v;
@@ -176,6 +225,12 @@ __device__ __forceinline__ void st_cg16(void *p, float a, float b, float c, floa
 __device__ __forceinline__ void st_cg16(void *p, double a, double b)
 {
     asm volatile("st.global.cg.v2.f64 [%0], {%1, %2};" ::"l"(p), "d"(a), "d"(b) : "memory");
+}
+
+__device__ __forceinline__ void st_cg16(void *p, uint4 v)
+{
+    asm volatile("st.global.cg.v4.u32 [%0], {%1, %2, %3, %4};" ::"l"(p), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w)
+                 : "memory");
 }
 
 // ---- SplitMix64 (Steele, Lea & Flood, OOPSLA 2014) --------------------------

@@ -7,33 +7,34 @@
 // over one pass of `len` consecutive levels n .. n+len (len = 1 except in
 // blocked free-running mode).  For each tile the PE
 //   * has already copied the subdomain's M state words into one of its
-//     shared-memory stages with a bulk (TMA-engine) copy, D tiles ahead;
-//   * has already chosen the delays k (prescribed, replayed, or -- free
-//     running -- read off the neighbour's progress flag, blocking only while
-//     the neighbour lags by more than the delay bound allows: the blocking
-//     branch of Algorithm 2) and copied the neighbours' delayed boundary
-//     values (levels n-k-m, Eq. AT1/AT2) from the ring buffers, one tile ahead;
+//     shared-memory stages (16-byte asynchronous copies, D tiles ahead);
+//   * has already read the neighbours' delayed boundary values (levels n-k-m,
+//     Eq. AT1/AT2) from the ring buffers, one tile ahead.  Every ring entry
+//     carries the level it holds, so what is not there yet shows by itself and
+//     is read again when the tile is reached: the blocking branch of
+//     Algorithm 2.  Free running, the delay k is what the entries show: the
+//     newest level the neighbour has published, at most L behind;
 //   * approximates the halo values ("approximate" step of Algorithm 2, split
 //     form of Sec. 5.2), applies the unchanged central stencil of order 2 or
 //     4 and the Euler update `len` times on the tile held in registers
 //     (neighbour values by warp shuffles), and writes the final level back in
 //     place;
-//   * after every level writes the new boundary values into ring slot
-//     (level mod T) and, on its two edge faces, releases the face's progress
-//     flag (the notified put).
+//   * after every level writes the new boundary values, with their level, into
+//     ring slot (level mod T) (the notified put: data and notification are one
+//     16-byte store).
 // Halo values never come from a neighbour's state array, only from the ring,
 // so each PE updates its own subdomains in place, and a PE never waits for
-// another PE of its CTA except through the same flags.
+// another PE of its CTA except through the same entries.
 //
 // Blocked free-running mode (temporal blocking): a pass of len <= L+1 levels
 // uses, at inner step i, the halo extrapolated with delay k0 + i from the
 // levels available when the pass started (Eq. AT1/AT2 with a larger k), so
 // the state is read and written once per pass instead of once per level.
 //
-// AT_SYNC replaces the flag waits with a grid barrier between steps
-// (Algorithm 1).  Every wait is bounded by timeout_ns; on expiry the kernel
-// latches AT_ERR_TIMEOUT in the control block, raises the abort word and
-// every PE leaves its loop (after its copies in flight have landed).
+// AT_SYNC puts a grid barrier between steps (Algorithm 1).  Every wait is
+// bounded by timeout_ns; on expiry the kernel latches AT_ERR_TIMEOUT in the
+// control block, raises the abort word and every PE leaves its loop (after
+// its copies in flight have landed).
 #pragma once
 
 #include "at_device.cuh"
@@ -42,19 +43,17 @@
 #ifndef AT_MIN_CTAS_PER_SM
 #define AT_MIN_CTAS_PER_SM 3
 #endif
-#ifndef AT_VGROUP
-#define AT_VGROUP 2
-#endif
 
 namespace atk {
 
 constexpr int kWarps = 4;                         // PEs (warps) per CTA
 constexpr int kThreads = 32 * kWarps;
-constexpr int kRingEntry = 16;                    // bytes per (slot, subdomain, face)
+constexpr int kRingHalf = 16;                     // bytes of a half of a ring entry: 8 of payload, 8 of level tag
 constexpr int kMaxS = 3;                          // levels per halo approximation
 constexpr int kStripBytes = 64;                  // blocked synchronous mode: edge strip per (subdomain, face)
-constexpr int kRawFace = 64;                      // raw bytes per face: kMaxS ring entries or one edge strip
-constexpr int kRawBytes = 2 * kRawFace;           // one tile's delayed levels [face][m] (or edge strips)
+constexpr int kRawEntry = 16;                     // payload of one ring entry in shared memory
+constexpr int kRawFace = 64;                      // per face: kMaxS of them
+constexpr int kRawBytes = 2 * kRawFace;           // one tile's delayed levels [face][m]
 constexpr int kMaxM = 1024;                       // points per subdomain (one warp's tile)
 constexpr int kMaxL = 16;
 constexpr int kMinStages = 2;                     // stages per PE (tile in use + one ahead)
@@ -62,51 +61,88 @@ constexpr int kMinStages = 2;                     // stages per PE (tile in use 
 enum : int { kModeSync = 0, kModeSeeded = 1, kModeFree = 2, kModeReplay = 3 };
 
 // Shared-memory layout of one CTA, shared by the host (launch set-up) and the
-// kernel: per PE `stages` mbarriers, delay counters, two raw-level buffers and
-// `stages` tile buffers; then a table of `tab_bytes`: the forcing tables
-// (sin/cos of the offsets in a subdomain, and of each PE's subdomain origins)
-// or, for an ensemble, each PE's subdomain records.
+// kernel: per PE a raw-level buffer and `stages` tile buffers;
+// then a table of `tab_bytes`: the forcing tables (sin/cos of the offsets in a
+// subdomain, and of each PE's subdomain origins) or, for an ensemble, each
+// PE's subdomain records.  M: points of a tile buffer (tile_points()).
 struct SmemLayout {
-    long long bar_off, hist_off, raw_off, stage_off, stage_bytes, tab_off, total;
+    long long raw_off, stage_off, stage_bytes, tab_off, total;
 };
 
 __host__ __device__ inline long long round_up(long long x, long long a) { return (x + a - 1) / a * a; }
 
-// Groups of 4 points a lane of the stepper holds consecutively (see run_pe).
-template <int GW, bool FULL, bool BATCH, int PREC>
-__host__ __device__ constexpr int group_run() { return (!BATCH && FULL && PREC != 2 && GW % AT_VGROUP == 0) ? AT_VGROUP : 1; }
-
-// Place of group g of a subdomain in the forcing tables: with runs of VG
-// groups per lane the tables are stored run-slot-major, so that the lanes of
-// a warp, reading slot i of their runs, read consecutive 16-byte words.
-template <int VG>
-__host__ __device__ inline int table_group(int g, int NG) { return VG == 1 ? g : (g % VG) * (NG / VG) + g / VG; }
+// Points of a tile buffer and of a forcing table for tiles of M points in
+// lanes of gw whole groups (all 32 of them: lanes beyond the tile then need no
+// guard) or, runs not full, of M points.
+__host__ __device__ inline long long tile_points(long long M, int gw, bool full)
+{
+    return full ? 128LL * gw : round_up(M, 32);
+}
 
 __host__ __device__ inline SmemLayout smem_layout(long long M, int word, int stages, long long tab_bytes, bool comp = false)
 {
     SmemLayout l;
-    l.bar_off = 0;
-    l.hist_off = round_up(8LL * kWarps * stages, 16);
-    l.raw_off = round_up(l.hist_off + 4LL * kWarps * 2 * (kMaxL + 1), 128);
-    l.stage_off = round_up(l.raw_off + 2LL * kWarps * kRawBytes, 128);
+    l.raw_off = 0;
+    l.stage_off = round_up(l.raw_off + (long long)kWarps * kRawBytes, 128);
     l.stage_bytes = round_up(M * word, 128) * (comp ? 2 : 1);     // tile (+ its error words)
     l.tab_off = l.stage_off + (long long)kWarps * stages * l.stage_bytes;
     l.total = l.tab_off + tab_bytes;
     return l;
 }
 
+// Place of 16-byte chunk c of a tile in its stage (and of the forcing tables):
+// a lane reads cpl consecutive chunks, so with cpl = 2, 4, 8 the 8 lanes that
+// share a shared-memory cycle would meet in the same banks cpl at a time;
+// exchanging chunks within blocks of 8 by the block's number spreads them, and
+// leaves the coalesced side (consecutive lanes, consecutive chunks) conflict-free.
+// An odd cpl has no conflicts, other even ones two-way ones.
+struct Swizzle {
+    int shift, mask;
+    __host__ __device__ static constexpr Swizzle of(int cpl)
+    {
+        return cpl == 16 ? Swizzle{4, 7} : (cpl == 2 || cpl == 4 || cpl == 8) ? Swizzle{3, cpl - 1} : Swizzle{0, 0};
+    }
+    __host__ __device__ constexpr int operator()(int c) const { return c ^ ((c >> shift) & mask); }
+    // byte offsets in the stage of chunk lane + 32 t (the coalesced side)
+    __device__ __forceinline__ int coalesced(int lane, int t) const
+    {
+        return 512 * t + (((lane ^ ((lane >> shift) & mask)) << 4) ^ ((((32 * t) >> shift) & mask) << 4));
+    }
+};
+
+// byte offset in the stage of chunk k of a lane that holds CPL whole chunks
+template <int CPL>
+__device__ __forceinline__ int lane_chunk(int lane, int k)
+{
+    const int lx = CPL == 16 ? lane & 7 : ((lane * CPL) >> 3) & (CPL - 1);
+    return ((16 * CPL * lane) | (lx << 4)) ^ (k << 4);
+}
+
+// A ring entry holds one face's R boundary words of one level (a compensated
+// state: R hi, then R lo words) in one or two halves of 16 bytes: 8 bytes of
+// payload and the level's tag.  A half is written and read as one 16-byte
+// access, so the words and their tag arrive together.
+template <typename T, int ORDER, int PREC>
+__host__ __device__ constexpr int entry_halves()
+{
+    return (int)sizeof(T) * (ORDER / 2) * (PREC == 2 ? 2 : 1) > 8 ? 2 : 1;
+}
+
+// Tag of a level (0, the cleared ring, is no level's).
+__host__ __device__ inline unsigned long long entry_tag(long long level) { return (unsigned long long)(level + 1); }
+
 // Ensembles: independent 1D problems of M-point subdomains laid end to end.
 // One record per subdomain (built on the host, copied to shared memory by the
 // PE that owns it) and one per problem instance.
 struct BatchSub {
-    double cA, cB;             // stencil factors of the instance (as Params::cA, cB)
+    double cA, cr;             // stencil factors of the instance (as Params::cA, cr; compensated state: cA, cB)
     unsigned long long seed;   // AT_SEEDED seed of the instance
     int L;                     // delay bound of the instance
     int lp;                    // index of the subdomain within its instance
     int Pi;                    // subdomains of the instance
     int inst;                  // instance
     long long left, right;     // global subdomain across face 0 / 1; -1 = exact boundary
-    long long pad_;
+    float cA32, cr32;          // cA, cr in FP32
 };
 static_assert(sizeof(BatchSub) == 64, "BatchSub is four 16-byte vectors");
 
@@ -127,14 +163,13 @@ static_assert(sizeof(BatchInst) == 64, "BatchInst is 64 bytes");
 // neighbour of the last subdomain is s0 of the next tile.  Stored as an int4
 // (s0, rec, cnt | link << 16, 0).
 struct TileInfo {
-    long long s0, rec;
-    int cnt, link;
+    int s0, rec, cnt, link;
 };
 
 struct Params {
     void *u;                   // state, N words, updated in place
-    unsigned char *ring;       // [T][P][2] entries of 16 bytes
-    unsigned long long *flag;  // [P][2] last level published per face
+    unsigned char *ring;       // [T][P][2] entries (see entry_halves)
+    int nh;                    // halves of an entry
     int *ctrl;                 // control block (status, abort, diagnostics)
     unsigned long long *hist;  // [L+1] delay counts
     unsigned long long *gbar;  // grid-barrier arrival counter (AT_SYNC)
@@ -157,13 +192,19 @@ struct Params {
                                // synchronous mode, where k = 0 and the ghost cells are recomputed)
     int alt;                   // sweep direction alternates from pass to pass (blocked free mode)
     unsigned long long seed;
-    double cA, cB, dtA;        // dt/(2dx) | dt/(12dx);  nu dt/dx^2 | nu dt/(12dx^2);  dt A
+    double cA, cB, cr;         // dt/(2dx) | dt/(12dx);  nu dt/dx^2 | nu dt/(12dx^2);  cB / cA
+    double fX;                 // forcing factor: A dt (FP64 viscous term, compensated state), else A dt / cA
+    float cA32, cB32, cr32, fX32;   // the same in FP32 (no conversion per tile)
     double x0, dx;
     int G;                     // CTAs
     int E;                     // PEs = G * kWarps
     int stages;                // tile buffers per PE
+    int gpl;                   // groups of 4 points per lane
+    int swz_shift, swz_mask;   // place of a tile's chunks in its stage (see Swizzle)
     long long smax;            // most subdomains of any PE
-    long long bar_off, hist_off, raw_off, stage_off, stage_bytes, tab_off;
+    int stage_bytes;           // bytes of a stage (compensated state: its second half holds the lo words)
+    int tab_words;             // words of a forcing table (M, padded)
+    long long raw_off, stage_off, tab_off;
     long long timeout_ns;
     int skip_publish;          // test knob: PE 0 stops releasing flags
     long long skip_step;
@@ -181,27 +222,6 @@ static __device__ __noinline__ void raise_timeout(const Params &p, int where, lo
         p.ctrl[kCtrlStep] = (int)n;
     }
     atomicExch(p.ctrl + kCtrlAbort, 1);
-}
-
-// Waits until *fl >= need (acquire).  Returns the value seen in *seen.
-static __device__ __noinline__ bool wait_flag(const Params &p, const unsigned long long *fl, long long need,
-                                       unsigned long long *seen, long long n, long long nb)
-{
-    unsigned long long v = ld_acquire(fl);
-    if ((long long)v >= need) { *seen = v; return true; }
-    const unsigned long long t0 = global_ns();
-    unsigned ns = 32;
-    for (;;) {
-        __nanosleep(ns);
-        if (ns < 256) ns <<= 1;
-        v = ld_acquire(fl);
-        if ((long long)v >= need) { *seen = v; return true; }
-        if (ld_relaxed(p.ctrl + kCtrlAbort)) return false;
-        if ((long long)(global_ns() - t0) > p.timeout_ns) {
-            raise_timeout(p, kWhereFlag, n, nb);
-            return false;
-        }
-    }
 }
 
 static __device__ __noinline__ bool wait_grid(const Params &p, unsigned long long target, long long n)
@@ -255,6 +275,14 @@ __device__ __forceinline__ void sts4(T *s, const T *v)
     }
 }
 
+// one 16-byte chunk (4 floats or 2 doubles)
+template <typename T, int CNT>
+__device__ __forceinline__ void stsv(T *s, const T *v)
+{
+    if constexpr (sizeof(T) == 4) *reinterpret_cast<float4 *>(s) = make_float4(v[0], v[1], v[2], v[3]);
+    else *reinterpret_cast<double2 *>(s) = make_double2(v[0], v[1]);
+}
+
 // 4 consecutive words to global memory (16-byte aligned), bypassing L1.
 template <typename T>
 __device__ __forceinline__ void stg4(T *g, const T *v)
@@ -267,14 +295,26 @@ __device__ __forceinline__ void stg4(T *g, const T *v)
     }
 }
 
-// One 16-byte ring entry holding R words (the rest zero).
-template <typename T, int R>
-__device__ __forceinline__ void st_entry(unsigned char *e, const T *v)
+// One ring entry: R words v (compensated state: and their lo words l) with the
+// level's tag in every half (`on`: predicate).
+template <typename T, int ORDER, int PREC>
+__device__ __forceinline__ void st_entry(bool on, unsigned char *e, const T *v, const T *l, unsigned long long tag)
 {
-    if constexpr (sizeof(T) == 4) {
-        st_cg16(e, v[0], R > 1 ? v[1] : 0.0f, 0.0f, 0.0f);
+    constexpr int R = ORDER / 2;
+    auto two = [](T a, T b) -> unsigned long long {
+        return ((unsigned long long)__float_as_uint((float)b) << 32) | __float_as_uint((float)a);
+    };
+    if constexpr (sizeof(T) == 8) {
+#pragma unroll
+        for (int q = 0; q < R; ++q)
+            st_tagged(on, e + q * kRingHalf, (unsigned long long)__double_as_longlong((double)v[q]), tag);
+    } else if constexpr (PREC == 2 && R == 2) {
+        st_tagged(on, e, two(v[0], v[1]), tag);
+        st_tagged(on, e + kRingHalf, two(l[0], l[1]), tag);
+    } else if constexpr (PREC == 2) {
+        st_tagged(on, e, two(v[0], l[0]), tag);
     } else {
-        st_cg16(e, v[0], R > 1 ? v[1] : 0.0);
+        st_tagged(on, e, two(v[0], R > 1 ? v[R - 1] : (T)0), tag);
     }
 }
 
@@ -292,12 +332,12 @@ __device__ __forceinline__ T approx_halo(const unsigned char *raw, int k, int r)
 {
     const T r0 = reinterpret_cast<const T *>(raw)[r];
     if (k == 0) return r0;
-    const T r1 = reinterpret_cast<const T *>(raw + kRingEntry)[r];
+    const T r1 = reinterpret_cast<const T *>(raw + kRawEntry)[r];
     const T d1 = r0 - r1;
     if constexpr (S_LEV == 2) {
         return r0 + (T)k * d1;
     } else {
-        const T r2 = reinterpret_cast<const T *>(raw + 2 * kRingEntry)[r];
+        const T r2 = reinterpret_cast<const T *>(raw + 2 * kRawEntry)[r];
         const T d2 = d1 - (r1 - r2);
         return r0 + ((T)k * d1 + (T)(k * (k + 1) / 2) * d2);
     }
@@ -316,106 +356,242 @@ __device__ __forceinline__ T approx_halo_lo(const unsigned char *raw, int k, int
     const T *e0 = reinterpret_cast<const T *>(raw);
     const T h0 = e0[r], l0 = e0[R + r];
     if (k == 0) return l0;
-    const T *e1 = reinterpret_cast<const T *>(raw + kRingEntry);
+    const T *e1 = reinterpret_cast<const T *>(raw + kRawEntry);
     const T h1 = e1[r], l1 = e1[R + r];
     const T d1 = (h0 - h1) + (l0 - l1);
     if constexpr (S_LEV == 2) {
         return l0 + (T)k * d1;
     } else {
-        const T *e2 = reinterpret_cast<const T *>(raw + 2 * kRingEntry);
+        const T *e2 = reinterpret_cast<const T *>(raw + 2 * kRawEntry);
         const T h2 = e2[r], l2 = e2[R + r];
         const T d2 = ((h0 - h1) - (h1 - h2)) + ((l0 - l1) - (l1 - l2));
         return l0 + (T)k * d1 + (T)(k * (k + 1) / 2) * d2;
     }
 }
 
-// One 16-byte ring entry of a compensated FP32 state: R hi words, R lo words.
-template <int R>
-__device__ __forceinline__ void st_entry2(unsigned char *e, const float *h, const float *l)
+// A dt sin x (scaled) of one point from the factors of its subdomain and of its
+// offset: fs = f sin x_j, fc = f cos x_j, sv/cv = sin/cos of the offset.
+template <typename T>
+__device__ __forceinline__ T forcing_point(T fs, T fc, T sv, T cv)
 {
-    if constexpr (R == 2) st_cg16(e, h[0], h[1], l[0], l[1]);
-    else st_cg16(e, h[0], l[0], 0.0f, 0.0f);
+    return fma(fc, sv, fs * cv);
 }
 
-// One point of the forward-Euler update: w[0 .. 2R] are the values at offsets
-// -R .. R (w[R] the point itself; wl the lo words of a compensated state),
-// cA = dt/(2dx) | dt/(12dx), cB = nu dt/dx^2 | nu dt/(12dx^2) (cB64 the
-// same in FP64), fs/fc and sv/cv the forcing factors of the subdomain and of
-// the point's offset (A dt sin x = fs cv + fc sv); returns the new value
-// (compensated state: updates the carried error too).  The stepper's tiles
-// and the ghost cells of the blocked synchronous mode both call it, so a
-// point computed twice is computed the same way twice.
-template <typename T, int ORDER, bool FORCED, int PREC>
-__device__ __forceinline__ T stencil_point(const T *w, const T *wl, T cA, T cB, double cB64, T fs, T fc, T sv, T cv,
-                                           T &err)
-{
-    constexpr int R = ORDER / 2;
-    const T cc = w[R];
-    T a, b;
-    if constexpr (PREC == 2) {
-        // differences word by word; the second difference as differences
-        // from the centre point
-        const T cl = wl[R];
-        if constexpr (ORDER == 2) {
-            a = (w[2] - w[0]) + (wl[2] - wl[0]);
-            b = ((w[2] - cc) + (w[0] - cc)) + ((wl[2] - cl) + (wl[0] - cl));
-        } else {
-            a = ((T)8 * (w[3] - w[1]) - (w[4] - w[0])) + ((T)8 * (wl[3] - wl[1]) - (wl[4] - wl[0]));
-            b = ((T)16 * ((w[3] - cc) + (w[1] - cc)) - ((w[4] - cc) + (w[0] - cc))) +
-                ((T)16 * ((wl[3] - cl) + (wl[1] - cl)) - ((wl[4] - cl) + (wl[0] - cl)));
-        }
-        T du = cB * b - cA * (cc + cl) * a;
-        if constexpr (FORCED) du = fs * cv + (fc * sv + du);
-        // two-sum of hi and (du + lo): exact sum t + err
-        const T y = du + err;
-        const T t = cc + y;
-        const T yy = t - cc;
-        err = (cc - (t - yy)) + (y - yy);
-        return t;
-    } else {
-        (void)wl;
-        (void)err;
+// The forward-Euler update u += dt (-u u_x + nu u_xx) + F of a run of points,
+// as u += cA (cr b - u a + F / cA): cA = dt/(2dx) | dt/(12dx), cA cr = nu
+// dt/dx^2 | nu dt/(12dx^2), a and b the stencil's first and second difference.
+// The factors 1, cr, cA each ride in a fused multiply-add, so the increment,
+// formed apart from u, takes 3 operations beside a and b (6 when cB b - cA u a
+// + F + u is taken term by term): 10 a point at order 4, forcing included, 6 at
+// order 2.
+//   FP32: a and b value by value, a = 8 (u_1 - u_-1) - (u_2 - u_-2), b = 16 (u_1
+// + u_-1) - (u_2 + u_-2) - 30 u.
+//   FP64: from the first differences d_i = u_{i+1} - u_i and second ones e_i =
+// d_i - d_{i-1}, formed once for the points that share them: a = 6 (d_i +
+// d_{i-1}) - (e_{i+1} - e_{i-1}), b = 14 e_i - (e_{i+1} + e_{i-1}); the same 10
+// operations, but differences of nearby values are exact.  (FP32 keeps the
+// values' form: there the last addition's rounding decides, and over runs of
+// hundreds of steps the sums' own rounding breaks up its bias: error against 64
+// bits 2.2e-6 against 2.9e-6 with the exact differences.)
+//   Compensated state: the differences word by word, hi and lo, and the factors
+// as cB b - cA u a, each rounded once.
+//
+// Every operation of the first two is written as the one instruction it is, so
+// that a point computed twice -- by its owner in group(), by a neighbour as a
+// ghost cell in point() -- is computed the same way twice.
+//
+// PLAIN: the order-2 update as cB b - cA u a, 7 operations.  The unforced FP32
+// single domain keeps it: its trajectories feed the FP32 gradient, which
+// divides their rounding by |u(T) - target|, and stay bit for bit what they
+// were before the factored form.
+template <typename T, int ORDER, int PREC, bool PLAIN>
+struct StencilK {
+    static constexpr int R = ORDER / 2;
+    static constexpr bool WINDOW = PREC == 1 || (PREC == 0 && sizeof(T) == 4);   // from the values of a window
+    T cA, cr, cB;
+    double cB64;
+    // (cr_: cr; a compensated state: cB)
+    __device__ __forceinline__ StencilK(T cA_, T cr_, const Params &p)
+        : cA(cA_), cr(cr_), cB(PREC == 2 ? cr_ : (T)p.cB32), cB64(p.cB)
+    {
+    }
+
+    // what a lane carries from point to point
+    struct Carry {
+        T w[2];                        // WINDOW: the R words left of the point
+        T d0, d1, e0, e1;              // else d_{i-1}, d_i (order 2: d0 = d_{i-1}); e_{i-1}, e_i
+        T l0, l1, g0;                  // compensated state: the differences of the lo words; d_{i-1} + its lo
+    };
+
+    // cr b - u a + F / cA
+    __device__ __forceinline__ T increment(T cc, T a, T b, T F, bool forced) const
+    {
+        return fma(-cc, a, forced ? fma(cr, b, F) : cr * b);
+    }
+
+    // PREC 1: the viscous term in FP64
+    __device__ __forceinline__ T point_v64(const T *w, T F, bool forced) const
+    {
+        const T cc = w[R];
+        T a;
+        double b64;
         if constexpr (ORDER == 2) {
             a = w[2] - w[0];
-            b = (w[2] + w[0]) - (T)2 * cc;
+            b64 = ((double)w[2] + (double)w[0]) - 2.0 * (double)cc;
         } else {
-            a = (T)8 * (w[3] - w[1]) - (w[4] - w[0]);
-            b = (T)16 * (w[3] + w[1]) - (w[4] + w[0]) - (T)30 * cc;
+            a = (T)8 * (w[2 * R - 1] - w[1]) - (w[2 * R] - w[0]);
+            b64 = 16.0 * ((double)w[2 * R - 1] + (double)w[1]) - ((double)w[2 * R] + (double)w[0]) - 30.0 * (double)cc;
         }
+        T rest = -cA * cc * a;
+        if (forced) rest = rest + F;
+        return (T)((double)cc + (cB64 * b64 + (double)rest));
+    }
+
+    // one point from its stencil values w[0 .. 2R] (offsets -R .. R)
+    template <bool FORCED>
+    __device__ __forceinline__ T point(const T *w, T F) const
+    {
+        const T cc = w[R];
         if constexpr (PREC == 1) {
-            double b64;
-            if constexpr (ORDER == 2) {
-                b64 = ((double)w[2] + (double)w[0]) - 2.0 * (double)cc;
-            } else {
-                b64 = 16.0 * ((double)w[3] + (double)w[1]) - ((double)w[4] + (double)w[0]) - 30.0 * (double)cc;
-            }
-            T rest = -cA * cc * a;
-            if constexpr (FORCED) rest = fs * cv + (fc * sv + rest);
-            (void)b;
-            return (T)((double)cc + (cB64 * b64 + (double)rest));
-        } else {
-            (void)cB64;
-            T du = cB * b - cA * cc * a;
-            if constexpr (FORCED) du = fs * cv + (fc * sv + du);   // two fused multiply-adds
+            return point_v64(w, F, FORCED);
+        } else if constexpr (PLAIN) {
+            const T a = w[2] - w[0], b = (w[2] + w[0]) - (T)2 * cc;
+            const T du = cB * b - cA * cc * a;
             return cc + du;
+        } else if constexpr (WINDOW && ORDER == 2) {
+            const T a = w[2] - w[0], b = fma((T)-2, cc, w[2] + w[0]);
+            return fma(cA, increment(cc, a, b, F, FORCED), cc);
+        } else if constexpr (WINDOW) {
+            const T a = fma((T)8, w[2 * R - 1] - w[1], -(w[2 * R] - w[0]));
+            const T b = fma((T)-30, cc, fma((T)16, w[2 * R - 1] + w[1], -(w[2 * R] + w[0])));
+            return fma(cA, increment(cc, a, b, F, FORCED), cc);
+        } else if constexpr (ORDER == 2) {
+            const T d0 = cc - w[0], d1 = w[2] - cc;
+            return fma(cA, increment(cc, d1 + d0, d1 - d0, F, FORCED), cc);
+        } else {
+            const T d0 = w[1] - w[0], d1 = cc - w[1], d2 = w[2 * R - 1] - cc, d3 = w[2 * R] - w[2 * R - 1];
+            T a, b;
+            from_differences(d2 - d1, d1 - d0, d3 - d2, d2 + d1, a, b);
+            return fma(cA, increment(cc, a, b, F, FORCED), cc);
         }
     }
-}
 
-// Waits (lane 0) for the bulk copy into a stage; bounded.
-static __device__ __noinline__ bool wait_stage(const Params &p, uint64_t *bar, unsigned parity)
-{
-    if (mbar_try_wait(bar, parity)) return true;
-    const unsigned long long t0 = global_ns();
-    for (;;) {
-        if (mbar_try_wait(bar, parity)) return true;
-        if ((long long)(global_ns() - t0) > p.timeout_ns) {
-            raise_timeout(p, kWhereTile, -1, -1);
-            return false;
+    // order 4: a and b from e_i, e_{i-1}, e_{i+1} and s = d_i + d_{i-1}
+    static __device__ __forceinline__ void from_differences(T e, T ep, T en, T s, T &a, T &b)
+    {
+        a = fma((T)6, s, -(en - ep));
+        b = fma((T)14, e, -(en + ep));
+    }
+
+    // the carry before the first point of a lane's run: lw the R words left of
+    // it, c the run (lwl, cl: lo words)
+    __device__ __forceinline__ void start(Carry &y, const T *lw, const T *lwl, const T *c, const T *cl) const
+    {
+        if constexpr (WINDOW) {
+#pragma unroll
+            for (int q = 0; q < R; ++q) y.w[q] = lw[q];
+        } else if constexpr (ORDER == 2) {
+            y.d0 = c[0] - lw[0];
+            if constexpr (PREC == 2) {
+                y.l0 = cl[0] - lwl[0];
+                y.g0 = y.d0 + y.l0;
+            }
+        } else {
+            const T dm = lw[R - 1] - lw[0];
+            y.d0 = c[0] - lw[R - 1];
+            y.d1 = c[1] - c[0];
+            if constexpr (PREC == 2) {
+                const T lm = lwl[R - 1] - lwl[0];
+                y.l0 = cl[0] - lwl[R - 1];
+                y.l1 = cl[1] - cl[0];
+                y.e0 = (y.d0 - dm) + (y.l0 - lm);
+                y.e1 = (y.d1 - y.d0) + (y.l1 - y.l0);
+                y.g0 = y.d0 + y.l0;
+            } else {
+                y.e0 = y.d0 - dm;
+                y.e1 = y.d1 - y.d0;
+            }
         }
     }
-}
 
+    // the 4 points c of a group, in place; nx the R words right of it
+    // (compensated state: cl, nxl the lo words), F their forcing
+    template <bool FORCED>
+    __device__ __forceinline__ void group(Carry &y, T *c, T *cl, const T *nx, const T *nxl, const T *F) const
+    {
+        if constexpr (WINDOW) {
+            T v[4 + 2 * R];
+#pragma unroll
+            for (int q = 0; q < R; ++q) {
+                v[q] = y.w[q];
+                v[R + 4 + q] = nx[q];
+                y.w[q] = c[4 - R + q];
+            }
+#pragma unroll
+            for (int e = 0; e < 4; ++e) v[R + e] = c[e];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) c[e] = point<FORCED>(v + e, FORCED ? F[FORCED ? e : 0] : (T)0);
+        } else {
+            T v[4 + R], vl[PREC == 2 ? 4 + R : 1];
+#pragma unroll
+            for (int e = 0; e < 4 + R; ++e) {
+                v[e] = e < 4 ? c[e < 4 ? e : 0] : nx[e >= 4 ? e - 4 : 0];
+                if constexpr (PREC == 2) vl[e] = e < 4 ? cl[e < 4 ? e : 0] : nxl[e >= 4 ? e - 4 : 0];
+            }
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const T f = FORCED ? F[FORCED ? e : 0] : (T)0;
+                const T cc = v[e];
+                T a, b;
+                if constexpr (ORDER == 2) {
+                    const T dn = v[e + 1] - cc;
+                    if constexpr (PREC == 2) {
+                        const T ln = vl[e + 1] - vl[e];
+                        const T gn = dn + ln;
+                        b = (dn - y.d0) + (ln - y.l0);
+                        a = gn + y.g0;
+                        y.l0 = ln;
+                        y.g0 = gn;
+                    } else {
+                        a = dn + y.d0;
+                        b = dn - y.d0;
+                    }
+                    y.d0 = dn;
+                } else {
+                    const T dn = v[e + 2] - v[e + 1];
+                    T en, s;
+                    if constexpr (PREC == 2) {
+                        const T ln = vl[e + 2] - vl[e + 1];
+                        const T gn = y.d1 + y.l1;
+                        en = (dn - y.d1) + (ln - y.l1);
+                        s = gn + y.g0;
+                        y.l1 = ln;
+                        y.g0 = gn;
+                    } else {
+                        en = dn - y.d1;
+                        s = y.d1 + y.d0;
+                    }
+                    from_differences(y.e1, y.e0, en, s, a, b);
+                    y.d0 = y.d1;
+                    y.d1 = dn;
+                    y.e0 = y.e1;
+                    y.e1 = en;
+                }
+                if constexpr (PREC == 2) {
+                    // two-sum of hi and (increment + lo): exact sum t + err
+                    T yy = fma(-(cA * cc), a, fma(cB, b, vl[e]));
+                    if constexpr (FORCED) yy = yy + f;
+                    const T t = cc + yy;
+                    const T z = t - cc;
+                    cl[e] = (cc - (t - z)) + (yy - z);
+                    c[e] = t;
+                } else {
+                    c[e] = fma(cA, increment(cc, a, b, f, FORCED), cc);
+                }
+            }
+        }
+    }
+};
 
 // Synchronous algorithm: grid barrier before step `step` (1-based within the
 // launch), combined per CTA.  Each warp counts itself on the CTA's shared
@@ -461,60 +637,49 @@ static __device__ __noinline__ bool cta_grid_sync(const Params &p, int *s_count,
 // needs a tile its neighbour finished about a pass earlier; and the tile at
 // the turn is the same subdomain twice in a row, continued in registers.
 //
-// startup: passes of one level while the level is below s-1 (the AT halos
-// need s levels); the synchronous modes read level n only and have none.
+// single: passes of one level while the level is below s-1 (the AT halos need
+// s levels); the synchronous modes read level n only and have none.
 struct Sweep {
-    long long n0, n_steps;
+    long long n0;              // level the launch starts from
+    int n_steps;               // levels of the launch (the host keeps it below 2^30)
     int sb;
+    int single;                // the first `single` levels take one-level passes (start-up)
     bool alt;
-    bool startup;
 };
 
-// Position of a tile in a PE's sweep: pass start level n, subdomain j, the
-// pass length, (alternating sweeps) the direction of the pass, and the
-// index of the pass within the launch.
+// Position of a tile in a PE's sweep: the pass's first level n relative to n0,
+// tile j (relative to the PE's first), the pass length, (alternating sweeps)
+// the direction of the pass, and the index of the pass within the launch.
 struct Cursor {
-    long long n, j;
-    int len;
+    int n, j, len, pass;
     bool rev;
-    long long pass;
 };
 
-__device__ __forceinline__ int pass_len(const Sweep &sw, long long n, int s_lev)
+__device__ __forceinline__ int pass_len(const Sweep &sw, int n)
 {
-    const long long left = sw.n0 + sw.n_steps - n;
-    int len = (int)(left < sw.sb ? left : sw.sb);
-    if (sw.startup && n < s_lev - 1) len = 1;
-    return len;
+    const int left = sw.n_steps - n;
+    return n < sw.single ? 1 : left < sw.sb ? left : sw.sb;
 }
 
-__device__ __forceinline__ long long count_passes(const Sweep &sw, int s_lev)
+__device__ __forceinline__ int count_passes(const Sweep &sw)
 {
-    if (!sw.startup) return (sw.n_steps + sw.sb - 1) / sw.sb;
-    long long single = (s_lev - 1) - sw.n0;
-    if (single < 0) single = 0;
-    if (single > sw.n_steps) single = sw.n_steps;
-    const long long rest = sw.n_steps - single;
-    return single + (rest + sw.sb - 1) / sw.sb;
+    const int single = sw.single < sw.n_steps ? sw.single : sw.n_steps;
+    return single + (sw.n_steps - single + sw.sb - 1) / sw.sb;
 }
 
-__device__ __forceinline__ void advance(const Sweep &sw, Cursor &c, long long lo, long long hi, int s_lev)
+// the next tile of a sweep over tiles 0 .. S-1
+__device__ __forceinline__ void advance(const Sweep &sw, Cursor &c, int S)
 {
-    if (!sw.alt) {
-        if (++c.j == hi) {
-            c.j = lo;
-            c.n += c.len;
-            c.len = pass_len(sw, c.n, s_lev);
-            ++c.pass;
-        }
-    } else if (c.rev ? c.j == lo : c.j == hi - 1) {
-        // turn: the next pass starts on the same subdomain
-        c.rev = !c.rev;
-        c.n += c.len;
-        c.len = pass_len(sw, c.n, s_lev);
-        ++c.pass;
-    } else {
+    const int end = c.rev ? 0 : S - 1;
+    if (c.j != end) {
         c.j += c.rev ? -1 : 1;
+    } else {
+        // the next pass: from the first tile, or (alternating) back from the same one
+        if (sw.alt) c.rev = !c.rev;
+        else c.j = 0;
+        c.n += c.len;
+        c.len = pass_len(sw, c.n);
+        ++c.pass;
     }
 }
 
@@ -552,20 +717,42 @@ __device__ __forceinline__ T exact_ghost2(const BatchInst *binst, const BatchSub
 // ---------------------------------------------------------------------------
 // one processing element (warp)
 // ---------------------------------------------------------------------------
-// Lane l keeps the 4-point groups g = l + 32 m (m < GW) of the tile in
-// registers for the whole pass, so that loads and stores stay coalesced.  The
-// left neighbours of group g are the last R words of group g-1 (lane l-1,
-// same m; for lane 0, lane 31 at m-1), the right neighbours the first R words
-// of group g+1 (lane l+1, same m; for lane 31, lane 0 at m+1): one shuffle
-// per word, no barrier.  Groups 0 and NG-1 take the approximated halo instead.
+// Lane l keeps the gpl consecutive groups of 4 points gpl l .. gpl l + gpl - 1
+// of the tile in registers for the whole pass, so that a level exchanges only
+// R words with each neighbouring lane (one shuffle per word) and every other
+// stencil value is the lane's own.  Lane 0 takes the left halo, the owner of
+// the last group the right one.  A lane sweeps its points in order and in
+// place, carrying the first and second differences from point to point.
+// What bounds it is instruction issue, so that layout is the one with the fewest
+// instructions: 16.8 a lane and update of the order-4 forced stencil in passes
+// of 4 levels, 10 of them arithmetic.  (Interleaved runs of two groups per lane
+// take four times the shuffles and a select per exchanged word, 23.8.  2^26
+// points, FP32, 100 levels: 5.91 ms then, 4.27 ms so; the compensated state on
+// 2^24 points 3.62 and 2.03 ms; FP64 on 2^22 points, 40 levels, bound by its
+// FP64 pipe, 4.48 and 3.63 ms.)
+//
+// The tile travels through a shared-memory stage: 16-byte asynchronous copies
+// in, coalesced in global memory and swizzled in the stage (see swizzle()), so
+// that the lanes' reads of their consecutive chunks do not collide in the
+// banks; the way back is the same stage in the other direction.  A warp's own
+// copies and stores need no barrier and no proxy fence, only __syncwarp().
+// A PE with one subdomain keeps it in registers for the whole launch.
+//
+// Halo values come from the ring entries of the neighbour's boundary words;
+// an entry's halves carry the level they belong to (see EntryTag), written and
+// read as single 16-byte accesses, so an entry is its own notification: one
+// read tells whether the level is there and brings it (a flag released after
+// the entry costs the writer a fence and the reader a second trip to the L2
+// cache: 16 subdomains of 256 FP64 points took 4.8 us a step that way, tiles
+// written back and re-read every step, and take 2.9).  One lane per level and
+// face reads them, a tile ahead; what is not there yet is read again when the
+// tile is reached (bounded).
 //
 // In an ensemble (BATCH) a tile is cnt consecutive subdomains of one instance
 // (see TileInfo; the faces between them at delay 0); the stencil factors,
 // delay bound and seed come from its records in shared memory; a face whose
 // record names no neighbour takes the instance's exact boundary values,
-// undelayed; a face whose neighbour is another PE's, or not in the adjacent
-// tile of the sweep (a periodic instance's wrap-around), goes through the
-// flags.
+// undelayed.
 //
 // PREC (FP32 state only) 1: the viscous term nu dt D2(u) is formed from the
 // stencil values in FP64 and added to u in FP64, rounded to FP32 once per
@@ -578,22 +765,27 @@ __device__ __forceinline__ T exact_ghost2(const BatchInst *binst, const BatchSub
 // new error as lo -- so that neither small increments nor the quantisation
 // of the stored field are lost to FP32 rounding.
 template <typename T, int ORDER, int GW, bool FORCED, bool FULL, bool BATCH, int PREC, bool BS>
-__device__ void run_pe(const Params &p, const Sweep &sw, long long lo, long long hi, uint64_t *bars, unsigned *hist,
-                       unsigned char *raw, unsigned char *stages, const T *sj, const T *cj, const T *spt,
-                       const T *cpt, const BatchSub *btab, int *s_count, volatile long long *s_epoch)
+__device__ void run_pe(const Params &p, const Sweep &sw, long long lo, int S, unsigned char *raw,
+                       unsigned char *stages, const T *sj, const T *cj, const T *spt, const T *cpt,
+                       const BatchSub *btab, int *s_count, volatile long long *s_epoch)
 {
     constexpr int R = ORDER / 2;
     constexpr int S_LEV = ORDER / 2 + 1;
     constexpr unsigned kAll = 0xffffffffu;
+    constexpr int NH = entry_halves<T, ORDER, PREC>();
+    constexpr int kEnt = kRingHalf * NH;                 // bytes of a ring entry
+    constexpr int CPG = (int)sizeof(T) / 4;              // 16-byte chunks per group of 4 points
+    constexpr int WPC = 16 / (int)sizeof(T);             // words per chunk
+    constexpr int NPT = 4 * GW;                          // points a lane holds at most
+    constexpr int NCH = GW * CPG;                        // chunks a lane holds at most
+    constexpr bool COMP = PREC == 2;
+    constexpr bool ONE_LANE = !(FULL && GW > 1);         // a tile may lie in one lane
+    constexpr bool bsync = BS;
+    constexpr bool PLAIN = sizeof(T) == 4 && ORDER == 2 && PREC == 0 && !BATCH && !FORCED;
+    using Stencil = StencilK<T, ORDER, PREC, PLAIN>;
     const int lane = threadIdx.x & 31;
-    const long long S = hi - lo;
-    // Groups of 4 points a lane holds consecutively (full single-domain
-    // tiles; else 1): register slot m of lane l is group
-    // VG l + m mod VG + 32 VG (m div VG), so that a lane updates runs of VG
-    // groups with register neighbours and exchanges words with its
-    // neighbour lanes once per run instead of once per group.
-    constexpr int VG = group_run<GW, FULL, BATCH, PREC>();
-    auto gidx = [&](int m) -> int { return VG * lane + (m % VG) + 32 * VG * (m / VG); };
+    const int gpl = FULL ? GW : p.gpl;                   // groups per lane
+    const int my_face = lane >> 4, my_m = lane & 15;     // halo work: lane 16 f + m serves face f
     // Blocked synchronous mode (AT_SYNC in passes of sb > 1 levels): every
     // delay is 0, a grid barrier precedes each pass, and a tile takes, instead
     // of the ring's per-level halo, its neighbours' edge strips of R sb points
@@ -605,226 +797,309 @@ __device__ void run_pe(const Params &p, const Sweep &sw, long long lo, long long
     // follows that.
     // (a separate instantiation, BS: the host launches it for AT_SYNC with
     // passes of more than one level only)
-    constexpr bool bsync = BS;
-    const long long ep_off = bsync ? 1 : 0;                 // grid barriers before the first pass
-    const long long n_ep = count_passes(sw, S_LEV) + ep_off; // arrivals of this launch
+    const int ep_off = bsync ? 1 : 0;                    // grid barriers before the first pass
+    const bool sync_mode = p.mode == kModeSync;
     if (S <= 0) {
         // a PE without subdomains still takes part in every grid barrier
-        if (p.mode == kModeSync) {
-            for (long long st = 1; st <= n_ep; ++st)
+        if (sync_mode) {
+            const int n_ep = count_passes(sw) + ep_off;  // arrivals of this launch
+            for (int st = 1; st <= n_ep; ++st)
                 if (!cta_grid_sync(p, s_count, s_epoch, st, st < n_ep)) break;
         }
         return;
     }
-    // the subdomains of tile t (single domain: tile t is subdomain t)
-    auto tile_info = [&](long long t) -> TileInfo {
+    // the subdomains of tile t of this PE (single domain: tile t is subdomain lo + t)
+    auto tile_info = [&](int t) -> TileInfo {
         if constexpr (BATCH) {
-            const int4 d = __ldg(p.tiles + t);
-            return TileInfo{(long long)d.x, (long long)d.y, d.z & 0xffff, d.z >> 16};
+            const int4 d = __ldg(p.tiles + lo + t);
+            return TileInfo{d.x, d.y, d.z & 0xffff, d.z >> 16};
         } else {
-            return TileInfo{t, t, 1, 0};
+            return TileInfo{(int)lo + t, 0, 1, 0};
         }
     };
-    long long rec_lo = 0;                // place of this PE's first record
-    if constexpr (BATCH) rec_lo = tile_info(lo).rec;
+    int rec_lo = 0;                      // place of this PE's first record
+    if constexpr (BATCH) rec_lo = tile_info(0).rec;
     // the first and last subdomain records of a tile (ensembles)
     auto rec_first = [&](const TileInfo &ti) -> const BatchSub & { return btab[ti.rec - rec_lo]; };
     auto rec_last = [&](const TileInfo &ti) -> const BatchSub & { return btab[ti.rec - rec_lo + ti.cnt - 1]; };
-    // whether face f of tile t takes its halo through the flags: its
-    // neighbour is not the adjacent tile of this PE's sweep (ensembles; the
-    // single domain: the PE's first and last tile)
-    auto link_edge = [&](long long t, const TileInfo &ti, int f) -> bool {
-        return f == 0 ? !(t - 1 >= lo && (ti.link & 1)) : !(t + 1 < hi && (ti.link & 2));
+    // whether face f of tile t is an edge of this PE's sweep: its neighbour is
+    // not the adjacent tile (ensembles; the single domain: the PE's first and
+    // last tile)
+    auto link_edge = [&](int t, const TileInfo &ti, int f) -> bool {
+        if constexpr (BATCH) return f == 0 ? !(t > 0 && (ti.link & 1)) : !(t + 1 < S && (ti.link & 2));
+        else return f == 0 ? t == 0 : t == S - 1;
     };
     const int NS = p.stages;
     // tiles loaded ahead; an alternating sweep revisits the subdomain of
     // position i after a turn 2i+1 tiles later, so at most 2 ahead there
-    int D = (int)((S - 1) < (NS - 1) ? (S - 1) : (NS - 1));
+    int D = S - 1 < NS - 1 ? S - 1 : NS - 1;
     if (sw.alt && D > 2) D = 2;
-    const long long Q = count_passes(sw, S_LEV) * S;
-    // groups of 4 points in the tile (an ensemble's tiles: cnt subdomains)
-    int NG = (int)(p.M / 4);
-    // owner of group NG-1 (compile-time when the tile is a multiple of 128 points)
-    int m_last = FULL ? GW - 1 : (NG - 1) >> 5;
-    int lane_last = FULL ? 31 : (NG - 1) & 31;
-    const T cA0 = (T)p.cA, cB0 = (T)p.cB;
-    const double cB64_0 = p.cB;
-    const size_t tile_bytes = (size_t)p.M * sizeof(T);                 // one subdomain
-    const size_t slot_stride = (size_t)p.P * 2 * kRingEntry;
-    const int up = (lane + 31) & 31, down = (lane + 1) & 31;
-    const bool edge_pub = !(p.skip_publish && blockIdx.x == 0 && threadIdx.x < 32);
-    unsigned *my_hist = hist + (lane & 1) * (kMaxL + 1);
+    // groups of the tile, owner of the last one (FULL: every lane's run is
+    // full, so the last group is the last of its lane)
+    const int M = (int)p.M;
+    int NG = M / 4;
+    int lane_last = (NG - 1) / gpl, m_last = FULL ? GW - 1 : (NG - 1) - lane_last * gpl;
+    const size_t tile_bytes = (size_t)M * sizeof(T);                   // one subdomain
+    const size_t slot_stride = (size_t)p.P * 2 * kEnt;
+    const unsigned tmask = (unsigned)p.T - 1u;
+    const unsigned n0lo = (unsigned)sw.n0;
+    const unsigned long long tag0 = entry_tag(sw.n0);    // tag of relative level 0
+    const bool stop_pub = p.skip_publish && blockIdx.x == 0 && threadIdx.x < 32;   // (test knob)
+    const T fX = sizeof(T) == 4 ? (T)p.fX32 : (T)p.fX;
+    const int err_off = p.stage_bytes / 2;               // (compensated state: the error words of a tile)
+    const Swizzle swz = FULL ? Swizzle::of(NCH) : Swizzle{p.swz_shift, p.swz_mask};
+    // this lane's chunk k in a stage
+    auto own_chunk = [&](int k) -> int { return FULL ? lane_chunk<NCH>(lane, k) : 16 * swz(gpl * CPG * lane + k); };
 
-    Cursor L{sw.n0, lo, pass_len(sw, sw.n0, S_LEV), false, 0};   // next tile to load
-    Cursor H = L;                                     // next tile whose halo is prepared
-    Cursor C = L;                                     // tile being processed
-
-    // --- state tile copies (lane 0): tile t goes to stage t % NS ------------
-    // (compensated state: the stage holds the tile, then its error words)
-    const size_t err_off = round_up((long long)tile_bytes * p.ktile, 128);
-    // (stage indices and phases are kept as running counters: no 64-bit
-    // division per tile)
-    auto issue_load = [&](int st, const Cursor &c) {
-        if (lane == 0) {
-            const TileInfo ti = tile_info(c.j);
-            const size_t bytes = tile_bytes * (size_t)ti.cnt;
-            uint64_t *bar = &bars[st];
-            mbar_arrive_expect_tx(bar, (unsigned)(PREC == 2 ? 2 * bytes : bytes));
-            bulk_load(stages + (size_t)st * p.stage_bytes,
-                      reinterpret_cast<const unsigned char *>(p.u) + (size_t)ti.s0 * tile_bytes, (unsigned)bytes, bar);
-            if constexpr (PREC == 2)
-                bulk_load(stages + (size_t)st * p.stage_bytes + err_off,
-                          reinterpret_cast<const unsigned char *>(p.ur) + (size_t)ti.s0 * tile_bytes, (unsigned)bytes,
-                          bar);
+    // --- state tile copies: every lane its 16-byte chunks, one group per tile
+    auto copy_in = [&](unsigned char *dst, const unsigned char *src, int nc) {
+        src += 16 * lane;
+        if (nc == 32 * NCH) {
+#pragma unroll
+            for (int t = 0; t < NCH; ++t) cp_async16(dst + swz.coalesced(lane, t), src + 512 * t);
+        } else {
+#pragma unroll
+            for (int t = 0; t < NCH; ++t)
+                if (lane + 32 * t < nc) cp_async16(dst + swz.coalesced(lane, t), src + 512 * t);
         }
     };
+    auto issue_load = [&](int st, int t) {
+        const TileInfo ti = tile_info(t);
+        const int nc = (int)tile_bytes * ti.cnt / 16;
+        unsigned char *dst = stages + st * p.stage_bytes;
+        const size_t off = (size_t)ti.s0 * tile_bytes;
+        copy_in(dst, reinterpret_cast<const unsigned char *>(p.u) + off, nc);
+        if constexpr (COMP) copy_in(dst + err_off, reinterpret_cast<const unsigned char *>(p.ur) + off, nc);
+        cp_async_commit();
+    };
 
-    // --- halo preparation (lane f for face f) -------------------------------
-    // Chooses the delay of face f of tile c and copies the delayed ring
-    // levels into raw buffer `buf`.  With block == false an edge face whose
-    // neighbour is not far enough yet is left pending (return 0); otherwise
-    // waits (bounded).  Returns 1 when done, -1 on abort.
+    // --- prescribed delays ----------------------------------------------------
     int kb = 0;                        // lane i: raw delay of (tile t0 + i/2, face i%2)
-    long long kb_t0 = -1;
-    auto raw_delay = [&](long long t, const Cursor &c) -> int {
+    unsigned kb_t0 = ~0u;
+    auto raw_delay = [&](unsigned t, const Cursor &c) -> int {
         // prescribed modes draw 16 tiles' delays at once (one per lane)
-        const long long t0 = t & ~15LL;
+        const unsigned t0 = t & ~15u;
         if (t0 != kb_t0) {
             // (n, j) of tile t0 + lane/2, stepping from c (tile t) back or forth
-            long long jj = c.j - (t - t0) + (lane >> 1), nn = c.n;
-            while (jj < lo) { jj += S; --nn; }
-            while (jj >= hi) { jj -= S; ++nn; }
+            int jj = c.j - (int)(t - t0) + (lane >> 1), nn = c.n;
+            while (jj < 0) { jj += S; --nn; }
+            while (jj >= S) { jj -= S; ++nn; }
             int k = 0;
-            if (t0 + (lane >> 1) < Q && nn >= sw.n0 && nn < sw.n0 + sw.n_steps) {
+            if (nn >= 0 && nn < sw.n_steps) {
                 // (prescribed delays: tiles of one subdomain)
                 const TileInfo tj = tile_info(jj);
                 if (p.mode == kModeSeeded) {
                     if constexpr (BATCH) {
                         const BatchSub &b = rec_first(tj);
-                        k = seeded_delay(b.seed, nn, b.lp, b.Pi, p.per_sub ? 0 : (lane & 1), b.L);
+                        k = seeded_delay(b.seed, sw.n0 + nn, b.lp, b.Pi, p.per_sub ? 0 : (lane & 1), b.L);
                     } else {
-                        k = seeded_delay(p.seed, nn, jj, p.P, p.per_sub ? 0 : (lane & 1), p.L);
+                        k = seeded_delay(p.seed, sw.n0 + nn, tj.s0, p.P, p.per_sub ? 0 : (lane & 1), p.L);
                     }
                 } else if (p.mode == kModeReplay) {
-                    k = p.delays[((nn - sw.n0) * p.P + tj.s0) * 2 + (lane & 1)];
+                    k = p.delays[((long long)nn * p.P + tj.s0) * 2 + (lane & 1)];
                 }
             }
             kb = k;
             kb_t0 = t0;
         }
-        const int i = 2 * (int)(t - t0);
-        const int k0 = __shfl_sync(kAll, kb, i), k1 = __shfl_sync(kAll, kb, i + 1);
-        return (lane & 1) ? k1 : k0;
+        return __shfl_sync(kAll, kb, 2 * (int)(t - t0) + my_face);
     };
 
-    int hk = 0;                        // lanes 0/1: delay at the start of the pass for the prepared tile
-    auto prep_halo = [&](long long t, const Cursor &c, int buf, bool block) -> int {
-        const int kr = (p.mode == kModeSeeded || p.mode == kModeReplay) ? raw_delay(t, c) : 0;
-        // phase 1: choose the delay and check (or wait for) the neighbour
-        int state = 1;
-        long long k = 0, q = 0;
-        bool bnd = false;              // exact boundary face (ensembles)
-        const TileInfo ti = tile_info(c.j);
-        if (lane < 2) {
-            const int f = lane;
-            const long long n = c.n;
-            const int len = c.len;
-            bool edge;
-            int Lj = p.L;
-            if constexpr (BATCH) {
-                const BatchSub &bf = rec_first(ti), &bl = rec_last(ti);
-                q = f ? bl.right : bf.left;
-                bnd = q < 0;
-                edge = !bnd && link_edge(c.j, ti, f);
-                Lj = bf.L;
-            } else {
-                q = (f == 0) ? (c.j == 0 ? p.P - 1 : c.j - 1) : (c.j == p.P - 1 ? 0 : c.j + 1);
-                edge = (f == 0) ? (c.j == lo) : (c.j == hi - 1);
+    // --- halo preparation -----------------------------------------------------
+    // Lanes 16 f + m serve face f of a tile: the delay (or, free running, the
+    // largest one the pass allows), and a first read of the neighbour's ring
+    // entry of level n - k - m.
+    unsigned long long hd[NH], ht[NH];   // the entry read: payload and level tag
+    unsigned long long h_tag = 0;        // the tag wanted
+    const unsigned char *h_at = nullptr; // the entry's address
+    bool h_act = false;                  // this lane reads one
+    int h_k = 0;                         // prescribed delay of the face (free running: 0)
+    int h_kmax = 0;                      // free running: largest delay at the pass start
+    int h_nb = 0;                        // the neighbour
+    TileInfo hti{0, 0, 1, 0};            // the tile prepared
+    T gvn = (T)0;                        // blocked synchronous mode: this lane's word of the edge strips
+    auto prep = [&](unsigned t, const Cursor &c) {
+        hti = tile_info(c.j);
+        const int f = my_face;
+        bool bnd = false, edge;
+        int Lj = p.L;
+        if constexpr (BATCH) {
+            const BatchSub &bf = rec_first(hti);
+            const long long nb = f ? rec_last(hti).right : bf.left;
+            bnd = nb < 0;
+            h_nb = bnd ? 0 : (int)nb;
+            edge = !bnd && link_edge(c.j, hti, f);
+            Lj = bf.L;
+        } else {
+            const int jg = hti.s0;
+            h_nb = f ? (jg + 1 == (int)p.P ? 0 : jg + 1) : (jg == 0 ? (int)p.P - 1 : jg - 1);
+            edge = link_edge(c.j, hti, f);
+        }
+        if constexpr (bsync) {
+            // the neighbours' edge strips at the pass's first level: lanes
+            // 0 .. G-1 the left neighbour's last G points, lanes 16 .. 16+G-1
+            // the right neighbour's first
+            const int G = R * c.len;
+            if (!bnd && my_m < G) {
+                const T *sp = reinterpret_cast<const T *>(
+                    p.strip + ((size_t)((c.pass & 1) * p.P + h_nb) * 2 + (1 - f)) * kStripBytes);
+                gvn = ld_cg(sp + (f ? my_m : p.strip_words - G + my_m));
             }
+        } else {
             // largest delay at the start of the pass such that the last inner
             // step stays within L, and no level below 0 is ever read
-            long long kmax = n - S_LEV + 1;
-            if (kmax < 0) kmax = 0;
-            if (kmax > Lj - (len - 1)) kmax = Lj - (len - 1);
-            k = kr;
-            if (k > kmax) k = kmax;
-            if (k < 0) k = 0;
-            if (edge && p.mode != kModeSync) {
-                const unsigned long long *fl = p.flag + q * 2 + (1 - f);
-                const long long need = (p.mode == kModeFree) ? n - kmax : n - k;
-                unsigned long long seen = ld_acquire(fl);
-                if ((long long)seen < need) {
-                    if (!block) state = 0;
-                    else if (!wait_flag(p, fl, need, &seen, n, q)) state = -1;
-                }
-                if (state == 1 && p.mode == kModeFree) {
-                    const long long avail = ((long long)seen < n) ? (long long)seen : n;
-                    k = n - avail;
-                }
+            int kmax = Lj - (c.len - 1);
+            if (sw.n0 + c.n < (long long)(kMaxL + S_LEV)) {
+                const int ks = (int)sw.n0 + c.n - S_LEV + 1;
+                kmax = ks < kmax ? ks : kmax;
             }
+            kmax = kmax < 0 ? 0 : kmax;
+            h_k = 0;
+            if (p.mode == kModeSeeded || p.mode == kModeReplay) {
+                const int kr = raw_delay(t, c);
+                h_k = kr < 0 ? 0 : kr < kmax ? kr : kmax;
+            }
+            h_kmax = (p.mode == kModeFree && edge) ? kmax : 0;
+            const int cnt = (h_k + h_kmax == 0 && c.len == 1) ? 1 : h_kmax + S_LEV;
+            h_act = my_m < cnt && !bnd;
+            const int d = c.n - h_k - my_m;              // relative level of this lane's entry
+            h_tag = tag0 + (long long)d;
+            h_at = p.ring + ((size_t)h_nb * 2 + (1 - f)) * kEnt + (size_t)((n0lo + (unsigned)d) & tmask) * slot_stride;
+            ld_tagged<NH>(h_act, h_at, hd, ht);
         }
-        // the warp agrees: any lane aborted -> -1, else any lane pending -> 0
-        const unsigned bad = __ballot_sync(kAll, state < 0), pend = __ballot_sync(kAll, state == 0);
-        if (bad) return -1;
-        if (pend) return 0;
-        // phase 2: both faces ready -- count, record and copy the levels
-        if (lane < 2) {
-            const int f = lane;
-            // (the synchronous modes use level n itself at every level: k = 0)
-            const int kstep = p.mode == kModeSync ? 0 : 1;
-            const long long sf = f ? ti.s0 + ti.cnt - 1 : ti.s0;      // the subdomain of face f
-            for (int i = 0; i < c.len; ++i) {
-                my_hist[k + kstep * i] += 1u;
-                if (p.delays && p.mode != kModeReplay)
-                    p.delays[((c.n - sw.n0 + i) * p.P + sf) * 2 + f] = (int8_t)(k + kstep * i);
-            }
-            if (BATCH && f == 0 && ti.cnt > 1) {
-                // the faces between the tile's subdomains: delay 0
-                for (int i = 0; i < c.len; ++i) {
-                    my_hist[0] += 2u * (unsigned)(ti.cnt - 1);
-                    if (p.delays && p.mode != kModeReplay)
-                        for (int s = 0; s + 1 < ti.cnt; ++s) {
-                            p.delays[((c.n - sw.n0 + i) * p.P + ti.s0 + s) * 2 + 1] = 0;
-                            p.delays[((c.n - sw.n0 + i) * p.P + ti.s0 + s + 1) * 2 + 0] = 0;
-                        }
-                }
-            }
-            hk = (int)k;
-            if constexpr (bsync) {
-                // the neighbour's edge strip at the pass's first level
-                const unsigned char *sb0 = p.strip +
-                    ((size_t)((c.pass & 1) * p.P + (bnd ? 0 : q)) * 2 + (1 - f)) * kStripBytes;
-                const int chunks = bnd ? 0 : p.strip_words * (int)sizeof(T) / 16;
-                for (int ch = 0; ch < chunks; ++ch)
-                    cp_async16(raw + (size_t)buf * kRawBytes + f * kRawFace + ch * 16, sb0 + ch * 16);
+    };
+    // Delay statistics: lane m counts the levels with delay m on its face
+    // (cnt16: the delay 16 that no lane stands for)
+    unsigned cnt_k = 0, cnt16 = 0;
+    auto entry_ok = [&]() -> bool {
+        bool ok = true;
+#pragma unroll
+        for (int h = 0; h < NH; ++h) ok = ok && ht[h] == h_tag;
+        return ok;
+    };
+    // Reads again (bounded) the entries of the prepared tile that are not
+    // there yet; free running, settles for the newest level that is there with
+    // the s - 1 before it, if it is recent enough.  `first`: place of the
+    // level n - k among the face's entries.  Returns false on abort.
+    auto wait_entries = [&](const Cursor &c, int &k, int &first) -> bool {
+        const int cnt = (h_k + h_kmax == 0 && c.len == 1) ? 1 : h_kmax + S_LEV;
+        const bool any = __any_sync(kAll, h_act);
+        (void)any;
+        const bool face = ((__ballot_sync(kAll, h_act) >> (lane & 16)) & 0xffffu) != 0u;   // (no exact boundary)
+        int base = 0;                  // offset of this lane's first entry
+        const unsigned long long t0 = global_ns();
+        for (int polls = 0;; ++polls) {
+            const unsigned seen = (__ballot_sync(kAll, h_act && entry_ok()) >> (lane & 16)) & 0xffffu;
+            bool ready = true;
+            if (!face) {
+                k = h_k;
+            } else if (h_kmax == 0) {
+                // the levels are given
+                const unsigned want = (1u << cnt) - 1u;
+                ready = (seen & want) == want;
+                k = h_k;
+            } else if (c.len == 1 && base == 0 && (seen & 1u)) {
+                k = 0;                                 // level n itself
+                first = 0;
             } else {
-                const unsigned char *rbase = p.ring + ((size_t)(bnd ? 0 : q) * 2 + (1 - f)) * kRingEntry;
-                const int levels = bnd ? 0 : (k == 0 && c.len == 1) ? 1 : S_LEV;
-                for (int m = 0; m < levels; ++m) {
-                    const long long lv = c.n - k - m;
-                    cp_async16(raw + (size_t)buf * kRawBytes + f * kRawFace + m * kRingEntry,
-                               rbase + (size_t)(lv & (p.T - 1)) * slot_stride);
+                unsigned run = seen & (seen >> 1);
+                if constexpr (S_LEV == 3) run &= seen >> 2;
+                run &= (2u << (h_kmax - base)) - 1u;
+                ready = run != 0u;
+                first = ready ? __ffs(run) - 1 : 0;
+                k = base + first;
+            }
+            if (__all_sync(kAll, ready)) return true;
+            if ((polls & 15) == 15) {
+                const bool late = (long long)(global_ns() - t0) > p.timeout_ns;
+                if (__any_sync(kAll, late || ld_relaxed(p.ctrl + kCtrlAbort) != 0)) {
+                    // (the first lane of a face that is not there reports it)
+                    if (late && !ready && my_m == 0) raise_timeout(p, kWhereFlag, sw.n0 + c.n, h_nb);
+                    return false;
                 }
+                if (polls > 64) __nanosleep(64);
+            }
+            // (delay bounds above 13: the oldest levels a face may use are
+            // read in turn with the newest 16)
+            if (!ready && h_kmax > 0 && cnt > 16) {
+                const int to = base ? 0 : cnt - 16, d = c.n - to - my_m;
+                base = to;
+                h_act = my_m + base < cnt;
+                h_tag = tag0 + (long long)d;
+                h_at = p.ring + ((size_t)h_nb * 2 + (1 - my_face)) * kEnt +
+                       (size_t)((n0lo + (unsigned)d) & tmask) * slot_stride;
+            }
+            if (!ready) ld_tagged<NH>(h_act, h_at, hd, ht);
+        }
+    };
+    int kcur = 0;                      // this face's delay at the pass start
+    // Settles the delays of the prepared tile, counts and records them and
+    // leaves the s entries of each face in `raw`.  Returns false on abort.
+    auto resolve = [&](const Cursor &c) -> bool {
+        int k = bsync ? 0 : h_k;
+        if constexpr (!bsync) {
+            int first = 0;
+            // (everything read is there: the levels given, or level n itself)
+            if (!__all_sync(kAll, !h_act || entry_ok())) {
+                if (!wait_entries(c, k, first)) return false;
+            }
+            // the entries of levels n - k - m, m = 0 .. s-1, in order
+            const unsigned e = (unsigned)(my_m - first);
+            if (h_act && e < (unsigned)S_LEV) {
+                unsigned long long *r = reinterpret_cast<unsigned long long *>(raw + my_face * kRawFace + e * kRawEntry);
+#pragma unroll
+                for (int h = 0; h < NH; ++h) r[h] = hd[h];
             }
         }
-        return 1;
+        // (the synchronous modes use level n itself at every level: k = 0)
+        if (sync_mode) cnt_k += my_m == 0 ? (unsigned)c.len : 0u;
+        else cnt_k += (unsigned)(my_m - k) < (unsigned)c.len ? 1u : 0u;
+        if (p.L > 15) cnt16 += (my_m == 0 && !sync_mode && (unsigned)(16 - k) < (unsigned)c.len) ? 1u : 0u;
+        // (the faces between a tile's subdomains: delay 0)
+        if constexpr (BATCH) cnt_k += lane == 0 ? 2u * (unsigned)(hti.cnt - 1) * (unsigned)c.len : 0u;
+        if (p.delays && p.mode != kModeReplay) {
+            const int kstep = sync_mode ? 0 : 1;
+            const int sf = my_face ? hti.s0 + hti.cnt - 1 : hti.s0;      // the subdomain of the face
+            for (int i = 0; i < c.len; ++i) {
+                int8_t *row = p.delays + (long long)(c.n + i) * p.P * 2;
+                if (my_m == 0) row[(size_t)sf * 2 + my_face] = (int8_t)(k + kstep * i);
+                if (BATCH && lane == 0)
+                    for (int s = 0; s + 1 < hti.cnt; ++s) {
+                        row[(size_t)(hti.s0 + s) * 2 + 1] = 0;
+                        row[(size_t)(hti.s0 + s + 1) * 2 + 0] = 0;
+                    }
+            }
+        }
+        kcur = k;
+        __syncwarp();
+        return true;
     };
 
     // --- prologue -------------------------------------------------------------
-    long long tl = 0;                  // next tile index to load
-    long long nl = 0;                  // loads issued
-    int sl = 0;                        // stage of the next load (nl % NS)
-    int sr = 0;                        // stage of the next loaded tile to use and the parity of its fill
-    unsigned ph = 0;
+    Cursor C{0, 0, pass_len(sw, 0), 0, false};        // tile being processed
+    Cursor L = C, N = C;                              // next tile to load; tile after C
+    advance(sw, N, S);
+    int lead = 0;                      // tile index of L minus that of C
+    int ahead = 0;                     // loads issued and not used yet
+    int sl = 0;                        // stage of the next load
+    int sr = 0;                        // stage of the next loaded tile to use
+    unsigned char *stage = stages;     // stage of the tile last read: its way back
     // after a load: move to the next tile that is loaded (a turn tile of an
-    // alternating sweep is not: it continues in registers)
-    auto next_load = [&]() {
-        const long long jj = L.j;
-        advance(sw, L, lo, hi, S_LEV);
-        ++tl;
-        while (sw.alt && L.j == jj && tl < Q) { advance(sw, L, lo, hi, S_LEV); ++tl; }
+    // alternating sweep is not: it continues in registers; nor is any later
+    // tile of a PE with one subdomain)
+    auto load_next = [&]() {
+        issue_load(sl, L.j);
+        const int jj = L.j;
+        advance(sw, L, S);
+        ++lead;
+        if (S == 1) {
+            L.n = sw.n_steps;
+        } else if (sw.alt && L.j == jj) {
+            advance(sw, L, S);
+            ++lead;
+        }
         sl = (sl + 1 == NS) ? 0 : sl + 1;
-        ++nl;
+        ++ahead;
     };
     bool ok = true;
     if constexpr (bsync) {
@@ -835,7 +1110,7 @@ __device__ void run_pe(const Params &p, const Sweep &sw, long long lo, long long
         const T *ust = reinterpret_cast<const T *>(p.u);
         long long nrec = S;
         if constexpr (BATCH) {
-            const TileInfo tl_ = tile_info(hi - 1);
+            const TileInfo tl_ = tile_info(S - 1);
             nrec = tl_.rec + tl_.cnt - rec_lo;
         }
         for (long long t = lane; t < nrec * 2 * sw4; t += 32) {
@@ -846,104 +1121,99 @@ __device__ void run_pe(const Params &p, const Sweep &sw, long long lo, long long
             const long long src = jj * p.M + (f ? p.M - sw4 : 0) + wd;
             reinterpret_cast<T *>(p.strip + ((size_t)jj * 2 + f) * kStripBytes)[wd] = ust[src];
         }
+        __syncwarp();
         if (!cta_grid_sync(p, s_count, s_epoch, 1, true)) ok = false;
+        __syncwarp();
     }
-    while (tl < D && tl < Q) { issue_load(sl, L); next_load(); }
-    bool pending = true;               // the halo of tile 0 is prepared in the loop
-    int k0cur = 0, k1cur = 0;
-    bool turn = false;                 // tile r continues tile r-1 in registers (alternating sweep)
-    T c[GW][4];                        // the tile's words, group g = lane + 32 m
-    T er[PREC == 2 ? GW : 1][4];       // compensated state: carried rounding errors
+    while (lead < D && L.n < sw.n_steps) load_next();
+    bool prepared = false;             // the halo of tile r has been prepared
+    bool turn = false;                 // tile r continues tile r-1 in registers
+    T c[NPT];                          // this lane's points
+    T er[COMP ? NPT : 1];              // compensated state: carried rounding errors
+    T F[FORCED ? NPT : 1];             // forcing (PREC 0: dt A sin x / cA; else dt A sin x)
 
-    for (long long r = 0; r < Q && ok; ++r) {
-        // state copy of tile r + D (stage of tile r - 1, complete: in order)
-        if (tl < Q && tl <= r + D) { issue_load(sl, L); next_load(); }
+    for (unsigned r = 0; C.n < sw.n_steps && ok; ++r) {
+        // state copy of tile r + D (stage of tile r - 1, written back)
+        if (lead <= D && L.n < sw.n_steps) load_next();
+        --lead;
         // synchronous algorithm: before the first tile of a pass (a step when
         // unblocked), all PEs have finished the previous pass (grid barrier,
         // Algorithm 1)
-        if (p.mode == kModeSync && C.pass > 0 && C.j == lo) {
+        if (sync_mode && C.pass > 0 && C.j == 0) {
             if (!cta_grid_sync(p, s_count, s_epoch, C.pass + ep_off, true)) { ok = false; break; }
-        }
-        // halo of tile r: prepared one tile ahead unless it was pending
-        const int buf = (int)(r & 1);
-        if (pending) {
-            if (prep_halo(r, C, buf, true) < 0) { ok = false; break; }
-            H = C;
-            advance(sw, H, lo, hi, S_LEV);
-        }
-        if (lane < 2) cp_async_wait_all();
-        k0cur = __shfl_sync(kAll, hk, 0);
-        k1cur = __shfl_sync(kAll, hk, 1);
-        __syncwarp();
-        // prepare the halo of tile r + 1 without blocking (in AT_SYNC it must
-        // wait for the grid barrier when tile r + 1 starts a new step).  Its
-        // internal right neighbour at the pass start was computed by tile
-        // r + 2 - S, which is tile r itself when S == 2: no prefetch then.
-        pending = true;
-        if (r + 1 < Q && (S != 2 || sw.alt)) {
-            const bool new_step = (H.j == lo);
-            if (!(p.mode == kModeSync && new_step)) {
-                const int st = prep_halo(r + 1, H, buf ^ 1, false);
-                if (st < 0) { ok = false; break; }
-                if (st > 0) {
-                    pending = false;
-                    advance(sw, H, lo, hi, S_LEV);
-                }
-            }
-        }
-        // the state tile (a turn tile is already in registers)
-        const T *stile = reinterpret_cast<const T *>(stages + (size_t)sr * p.stage_bytes);
-        if (!turn) {
-            int good = 1;
-            if (lane == 0 && !mbar_try_wait(&bars[sr], ph)) good = wait_stage(p, &bars[sr], ph);
-            good = __shfl_sync(kAll, good, 0);
             __syncwarp();
-            if (!good) { ok = false; break; }
-            if (++sr == NS) { sr = 0; ph ^= 1u; }
         }
-        const unsigned char *rw = raw + (size_t)buf * kRawBytes;
-        const long long j = C.j, n = C.n;                 // tile, level at the pass start
-        const int len = C.len;
-        const TileInfo ti = tile_info(j);
-        const long long s0 = ti.s0, s1 = ti.s0 + ti.cnt - 1;   // its first and last subdomain
-        T *ug = reinterpret_cast<T *>(p.u) + (size_t)s0 * p.M;
-        T cA = cA0, cB = cB0;
-        double cB64 = cB64_0;
+        if (!prepared) prep(r, C);
+        if (!resolve(C)) { ok = false; break; }
+        const TileInfo ti = hti;
+        T gv = gvn;
+        const int kf0 = kcur;
+        // read the entries of tile r + 1 (in AT_SYNC not across the grid
+        // barrier)
+        prepared = N.n < sw.n_steps && !(sync_mode && N.j == 0);
+        if (prepared) prep(r + 1, N);
+        const int n = C.n, len = C.len;                   // level at the pass start
+        const int s0 = ti.s0, s1 = ti.s0 + ti.cnt - 1;    // its first and last subdomain
+        T cA = sizeof(T) == 4 ? (T)p.cA32 : (T)p.cA;
+        T cr = COMP ? (T)p.cB32 : sizeof(T) == 4 ? (T)p.cr32 : (T)p.cr;
         bool bnd0 = false, bnd1 = false;
         if constexpr (BATCH) {
             const BatchSub &bf = rec_first(ti), &bl = rec_last(ti);
-            cA = (T)bf.cA;
-            cB = (T)bf.cB;
-            cB64 = bf.cB;
+            if constexpr (sizeof(T) == 4) { cA = bf.cA32; cr = bf.cr32; }
+            else { cA = (T)bf.cA; cr = (T)bf.cr; }
             bnd0 = bf.left < 0;
             bnd1 = bl.right < 0;
-            if constexpr (!FULL) {
-                NG = (int)(ti.cnt * p.M / 4);
-                m_last = (NG - 1) >> 5;
-                lane_last = (NG - 1) & 31;
-            }
+            NG = ti.cnt * M / 4;
+            lane_last = (NG - 1) / gpl;
+            if constexpr (!FULL) m_last = (NG - 1) - lane_last * gpl;
         }
-
+        const bool is_first = lane == 0, is_last = lane == lane_last;
+        // the state tile (a turn tile is already in registers)
         if (!turn) {
+            cp_async_wait(--ahead);
+            __syncwarp();
+            stage = stages + sr * p.stage_bytes;
+            if (++sr == NS) sr = 0;
 #pragma unroll
             for (int m = 0; m < GW; ++m) {
-                const int g = gidx(m);
-                if (FULL || g < NG) lds<T, 4>(stile + 4 * g, c[m]);
-                else { c[m][0] = c[m][1] = c[m][2] = c[m][3] = (T)0; }
-                if constexpr (PREC == 2) {
-                    const T *se =
-                        reinterpret_cast<const T *>(reinterpret_cast<const unsigned char *>(stile) + err_off);
-                    if (FULL || g < NG) lds<T, 4>(se + 4 * g, er[m]);
-                    else { er[m][0] = er[m][1] = er[m][2] = er[m][3] = (T)0; }
+                const bool has = FULL || (m < gpl && gpl * lane + m < NG);
+#pragma unroll
+                for (int h = 0; h < CPG; ++h) {
+                    // (FULL: lanes beyond the tile read what the stage holds)
+                    T *d = c + 4 * m + h * WPC;
+                    if (has) lds<T, WPC>(reinterpret_cast<const T *>(stage + own_chunk(m * CPG + h)), d);
+                    else
+#pragma unroll
+                        for (int e = 0; e < WPC; ++e) d[e] = (T)0;
+                    if constexpr (COMP) {
+                        T *de = er + 4 * m + h * WPC;
+                        if (has)
+                            lds<T, WPC>(reinterpret_cast<const T *>(stage + err_off + own_chunk(m * CPG + h)), de);
+                        else
+#pragma unroll
+                            for (int e = 0; e < WPC; ++e) de[e] = (T)0;
+                    }
                 }
             }
-        }
-        // A sin(x) dt = (dt A sin x_j) cos(i dx) + (dt A cos x_j) sin(i dx)
-        // (the tables hold subdomains lo-1 .. hi: entry j - lo + 1)
-        T fs = (T)0, fc = (T)0;
-        if constexpr (FORCED) {
-            fs = (T)(p.dtA * (double)spt[j - lo + 1]);
-            fc = (T)(p.dtA * (double)cpt[j - lo + 1]);
+            if constexpr (FORCED) {
+                // A sin(x) dt = (dt A sin x_j) cos(i dx) + (dt A cos x_j) sin(i dx)
+                // (the tables hold the PE's subdomains -1 .. S: entry j + 1),
+                // formed once per pass and kept in registers
+                const T fs = fX * spt[C.j + 1], fc = fX * cpt[C.j + 1];
+#pragma unroll
+                for (int m = 0; m < GW; ++m) {
+                    const bool has = FULL || (m < gpl && gpl * lane + m < NG);
+#pragma unroll
+                    for (int h = 0; h < CPG; ++h) {
+                        T sv[WPC], cv[WPC];
+                        const int at = has ? own_chunk(m * CPG + h) : 0;
+                        lds<T, WPC>(reinterpret_cast<const T *>(reinterpret_cast<const unsigned char *>(sj) + at), sv);
+                        lds<T, WPC>(reinterpret_cast<const T *>(reinterpret_cast<const unsigned char *>(cj) + at), cv);
+#pragma unroll
+                        for (int e = 0; e < WPC; ++e) F[4 * m + h * WPC + e] = forcing_point(fs, fc, sv[e], cv[e]);
+                    }
+                }
+            }
         }
 
         // blocked synchronous mode: ghost cells.  Lanes 0 .. G-1 hold the left
@@ -951,98 +1221,150 @@ __device__ void run_pe(const Params &p, const Sweep &sw, long long lo, long long
         // 16 .. 16+G-1 the right neighbour's points M .. M+G-1, at the level
         // being advanced (G = R len; at the pass start, the strips)
         const int G = R * len;
-        T gv = (T)0;
-        T fsl = (T)0, fcl = (T)0, fsr = (T)0, fcr = (T)0;    // forcing factors of the neighbours
-        if constexpr (bsync) {
-            const T *stl = reinterpret_cast<const T *>(rw);
-            const T *str = reinterpret_cast<const T *>(rw + kRawFace);
-            if (lane < G) gv = stl[p.strip_words - G + lane];
-            else if (lane >= 16 && lane < 16 + G) gv = str[lane - 16];
-            if constexpr (FORCED) {
-                fsl = (T)(p.dtA * (double)spt[j - lo]);
-                fcl = (T)(p.dtA * (double)cpt[j - lo]);
-                fsr = (T)(p.dtA * (double)spt[j - lo + 2]);
-                fcr = (T)(p.dtA * (double)cpt[j - lo + 2]);
+        T gF = (T)0;                                         // this ghost point's forcing
+        if constexpr (bsync && FORCED) {
+            if (my_m < G) {
+                const int sub = C.j + (my_face ? 2 : 0);
+                const int off = my_face ? my_m : M + my_m - G;
+                const int at = WPC * swz(off / WPC) + off % WPC;
+                gF = forcing_point(fX * spt[sub], fX * cpt[sub], sj[at], cj[at]);
             }
         }
 
-        // halo values of every inner level (delays k0 + i, k1 + i): lane
-        // x < 2 R len computes one of them once per tile; each level then
-        // takes its 2R values by shuffle
-        const bool hv_lanes = !bsync && 2 * R * len <= 32;
+        // halo values of every inner level (delays k + i): lane 16 f + x, x <
+        // R len, computes word x % R of level x / R once per tile; each level
+        // then takes its 2R values by shuffle
+        const bool hv_lanes = bsync || G <= 16;
         T hv = (T)0, hvl = (T)0;       // (hvl: lo word of a compensated state)
-        if (hv_lanes && lane < 2 * R * len) {
-            const int f = lane / (R * len), rem = lane % (R * len);
-            const unsigned char *rf = rw + f * kRawFace;
-            const int kf = (f ? k1cur : k0cur) + rem / R;
-            if constexpr (PREC == 2) {
-                if (BATCH && (f ? bnd1 : bnd0)) {
-                    hv = exact_ghost2<T, R>(p.binst, f ? rec_last(ti) : rec_first(ti), p.M, f, rem % R, n + rem / R,
-                                            hvl);
-                } else {
-                    hv = reinterpret_cast<const T *>(rf)[rem % R];
-                    hvl = approx_halo_lo<T, S_LEV, R>(rf, kf, rem % R);
-                }
+        if (!bsync && hv_lanes && my_m < G) {
+            const int i = my_m / R, q = my_m % R;
+            const unsigned char *rf = raw + my_face * kRawFace;
+            if (BATCH && (my_face ? bnd1 : bnd0)) {
+                const BatchSub &b = my_face ? rec_last(ti) : rec_first(ti);
+                if constexpr (COMP) hv = exact_ghost2<T, R>(p.binst, b, p.M, my_face, q, sw.n0 + n + i, hvl);
+                else hv = exact_ghost<T, R>(p.binst, b, p.M, my_face, q, sw.n0 + n + i);
+            } else if constexpr (COMP) {
+                hv = reinterpret_cast<const T *>(rf)[q];
+                hvl = approx_halo_lo<T, S_LEV, R>(rf, kf0 + i, q);
             } else {
-                if (BATCH && (f ? bnd1 : bnd0))
-                    hv = exact_ghost<T, R>(p.binst, f ? rec_last(ti) : rec_first(ti), p.M, f, rem % R, n + rem / R);
-                else
-                    hv = approx_halo<T, S_LEV>(rf, kf, rem % R);
+                hv = approx_halo<T, S_LEV>(rf, kf0 + i, q);
             }
         }
-        // this lane's ring entry (slot 0) and flag of the face it publishes,
-        // and whether the consumer across that face waits on the flag
-        // (lane_last == 0: lane 0 publishes both faces, face 1 via prel1)
-        const int pf = (lane == 0) ? 0 : 1;
-        const long long sp = pf ? s1 : s0;                  // the subdomain of that face
-        unsigned char *const pe0 = p.ring + ((size_t)sp * 2 + pf) * kRingEntry;
-        unsigned long long *const pflag = p.flag + sp * 2 + pf;
-        bool prel, prel1 = false;
-        if constexpr (BATCH) {
-            const BatchSub &bf = rec_first(ti), &bl = rec_last(ti);
-            const long long q0 = pf ? bl.right : bf.left;
-            prel = q0 >= 0 && link_edge(j, ti, pf);
-            prel1 = bl.right >= 0 && link_edge(j, ti, 1);
-        } else {
-            prel = pf ? j == hi - 1 : j == lo;
-            prel1 = j == hi - 1;
-        }
-        // one level of the tile, in place (cs and cd are the same array: a
-        // group's old words are copied into its window before it is written)
-        auto level = [&](int i, T (&cs)[GW][4], T (&cd)[GW][4]) {
-            const long long lev = n + i + 1;                 // level being computed
-            T hl[R], hr[R];
-            T hll[R], hrl[R];                                // lo words (compensated state)
-            if constexpr (bsync) {
-                // the halo of level n+i from the ghost lanes (an ensemble's
-                // domain ends: the exact values)
+        const int k0cur = hv_lanes ? 0 : __shfl_sync(kAll, kf0, 0), k1cur = hv_lanes ? 0 : __shfl_sync(kAll, kf0, 16);
+        // this lane's ring entry (slot 0) of the face it publishes, and the
+        // faces published (the test knob stops those across the sweep's edges)
+        unsigned char *const pe0 = p.ring + (is_first ? (size_t)s0 * 2 : (size_t)s1 * 2 + 1) * kEnt;
+        const Stencil K(cA, cr, p);
+        // one level of the tile, in place
+        auto level = [&](int i) {
+            const int lev = n + i + 1;                       // level being computed (relative)
+            // the R words left and right of the lane's run: the neighbour
+            // lanes' words, or the halo
+            T lw[R], rw[R], lwl[R], rwl[R];                  // (.l: lo words of a compensated state)
+            T hx[R], hxl[R];                                 // lane 0: left halo; others: right halo
+            T hy[R], hyl[R];                                 // right halo of a one-lane tile
+            T ownl[R], ownr[R];
+            if (hv_lanes) {
+                const int src_lane = is_first ? (bsync ? G - R : i * R) : (bsync ? 16 : 16 + i * R);
+                const T src = bsync ? gv : hv;
 #pragma unroll
                 for (int q = 0; q < R; ++q) {
-                    hll[q] = hrl[q] = (T)0;
-                    hl[q] = __shfl_sync(kAll, gv, G - R + q);
-                    hr[q] = __shfl_sync(kAll, gv, 16 + q);
-                    if constexpr (BATCH) {
-                        if (bnd0) hl[q] = exact_ghost<T, R>(p.binst, rec_first(ti), p.M, 0, q, n + i);
-                        if (bnd1) hr[q] = exact_ghost<T, R>(p.binst, rec_last(ti), p.M, 1, q, n + i);
+                    hx[q] = __shfl_sync(kAll, src, src_lane + q);
+                    if constexpr (COMP) hxl[q] = __shfl_sync(kAll, hvl, src_lane + q);
+                    if (ONE_LANE) {
+                        hy[q] = __shfl_sync(kAll, src, (bsync ? 16 : 16 + i * R) + q);
+                        if constexpr (COMP) hyl[q] = __shfl_sync(kAll, hvl, (bsync ? 16 : 16 + i * R) + q);
                     }
                 }
+                if constexpr (bsync && BATCH) {
+                    // an ensemble's domain ends: the exact values
+#pragma unroll
+                    for (int q = 0; q < R; ++q) {
+                        if (bnd0 && is_first)
+                            hx[q] = exact_ghost<T, R>(p.binst, rec_first(ti), p.M, 0, q, sw.n0 + n + i);
+                        if (bnd1 && is_last) {
+                            const T g = exact_ghost<T, R>(p.binst, rec_last(ti), p.M, 1, q, sw.n0 + n + i);
+                            if (ONE_LANE && is_first) hy[q] = g;
+                            else hx[q] = g;
+                        }
+                    }
+                }
+            } else {
+                // (long passes: R len > 16) the face's value, level by level
+#pragma unroll
+                for (int q = 0; q < R; ++q) {
+                    auto val = [&](int f, T &l) -> T {
+                        const unsigned char *rf = raw + f * kRawFace;
+                        const int kf = (f ? k1cur : k0cur) + i;
+                        l = (T)0;
+                        if (BATCH && (f ? bnd1 : bnd0)) {
+                            const BatchSub &b = f ? rec_last(ti) : rec_first(ti);
+                            if constexpr (COMP) return exact_ghost2<T, R>(p.binst, b, p.M, f, q, sw.n0 + n + i, l);
+                            else return exact_ghost<T, R>(p.binst, b, p.M, f, q, sw.n0 + n + i);
+                        }
+                        if constexpr (COMP) {
+                            l = approx_halo_lo<T, S_LEV, R>(rf, kf, q);
+                            return reinterpret_cast<const T *>(rf)[q];
+                        } else {
+                            return approx_halo<T, S_LEV>(rf, kf, q);
+                        }
+                    };
+                    hx[q] = val(is_first ? 0 : 1, hxl[q]);
+                    if (ONE_LANE) hy[q] = val(1, hyl[q]);
+                }
+            }
+            // (runs that are not full: the last word of a lane's run is in
+            // slot gpl - 1, and the last group may be in an earlier slot)
+            T tail[R], taill[R];
+#pragma unroll
+            for (int q = 0; q < R; ++q) {
+                tail[q] = c[NPT - R + q];
+                if constexpr (COMP) taill[q] = er[NPT - R + q];
+                if constexpr (!FULL) {
+#pragma unroll
+                    for (int m = 0; m + 1 < GW; ++m)
+                        if (m == gpl - 1) {
+                            tail[q] = c[4 * m + 4 - R + q];
+                            if constexpr (COMP) taill[q] = er[4 * m + 4 - R + q];
+                        }
+                }
+            }
+            if constexpr (bsync) {
+                // the tile's own edge words, for the ghost cells below
+#pragma unroll
+                for (int q = 0; q < R; ++q) {
+                    T el = tail[q];
+                    if constexpr (!FULL) {
+#pragma unroll
+                        for (int m = 0; m < GW; ++m) el = (m == m_last) ? c[4 * m + 4 - R + q] : el;
+                    }
+                    ownl[q] = __shfl_sync(kAll, c[q], 0);
+                    ownr[q] = __shfl_sync(kAll, el, lane_last);
+                }
+            }
+#pragma unroll
+            for (int q = 0; q < R; ++q) {
+                lw[q] = __shfl_up_sync(kAll, tail[q], 1);
+                rw[q] = __shfl_down_sync(kAll, c[q], 1);
+                lw[q] = is_first ? hx[q] : lw[q];
+                if constexpr (COMP) {
+                    lwl[q] = __shfl_up_sync(kAll, taill[q], 1);
+                    rwl[q] = __shfl_down_sync(kAll, er[q], 1);
+                    lwl[q] = is_first ? hxl[q] : lwl[q];
+                }
+                if (ONE_LANE) {
+                    hx[q] = is_first ? hy[q] : hx[q];
+                    if constexpr (COMP) hxl[q] = is_first ? hyl[q] : hxl[q];
+                }
+                if constexpr (FULL) {
+                    rw[q] = is_last ? hx[q] : rw[q];
+                    if constexpr (COMP) rwl[q] = is_last ? hxl[q] : rwl[q];
+                }
+            }
+            if constexpr (bsync) {
                 if (i + 1 < len) {
                     // the ghost cells of level n+i+1 from level n+i: ghost
                     // lanes and the tile's own edge words (not yet updated)
-                    T el[R];
-#pragma unroll
-                    for (int q = 0; q < R; ++q) el[q] = (T)0;
-#pragma unroll
-                    for (int m = 0; m < GW; ++m) {
-#pragma unroll
-                        for (int q = 0; q < R; ++q) el[q] = (m == m_last) ? cs[m][4 - R + q] : el[q];
-                    }
-                    T ownl[R], ownr[R];
-#pragma unroll
-                    for (int q = 0; q < R; ++q) {
-                        ownl[q] = __shfl_sync(kAll, cs[0][q], 0);
-                        ownr[q] = __shfl_sync(kAll, el[q], lane_last);
-                    }
                     const bool left = lane < 16;
                     const int xo = left ? lane - G : lane - 16;      // x, or x - M on the right
                     T w[2 * R + 1];
@@ -1055,217 +1377,84 @@ __device__ void run_pe(const Params &p, const Sweep &sw, long long lo, long long
                         else v = (y >= 0) ? gq : ((R == 1 || y == -1) ? ownr[R - 1] : ownr[0]);
                         w[jj + R] = v;
                     }
-                    T sv = (T)0, cv = (T)0;
-                    if constexpr (FORCED) {
-                        if (left ? lane < G : lane - 16 < G) {
-                            const int off = left ? (int)p.M + xo : xo;
-                            const int tp = 4 * table_group<VG>(off >> 2, (int)(p.M / 4)) + (off & 3);
-                            sv = sj[tp];
-                            cv = cj[tp];
-                        }
-                    }
-                    T unused = (T)0;
-                    gv = stencil_point<T, ORDER, FORCED, PREC>(w, w, cA, cB, cB64, left ? fsl : fsr, left ? fcl : fcr,
-                                                               sv, cv, unused);
-                }
-            } else {
-#pragma unroll
-            for (int q = 0; q < R; ++q) {
-                hll[q] = hrl[q] = (T)0;
-                if (hv_lanes) {
-                    hl[q] = __shfl_sync(kAll, hv, i * R + q);
-                    hr[q] = __shfl_sync(kAll, hv, R * len + i * R + q);
-                    if constexpr (PREC == 2) {
-                        hll[q] = __shfl_sync(kAll, hvl, i * R + q);
-                        hrl[q] = __shfl_sync(kAll, hvl, R * len + i * R + q);
-                    }
-                } else if constexpr (PREC == 2) {
-                    const unsigned char *rr = rw + kRawFace;
-                    if (BATCH && bnd0) {
-                        hl[q] = exact_ghost2<T, R>(p.binst, rec_first(ti), p.M, 0, q, n + i, hll[q]);
-                    } else {
-                        hl[q] = reinterpret_cast<const T *>(rw)[q];
-                        hll[q] = approx_halo_lo<T, S_LEV, R>(rw, k0cur + i, q);
-                    }
-                    if (BATCH && bnd1) {
-                        hr[q] = exact_ghost2<T, R>(p.binst, rec_last(ti), p.M, 1, q, n + i, hrl[q]);
-                    } else {
-                        hr[q] = reinterpret_cast<const T *>(rr)[q];
-                        hrl[q] = approx_halo_lo<T, S_LEV, R>(rr, k1cur + i, q);
-                    }
-                } else {
-                    hl[q] = (BATCH && bnd0) ? exact_ghost<T, R>(p.binst, rec_first(ti), p.M, 0, q, n + i)
-                                            : approx_halo<T, S_LEV>(rw, k0cur + i, q);
-                    hr[q] = (BATCH && bnd1) ? exact_ghost<T, R>(p.binst, rec_last(ti), p.M, 1, q, n + i)
-                                            : approx_halo<T, S_LEV>(rw + kRawFace, k1cur + i, q);
+                    gv = K.template point<FORCED>(w, gF);
                 }
             }
-            }
-            // One point: w[0 .. 2R] are the values at offsets -R .. R (w[R] the
-            // point itself), sv/cv the forcing table entries; returns the new
-            // value (compensated state: updates the carried error too).
-            auto point = [&](const T *w, const T *wl, T sv, T cv, T &err) -> T {
-                return stencil_point<T, ORDER, FORCED, PREC>(w, wl, cA, cB, cB64, fs, fc, sv, cv, err);
-            };
-            // lane l holds runs of VG groups of 4 points (group gidx(m) in
-            // slot m); the neighbour words of a run come from the adjacent
-            // lanes (lane 0 / 31: the other end of the warp at the previous /
-            // next run, or the halo), those within a run from the lane's own
-            // registers
-            T tail[R], rb[R];                                // old last words of the previous run; new last words of NG-1
-            T tail_l[R], rb_l[R];                            // (the same for the lo words, PREC 2)
+            // the lane's points, left to right
+            typename Stencil::Carry cy;
+            K.start(cy, lw, lwl, c, er);
+            T rb[R], rbl[R];                                 // new last words of the tile (its owner's)
 #pragma unroll
-            for (int q = 0; q < R; ++q) { tail[q] = (T)0; rb[q] = (T)0; tail_l[q] = (T)0; rb_l[q] = (T)0; }
-#pragma unroll
-            for (int b = 0; b < GW / VG; ++b) {
-                const int mf = b * VG, ml = mf + VG - 1;     // the run's first and last slot
-                T lh[R], rh[R];                              // words left of the run's first group, right of its last
-                T lhl[R], rhl[R];
+            for (int m = 0; m < GW; ++m) {
+                if (!FULL && m >= gpl) break;
+                T nx[R], nxl[R];                             // the words right of the group
 #pragma unroll
                 for (int q = 0; q < R; ++q) {
-                    const T to_next = (lane == 31) ? tail[q] : cs[ml][4 - R + q];
-                    lh[q] = __shfl_sync(kAll, to_next, up);
-                    const T to_prev = (lane == 0) ? cs[b + 1 < GW / VG ? mf + VG : mf][q] : cs[mf][q];
-                    rh[q] = __shfl_sync(kAll, to_prev, down);
-                    lhl[q] = rhl[q] = (T)0;
-                    if constexpr (PREC == 2) {
-                        const T ln = (lane == 31) ? tail_l[q] : er[ml][4 - R + q];
-                        lhl[q] = __shfl_sync(kAll, ln, up);
-                        const T lp = (lane == 0) ? er[b + 1 < GW / VG ? mf + VG : mf][q] : er[mf][q];
-                        rhl[q] = __shfl_sync(kAll, lp, down);
-                    }
+                    nx[q] = m + 1 < GW ? c[4 * (m + 1 < GW ? m + 1 : m) + q] : rw[q];
+                    if constexpr (COMP) nxl[q] = m + 1 < GW ? er[4 * (m + 1 < GW ? m + 1 : m) + q] : rwl[q];
                 }
-#pragma unroll
-                for (int q = 0; q < R; ++q) {
-                    tail[q] = cs[ml][4 - R + q];
-                    if constexpr (PREC == 2) tail_l[q] = er[ml][4 - R + q];
-                }
-                if (b == 0) {
+                if (!FULL && m >= m_last) {
 #pragma unroll
                     for (int q = 0; q < R; ++q) {
-                        lh[q] = (lane == 0) ? hl[q] : lh[q];
-                        if constexpr (PREC == 2) lhl[q] = (lane == 0) ? hll[q] : lhl[q];
+                        if (m == gpl - 1) {
+                            nx[q] = rw[q];
+                            if constexpr (COMP) nxl[q] = rwl[q];
+                        }
+                        if (m == m_last) {
+                            nx[q] = is_last ? hx[q] : nx[q];
+                            if constexpr (COMP) nxl[q] = is_last ? hxl[q] : nxl[q];
+                        }
                     }
                 }
-                const bool is_last = (ml == m_last) && (lane == lane_last);
-#pragma unroll
-                for (int q = 0; q < R; ++q) {
-                    rh[q] = is_last ? hr[q] : rh[q];
-                    if constexpr (PREC == 2) rhl[q] = is_last ? hrl[q] : rhl[q];
-                }
-#pragma unroll
-                for (int i = 0; i < VG; ++i) {
-                    const int m = mf + i;
-                    const int g = gidx(m);
-                    T v[4 + 2 * R];
-                    T vl[PREC == 2 ? 4 + 2 * R : 1];
+                K.template group<FORCED>(cy, c + 4 * m, COMP ? er + 4 * m : er, nx, nxl, FORCED ? F + 4 * m : F);
+                if (FULL ? m == GW - 1 : m == m_last) {
 #pragma unroll
                     for (int q = 0; q < R; ++q) {
-                        v[q] = lh[q];
-                        v[R + 4 + q] = (i == VG - 1) ? rh[q] : cs[m + 1 < GW ? m + 1 : m][q];
-                        lh[q] = cs[m][4 - R + q];            // old words: the next group's left neighbours
-                        if constexpr (PREC == 2) {
-                            vl[q] = lhl[q];
-                            vl[R + 4 + q] = (i == VG - 1) ? rhl[q] : er[m + 1 < GW ? m + 1 : m][q];
-                            lhl[q] = er[m][4 - R + q];
-                        }
-                    }
-#pragma unroll
-                    for (int e = 0; e < 4; ++e) {
-                        v[R + e] = cs[m][e];
-                        if constexpr (PREC == 2) vl[R + e] = er[m][e];
-                    }
-                    T s4[4], c4[4];
-                    if constexpr (FORCED) {
-                        // (full tiles: offsets known at compile time)
-                        const int gg = (FULL || g < NG) ? g : NG - 1;
-                        const int tg = table_group<VG>(gg, FULL ? 32 * GW : NG);
-                        lds<T, 4>(sj + 4 * tg, s4);
-                        lds<T, 4>(cj + 4 * tg, c4);
-                    }
-#pragma unroll
-                    for (int e = 0; e < 4; ++e)
-                        cd[m][e] = point(v + e, vl + (PREC == 2 ? e : 0), s4[e], c4[e],
-                                         er[PREC == 2 ? m : 0][PREC == 2 ? e : 0]);
-#pragma unroll
-                    for (int q = 0; q < R; ++q) rb[q] = (m == m_last) ? cd[m][4 - R + q] : rb[q];
-                    if constexpr (PREC == 2) {
-#pragma unroll
-                        for (int q = 0; q < R; ++q) rb_l[q] = (m == m_last) ? er[m][4 - R + q] : rb_l[q];
+                        rb[q] = c[4 * m + 4 - R + q];
+                        if constexpr (COMP) rbl[q] = er[4 * m + 4 - R + q];
                     }
                 }
             }
-            // publish the new boundary values and release the edge flags
-            // (face 0 by lane 0, face 1 by the owner of group NG-1; the
-            // tile's entry addresses and release conditions are set above)
-            if (lane == 0 || lane == lane_last) {
-                const size_t slot_off = (size_t)(lev & (p.T - 1)) * slot_stride;
-                const bool pub_ok = edge_pub || lev <= p.skip_step;
-                if (FULL || lane_last != 0) {
-                    T w[R], wl[R];             // word by word: no runtime choice between arrays
-#pragma unroll
-                    for (int q = 0; q < R; ++q) w[q] = pf ? rb[q] : cd[0][q];
-                    if constexpr (PREC == 2) {
-#pragma unroll
-                        for (int q = 0; q < R; ++q) wl[q] = pf ? rb_l[q] : er[0][q];
-                        st_entry2<R>(pe0 + slot_off, w, wl);
-                    } else {
-                        st_entry<T, R>(pe0 + slot_off, w);
-                    }
-                    if (p.mode == kModeSync) __threadfence();
-                    if (prel && pub_ok) st_release(pflag, (unsigned long long)lev);
-                } else {
-                    // one group: lane 0 publishes both faces
-#pragma unroll
-                    for (int f = 0; f < 2; ++f) {
-                        T w[R], wl[R];
-#pragma unroll
-                        for (int q = 0; q < R; ++q) w[q] = f ? rb[q] : cd[0][q];
-                        if constexpr (PREC == 2) {
-#pragma unroll
-                            for (int q = 0; q < R; ++q) wl[q] = f ? rb_l[q] : er[0][q];
-                            st_entry2<R>(pe0 + f * kRingEntry + slot_off, w, wl);
-                        } else {
-                            st_entry<T, R>(pe0 + f * kRingEntry + slot_off, w);
-                        }
-                        if (p.mode == kModeSync) __threadfence();
-                        if ((f ? prel1 : prel) && pub_ok) st_release(pflag + f, (unsigned long long)lev);
-                    }
-                }
+            // publish the new boundary values: face 0 by lane 0, face 1 by
+            // the owner of the last group
+            const size_t slot = (size_t)((n0lo + (unsigned)lev) & tmask) * slot_stride;
+            const unsigned long long tag = tag0 + (unsigned)lev;
+            bool pub0 = true, pub1 = true;
+            if (stop_pub && sw.n0 + lev > p.skip_step) {
+                pub0 = !link_edge(C.j, ti, 0);
+                pub1 = !link_edge(C.j, ti, 1);
             }
-            if constexpr (BATCH) {
+            {
+                T w[R], wl[R];             // word by word: no runtime choice between arrays
+#pragma unroll
+                for (int q = 0; q < R; ++q) {
+                    w[q] = is_first ? c[q] : rb[q];
+                    if constexpr (COMP) wl[q] = is_first ? er[q] : rbl[q];
+                }
+                st_entry<T, ORDER, PREC>((is_first && pub0) || (is_last && !is_first && pub1), pe0 + slot, w, wl, tag);
+                // (a one-lane tile: lane 0 publishes both faces)
+                if (ONE_LANE)
+                    st_entry<T, ORDER, PREC>(is_first && is_last && pub1, p.ring + ((size_t)s1 * 2 + 1) * kEnt + slot, rb,
+                                             rbl, tag);
+            }
+            if constexpr (BATCH && FULL) {
                 // the faces between the subdomains of a multi-subdomain tile
-                // (subdomains of 128, 256 or 512 points: a subdomain's first
-                // group is lane 0's, its last lane 31's): ring entries only,
-                // and only of the launch's last L + s levels -- no tile of this
-                // launch reads them, and a later launch with other tiles reads
-                // back to its first level - L - s + 1 at most
-                if (ti.cnt > 1 && (lane == 0 || lane == 31) && lev > sw.n0 + sw.n_steps - (p.L + S_LEV)) {
-                    const size_t slot_off = (size_t)(lev & (p.T - 1)) * slot_stride;
-                    const int gsh = p.M == 128 ? 0 : p.M == 256 ? 1 : 2;      // m slots per subdomain: 1 << gsh
-                    const int gmask = (1 << gsh) - 1;
+                // (a subdomain is M / (4 GW) whole lanes): ring entries only of
+                // the launch's last L + s levels -- no tile of this launch
+                // reads them, and a later launch with other tiles reads back
+                // to its first level - L - s + 1 at most
+                if (ti.cnt > 1 && lev > sw.n_steps - (p.L + S_LEV)) {
+                    const int lps = M / NPT, sidx = lane / lps, place = lane - sidx * lps;
+                    unsigned char *const e = p.ring + slot + ((size_t)(s0 + sidx) * 2) * kEnt;
+                    T w[R], wl[R];
 #pragma unroll
-                    for (int m = 0; m < GW; ++m) {
-                        const int sidx = m >> gsh;
-                        const bool fst = lane == 0 && (m & gmask) == 0 && sidx >= 1 && sidx < ti.cnt;
-                        const bool lst = lane == 31 && (m & gmask) == gmask && sidx + 1 < ti.cnt;
-                        if (!(fst || lst)) continue;
-                        const int fi = fst ? 0 : 1;
-                        T w[R], wl[R];
-#pragma unroll
-                        for (int q = 0; q < R; ++q) {
-                            w[q] = fst ? cd[m][q] : cd[m][4 - R + q];
-                            wl[q] = (T)0;
-                            if constexpr (PREC == 2) wl[q] = fst ? er[m][q] : er[m][4 - R + q];
-                        }
-                        unsigned char *e = p.ring + slot_off + ((size_t)(s0 + sidx) * 2 + fi) * kRingEntry;
-                        if constexpr (PREC == 2) st_entry2<R>(e, w, wl);
-                        else st_entry<T, R>(e, w);
-                    }
+                    for (int q = 0; q < R; ++q) { w[q] = c[NPT - R + q]; wl[q] = COMP ? er[COMP ? NPT - R + q : 0] : (T)0; }
+                    st_entry<T, ORDER, PREC>(place == 0 && sidx >= 1 && sidx < ti.cnt, e, c, er, tag);
+                    st_entry<T, ORDER, PREC>(place == lps - 1 && sidx + 1 < ti.cnt, e + kEnt, w, wl, tag);
                 }
             }
         };
-        for (int i = 0; i < len; ++i) level(i, c, c);
+        for (int i = 0; i < len; ++i) level(i);
         if constexpr (bsync) {
             // edge strips of the pass's last level for the next pass
             const int gq = p.strip_words / 4;
@@ -1276,58 +1465,67 @@ __device__ void run_pe(const Params &p, const Sweep &sw, long long lo, long long
             // of this tile and the fence of the arrival order them before it)
 #pragma unroll
             for (int m = 0; m < GW; ++m) {
-                const int g = gidx(m);
-                if (g < gq) stg4<T>(st0 + 4 * g, c[m]);
-                if (g >= NG - gq && g < NG) stg4<T>(st1 + 4 * (g - (NG - gq)), c[m]);
+                const int g = gpl * lane + m;
+                if (!FULL && m >= gpl) continue;
+                if (g < gq) stg4<T>(st0 + 4 * g, c + 4 * m);
+                if (g >= NG - gq && g < NG) stg4<T>(st1 + 4 * (g - (NG - gq)), c + 4 * m);
             }
         }
-        // the next tile; before a turn the words stay in registers
-        Cursor Cn = C;
-        advance(sw, Cn, lo, hi, S_LEV);
-        const bool keep = sw.alt && Cn.j == j && r + 1 < Q;
-        if (!keep) {
+        // before a turn, and with one subdomain, the words stay in registers
+        const bool keep = N.j == C.j && N.n < sw.n_steps;
+        if (!keep || p.levels) {
+            // back through the tile's stage to coalesced 16-byte stores
+            // (lanes beyond a FULL tile write chunks nobody reads)
 #pragma unroll
             for (int m = 0; m < GW; ++m) {
-                const int g = gidx(m);
-                if (FULL || g < NG) stg4<T>(ug + 4 * g, c[m]);
-                if constexpr (PREC == 2) {
-                    if (FULL || g < NG) stg4<T>(reinterpret_cast<T *>(p.ur) + (size_t)s0 * p.M + 4 * g, er[m]);
+                if (FULL || (m < gpl && gpl * lane + m < NG)) {
+#pragma unroll
+                    for (int h = 0; h < CPG; ++h) {
+                        stsv<T, WPC>(reinterpret_cast<T *>(stage + own_chunk(m * CPG + h)), c + 4 * m + h * WPC);
+                        if constexpr (COMP)
+                            stsv<T, WPC>(reinterpret_cast<T *>(stage + err_off + own_chunk(m * CPG + h)),
+                                         er + 4 * m + h * WPC);
+                    }
                 }
             }
-        }
-        if (p.levels) {
-            T *lg = reinterpret_cast<T *>(p.levels) + (size_t)((n + len) % p.levels_depth) * (size_t)p.N +
-                    (size_t)s0 * p.M;
+            __syncwarp();
+            const int nc = (int)tile_bytes * ti.cnt / 16;
+            auto copy_out = [&](const unsigned char *src, unsigned char *dst) {
+                dst += 16 * lane;
+                if (nc == 32 * NCH) {
 #pragma unroll
-            for (int m = 0; m < GW; ++m) {
-                const int g = gidx(m);
-                if (FULL || g < NG) stg4<T>(lg + 4 * g, c[m]);
+                    for (int t = 0; t < NCH; ++t)
+                        st_cg16(dst + 512 * t, *reinterpret_cast<const uint4 *>(src + swz.coalesced(lane, t)));
+                } else {
+#pragma unroll
+                    for (int t = 0; t < NCH; ++t)
+                        if (lane + 32 * t < nc)
+                            st_cg16(dst + 512 * t, *reinterpret_cast<const uint4 *>(src + swz.coalesced(lane, t)));
+                }
+            };
+            const size_t off = (size_t)s0 * tile_bytes;
+            if (!keep) {
+                copy_out(stage, reinterpret_cast<unsigned char *>(p.u) + off);
+                if constexpr (COMP) copy_out(stage + err_off, reinterpret_cast<unsigned char *>(p.ur) + off);
             }
+            if (p.levels)
+                copy_out(stage, reinterpret_cast<unsigned char *>(p.levels) +
+                                    (size_t)((sw.n0 + n + len) % p.levels_depth) * (size_t)p.N * sizeof(T) + off);
         }
-        // the next read of this tile is a bulk copy (async proxy), issued by
-        // lane 0 after the warp barrier
-        fence_proxy_async_global();
+        // orders this tile's stores (and the raw entries' reads) before the
+        // other lanes' next copies of it
         __syncwarp();
-        C = Cn;
-        turn = keep;
+        turn = N.j == C.j;
+        C = N;
+        advance(sw, N, S);
     }
     // synchronous algorithm: the last pass's arrival at the grid barrier
-    if (ok && p.mode == kModeSync) cta_grid_sync(p, s_count, s_epoch, n_ep, false);
+    if (ok && sync_mode) cta_grid_sync(p, s_count, s_epoch, count_passes(sw) + ep_off, false);
     // let every copy in flight land before the warp leaves
-    if (lane < 2) cp_async_wait_all();
-    if (lane == 0) {
-        for (long long t = (nl > NS ? nl - NS : 0); t < nl; ++t) {
-            const unsigned long long t0 = global_ns();
-            while (!mbar_try_wait(&bars[t % NS], (unsigned)((t / NS) & 1)) &&
-                   (long long)(global_ns() - t0) < p.timeout_ns) {
-            }
-        }
-    }
+    cp_async_wait(0);
     __syncwarp();
-    if (lane < 2) {
-        for (int i = 0; i <= p.L && i <= kMaxL; ++i)
-            if (my_hist[i]) atomicAdd(p.hist + i, (unsigned long long)my_hist[i]);
-    }
+    if (my_m <= p.L && cnt_k) atomicAdd(p.hist + my_m, (unsigned long long)cnt_k);
+    if (cnt16) atomicAdd(p.hist + 16, (unsigned long long)cnt16);
 }
 
 // ---------------------------------------------------------------------------
@@ -1342,34 +1540,32 @@ __global__ void __launch_bounds__(kThreads, AT_MIN_CTAS_PER_SM) at_stepper(const
     const long long lo = e * p.ntiles / p.E;                  // this PE's tiles
     const long long hi = (e + 1) * p.ntiles / p.E;
     const long long S = hi - lo;
-    uint64_t *bars = reinterpret_cast<uint64_t *>(smem + p.bar_off) + (size_t)w * p.stages;
-    unsigned *hist = reinterpret_cast<unsigned *>(smem + p.hist_off) + (size_t)w * 2 * (kMaxL + 1);
-    unsigned char *raw = smem + p.raw_off + (size_t)w * 2 * kRawBytes;
+    unsigned char *raw = smem + p.raw_off + (size_t)w * kRawBytes;
     unsigned char *stages = smem + p.stage_off + (size_t)w * p.stages * p.stage_bytes;
     T *tab = reinterpret_cast<T *>(smem + p.tab_off);
-    T *sj = tab, *cj = tab + p.M;
-    T *spt = tab + 2 * p.M + (size_t)w * 2 * (p.smax + 2), *cpt = spt + p.smax + 2;
+    T *sj = tab, *cj = tab + p.tab_words;
+    T *spt = tab + 2 * p.tab_words + (size_t)w * 2 * (p.smax + 2), *cpt = spt + p.smax + 2;
     BatchSub *btab = reinterpret_cast<BatchSub *>(smem + p.tab_off) + (size_t)w * p.smax;
     // time level of the state, advanced at the end of the previous launch
-    Sweep sw{*reinterpret_cast<const volatile long long *>(p.ctrl + kCtrlN0), p.n_steps, p.sb, p.alt != 0,
-             p.mode != kModeSync};
+    Sweep sw;
+    sw.n0 = *reinterpret_cast<const volatile long long *>(p.ctrl + kCtrlN0);
+    sw.n_steps = (int)p.n_steps;
+    sw.sb = p.sb;
+    sw.alt = p.alt != 0;
+    sw.single = (p.mode != kModeSync && sw.n0 < ORDER / 2) ? ORDER / 2 - (int)sw.n0 : 0;
 
     __shared__ int s_count;                   // grid-barrier arrivals of this CTA's warps
     __shared__ long long s_epoch;             // last grid barrier this CTA passed
     if (threadIdx.x == 0) { s_count = 0; s_epoch = 0; }
-    if (lane == 0) {
-        for (int i = 0; i < p.stages; ++i) mbar_init(&bars[i], 1);
-        mbar_fence_init();
-    }
-    for (int i = lane; i < 2 * (kMaxL + 1); i += 32) hist[i] = 0u;
     if (FORCED) {
         // sin/cos of the offsets j dx within a subdomain and of the subdomain
         // origins x0 + p M dx (FP64), so that A sin(x_i) needs two FMAs
         for (long long i = threadIdx.x; i < p.M; i += blockDim.x) {
             double sv, cv;
             sincos((double)i * p.dx, &sv, &cv);
-            constexpr int VG = group_run<GW, FULL, BATCH, PREC>();
-            const long long tp = 4LL * table_group<VG>((int)(i >> 2), (int)(p.M / 4)) + (i & 3);
+            constexpr int WPC = 16 / (int)sizeof(T);
+            const Swizzle swz{p.swz_shift, p.swz_mask};
+            const int tp = WPC * swz((int)i / WPC) + (int)i % WPC;
             sj[tp] = (T)sv;
             cj[tp] = (T)cv;
         }
@@ -1405,8 +1601,8 @@ __global__ void __launch_bounds__(kThreads, AT_MIN_CTAS_PER_SM) at_stepper(const
         if (p.mode != kModeSync && sw.sb > lmin + 1) sw.sb = lmin + 1;
     }
     __syncthreads();
-    run_pe<T, ORDER, GW, FORCED, FULL, BATCH, PREC, BS>(p, sw, lo, hi, bars, hist, raw, stages, sj, cj, spt, cpt,
-                                                       btab, &s_count, &s_epoch);
+    run_pe<T, ORDER, GW, FORCED, FULL, BATCH, PREC, BS>(p, sw, lo, (int)S, raw, stages, sj, cj, spt, cpt, btab, &s_count,
+                                                       &s_epoch);
     // the last CTA to finish advances the level of the state and rearms the
     // grid barrier for the next launch (every CTA has read the level by now)
     __syncthreads();
@@ -1422,20 +1618,29 @@ __global__ void __launch_bounds__(kThreads, AT_MIN_CTAS_PER_SM) at_stepper(const
 }
 
 // ---------------------------------------------------------------------------
-// state (re)initialisation: level-0 boundary values into ring slot 0, flags 0
+// state (re)initialisation: level-0 boundary values into ring slot 0 (the host
+// has cleared the ring)
 // ---------------------------------------------------------------------------
+// Ring entry of R words at u (a compensated state starts with lo words of 0).
+template <typename T, int R>
+__device__ __forceinline__ void put_entry(const Params &p, unsigned char *e, const T *u, long long level)
+{
+    const T v[2] = {u[0], R > 1 ? u[R - 1] : (T)0}, l[2] = {(T)0, (T)0};
+    if constexpr (sizeof(T) == 4 && R == 2) {
+        if (p.nh == 2) { st_entry<T, 2 * R, 2>(true, e, v, l, entry_tag(level)); return; }
+    }
+    st_entry<T, 2 * R, 0>(true, e, v, l, entry_tag(level));
+}
+
 template <typename T, int R>
 __global__ void at_init(const Params p)
 {
     const long long stride = (long long)gridDim.x * blockDim.x;
     for (long long j = (long long)blockIdx.x * blockDim.x + threadIdx.x; j < p.P; j += stride) {
         const T *u = reinterpret_cast<const T *>(p.u) + j * p.M;
-        T a[2] = {u[0], R > 1 ? u[1] : (T)0};
-        T b[2] = {u[p.M - R], R > 1 ? u[p.M - R + 1] : (T)0};
-        st_entry<T, R>(p.ring + ((size_t)j * 2 + 0) * kRingEntry, a);
-        st_entry<T, R>(p.ring + ((size_t)j * 2 + 1) * kRingEntry, b);
-        p.flag[j * 2 + 0] = 0ull;
-        p.flag[j * 2 + 1] = 0ull;
+        unsigned char *e = p.ring + (size_t)j * 2 * kRingHalf * p.nh;
+        put_entry<T, R>(p, e, u, 0);
+        put_entry<T, R>(p, e + kRingHalf * p.nh, u + p.M - R, 0);
     }
     if (blockIdx.x == 0) {
         if (threadIdx.x < kCtrlWords) p.ctrl[threadIdx.x] = 0;
@@ -1446,27 +1651,21 @@ __global__ void at_init(const Params p)
 
 // ---------------------------------------------------------------------------
 // restart from stored levels: ring slots of levels lo_level .. level from the
-// full fields levels[l mod depth], every flag at `level`, the control block
-// cleared with the state's level set to `level`
+// full fields levels[l mod depth] (the host has cleared the ring), the control
+// block cleared with the state's level set to `level`
 // ---------------------------------------------------------------------------
 template <typename T, int R>
 __global__ void at_restore(const Params p, const T *levels, long long depth, long long lo_level, long long level)
 {
     const long long nl = level - lo_level + 1;
     const long long stride = (long long)gridDim.x * blockDim.x;
-    const size_t slot_stride = (size_t)p.P * 2 * kRingEntry;
+    const size_t ent = (size_t)kRingHalf * p.nh;
     for (long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x; t < p.P * nl; t += stride) {
         const long long j = t % p.P, l = lo_level + t / p.P;
         const T *u = levels + (size_t)(l % depth) * (size_t)p.N + (size_t)j * p.M;
-        T a[2] = {u[0], R > 1 ? u[1] : (T)0};
-        T b[2] = {u[p.M - R], R > 1 ? u[p.M - R + 1] : (T)0};
-        unsigned char *e = p.ring + (size_t)(l & (p.T - 1)) * slot_stride + (size_t)j * 2 * kRingEntry;
-        st_entry<T, R>(e, a);
-        st_entry<T, R>(e + kRingEntry, b);
-        if (l == level) {
-            p.flag[j * 2 + 0] = (unsigned long long)level;
-            p.flag[j * 2 + 1] = (unsigned long long)level;
-        }
+        unsigned char *e = p.ring + ((size_t)(l & (p.T - 1)) * p.P + j) * 2 * ent;
+        put_entry<T, R>(p, e, u, l);
+        put_entry<T, R>(p, e + ent, u + p.M - R, l);
     }
     if (blockIdx.x == 0) {
         if (threadIdx.x < kCtrlWords) p.ctrl[threadIdx.x] = 0;
