@@ -21,6 +21,7 @@
 #include "at_adjoint.cuh"
 #include "at_kernels.cuh"
 #include "at_kernels3d_blk.cuh"
+#include "at_kernels3d_v4.cuh"
 
 void *atk_stepper_kernel_f32(int order, int gw, bool forced, bool full);
 void *atk_stepper_kernel_f32v(int order, int gw, bool forced, bool full);
@@ -40,9 +41,10 @@ void *atk_restore_kernel_f32(int order);
 void *atk_restore_kernel_f64(int order);
 void *atk_adjoint_kernel(int w, int order);
 void *atk_adjoint_own_kernel(int w, int order);
-void *atk_stepper3d_kernel(int w, int tc, int vw);
-void *atk_stepper3d_iso_kernel(int w, int tc, int vw);
-void *atk_system3d_kernel(int w, int tc, int nf, int vw);
+void *atk_stepper3d_kernel(int w, int tc);
+void *atk_stepper3d_iso_kernel(int w, int tc);
+void *atk_system3d_kernel(int w, int tc, int nf);
+void *atk_stepper3d_v4_kernel(int nf, int nt, int tc, int iso);
 void *atk_init3d_kernel(int w);
 void *atk_stepper3d_blk_kernel(int w, int sb, int iso);
 void *atk_stepper3d_blk32_kernel(int w, int sb, int iso);
@@ -605,34 +607,40 @@ static int create3d(const at_grid *grid, int64_t P, int L, int nf, const double 
     cudaDeviceGetAttribute(&smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
     if (!coop) return fail(AT_ERR_RESIDENCY, "device does not support cooperative launch");
 
-    // a thread takes one group of vw = 4 consecutive columns (FP32 planes of
-    // 1024 points: every thread busy) or 1, 2 or 4 single columns
+    // FP32 with rows of a power of two of 4-point groups (a row lies in one
+    // warp): the kernel with one or two groups of 4 consecutive columns per
+    // thread, CTAs as small as the plane allows; else 256 threads of 1, 2 or 4
+    // single columns
     const int pw = d.m[0] * d.m[1];
-    // (a row of sub[0] / 4 groups must lie within one warp: sub[0] <= 128)
-    const int vw = (w == 4 && d.m[0] % 4 == 0 && d.m[0] <= 128 && pw == 4 * atk::kThreads3) ? 4 : 1;
-    // the scalar equation with groups of 4: CTAs of 128 threads, two groups
-    // each (4 CTAs per SM: one CTA's tile start overlaps the others' planes)
-    const int nt = (vw == 4 && nf == 1) ? 128 : atk::kThreads3;
-    const int tc = vw == 4 ? (nf == 1 ? 2 : 1) : pw <= atk::kThreads3 ? 1 : pw <= 2 * atk::kThreads3 ? 2 : 4;
-    if (nf > 1 && vw == 1 && tc > 2) return fail(AT_ERR_ARG, "the 3D system needs sub[0] * sub[1] <= 512 (or 1024, FP32)");
+    const bool v4 = w == 4 && d.m[0] <= 128 && (d.m[0] & (d.m[0] - 1)) == 0;
+    const int groups = pw / 4;
+    const int nt = !v4 ? atk::kThreads3 : groups <= 32 ? 32 : groups <= 64 ? 64 : (groups <= 128 || nf == 1) ? 128 : 256;
+    const int teams = (v4 && nf == 1 && groups <= nt) ? atk::kThreads3 / nt : 1;   // (see at_stepper3d_v4)
+    const int tc = v4 ? (groups > nt ? 2 : 1) : pw <= atk::kThreads3 ? 1 : pw <= 2 * atk::kThreads3 ? 2 : 4;
+    if (nf > 1 && !v4 && tc > 2) return fail(AT_ERR_ARG, "the 3D system needs sub[0] * sub[1] <= 512 (or 1024, FP32)");
     const int sb = grid->steps_per_pass > 0 ? grid->steps_per_pass : 1;
     if (nf > 1 && sb > 1) return fail(AT_ERR_ARG, "the 3D system takes one level per pass");
     // (the scalar equation with equal spacing on the three axes: one
     // coefficient pair, the neighbours summed first)
     const int iso = dx[0] == dx[1] && dx[1] == dx[2];
-    void *kern = nf == 1 ? (iso ? atk_stepper3d_iso_kernel(w, tc, vw) : atk_stepper3d_kernel(w, tc, vw))
-                         : atk_system3d_kernel(w, tc, nf, vw);
+    void *kern = v4 ? atk_stepper3d_v4_kernel(nf, nt, tc, iso)
+                 : nf == 1 ? (iso ? atk_stepper3d_iso_kernel(w, tc) : atk_stepper3d_kernel(w, tc))
+                           : atk_system3d_kernel(w, tc, nf);
     // plane buffers: at least 3 (planes z and z+1 in use, one arriving), at most sub[2]
     int stages = grid->stages > 0 ? grid->stages : 4;
     if (stages < 3) stages = 3;
     if (stages > d.m[2]) stages = d.m[2];
-    atk::Smem3 sl3 = atk::smem3_layout(d.m[0], d.m[1], d.m[2], w, stages, nf);
-    while (sl3.total > smem_optin && stages > 3) sl3 = atk::smem3_layout(d.m[0], d.m[1], d.m[2], w, --stages, nf);
-    if (sl3.total > smem_optin) return fail(AT_ERR_RESIDENCY, "shared memory %lld exceeds %d", sl3.total, smem_optin);
-    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sl3.total);
+    auto smem_for = [&](int st) {
+        return v4 ? teams * atk::smem3v4_layout(d.m[0], d.m[1], d.m[2], st, nf).total
+                  : atk::smem3_layout(d.m[0], d.m[1], d.m[2], w, st, nf).total;
+    };
+    while (smem_for(stages) > smem_optin && stages > 3) --stages;
+    const long long smem = smem_for(stages);
+    if (smem > smem_optin) return fail(AT_ERR_RESIDENCY, "shared memory %lld exceeds %d", smem, smem_optin);
+    e = allow_smem(kern, smem_optin);
     if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute");
     int occ = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, nt, (size_t)sl3.total);
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, nt * teams, (size_t)smem);
     if (e != cudaSuccess) return cuda_fail(e, "cudaOccupancyMaxActiveBlocksPerMultiprocessor");
     int64_t G = grid->max_ctas > 0 ? grid->max_ctas : (int64_t)occ * sms;
     if (G > P) G = P;
@@ -646,7 +654,7 @@ static int create3d(const at_grid *grid, int64_t P, int L, int nf, const double 
     h->dim = 3;
     h->d3 = d;
     h->tc = tc;
-    h->nt3 = nt;
+    h->nt3 = nt * teams;
     h->nf = nf;
     for (int f = 0; f < nf; ++f) h->kappa[f] = kappa[f];
     h->N = (int64_t)nf * d.n[0] * d.n[1] * d.n[2];   // words of the state (all fields)
@@ -662,7 +670,7 @@ static int create3d(const at_grid *grid, int64_t P, int L, int nf, const double 
     h->init_kernel = atk_init3d_kernel(w);
     h->G = (int)G;
     h->stages = stages;
-    h->smem = (int)sl3.total;
+    h->smem = (int)smem;
     h->sb = sb;
     h->lmin = L;
     h->kernel_b3 = nullptr;
@@ -682,7 +690,7 @@ static int create3d(const at_grid *grid, int64_t P, int L, int nf, const double 
             delete h;
             return fail(AT_ERR_RESIDENCY, "blocked 3D passes: shared memory %lld exceeds %d", sb3.total, smem_optin);
         }
-        e = cudaFuncSetAttribute(kb, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sb3.total);
+        e = allow_smem(kb, smem_optin);
         if (e != cudaSuccess) { delete h; return cuda_fail(e, "cudaFuncSetAttribute"); }
         int occb = 0;
         e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occb, kb, atk::kThreads3b, (size_t)sb3.total);

@@ -11,12 +11,10 @@
 // plane (an m0 x m1 box) is brought into one of `stages` shared-memory buffers
 // by one TMA tensor copy (3D tensor map over the state; completion counted on
 // the stage's mbarrier), several planes ahead; the last warp to finish with a
-// stage (a shared counter per stage) refills it.  A thread owns up to TC
-// groups of VW consecutive (x, y) columns; it keeps the values of its columns
-// at planes z-1, z in registers, reads the plane z+1 and the y neighbours as
-// VW-word vectors, and the two x neighbours beyond a group by warp shuffles
-// (VW = 4) or as single words from shared memory (VW = 1).  The halo planes
-// of a tile are staged once at its start, face by face, one warp per face.
+// stage (a shared counter per stage) refills it.  A thread owns up to TC (x, y)
+// columns; it keeps their values at planes z-1, z in registers and reads the
+// other neighbours from shared memory.  The halo planes of a tile are staged
+// once at its start, face by face, one warp per face.
 // Neighbours across a subdomain face come from the ring of face planes:
 // entry [slot][subdomain][face] holds the face's boundary values at level
 // slot (faces 0/1: the x = 0 / x = m0-1 planes indexed [z][y]; 2/3: y planes
@@ -24,6 +22,9 @@
 // levels n-k, n-k-1.  After a tile every face's progress flag is released.
 // The update is written in place; the next read of a plane is a bulk copy,
 // so writers fence the async proxy before it is issued.
+//
+// (This kernel serves FP64 and rows that are no power of two of 4-point groups;
+// the others take at_kernels3d_v4.cuh.)
 //
 // Delays: one per (level, subdomain, face): seeded (counter (n P + p) 6 + f),
 // replayed, free-running (read off the neighbour's flag, waiting only while
@@ -37,11 +38,16 @@
 
 namespace atk {
 
-constexpr int kThreads3 = 256;          // threads of a CTA (128 for groups of 4 columns)
+constexpr int kThreads3 = 256;          // threads of a CTA
 constexpr int kMaxFields3 = 6;          // fields of the system (u, v, w and up to 3 scalars)
 #ifndef AT_MIN_CTAS_3D
 #define AT_MIN_CTAS_3D 2      // resident CTAs per SM the 3D stepper is compiled for
 #endif
+
+template <int V>
+struct IntC {
+    static constexpr int value = V;
+};
 
 struct Params3 {
     void *u;
@@ -181,11 +187,6 @@ __device__ __forceinline__ T *ring_entry(const Params3 &p, long long level, long
            (((size_t)(level & (p.T - 1)) * p.P + sub) * 6 + face) * (size_t)p.face_words * (size_t)p.nf;
 }
 
-// NF fields stored one after another; SYS: the system of Eq. BS (fields 0, 1,
-// 2 are the velocity (u, v, w), each field is advected by it and diffused with
-// its own kappa); otherwise NF = 1 and the scalar equation
-// u_t + u (u_x + u_y + u_z) = nu lap u.  A plane of every field arrives with
-// one copy of a 4D tensor map (x, y, z, field).
 // VW consecutive words (VW = 1 or 4; 16-byte aligned for 4) to global memory
 template <typename T, int VW>
 __device__ __forceinline__ void stv(T *g, const T *v)
@@ -198,10 +199,15 @@ __device__ __forceinline__ void stv(T *g, const T *v)
     }
 }
 
+// NF fields stored one after another; SYS: the system of Eq. BS (fields 0, 1,
+// 2 are the velocity (u, v, w), each field is advected by it and diffused with
+// its own kappa); otherwise NF = 1 and the scalar equation
+// u_t + u (u_x + u_y + u_z) = nu lap u.  A plane of every field arrives with
+// one copy of a 4D tensor map (x, y, z, field).
 // ISO (the scalar equation): equal spacing on the three axes, one
 // coefficient pair, the six neighbours summed before scaling
-template <typename T, int TC, int NF, bool SYS, int VW, int NT = kThreads3, bool ISO = false>
-__global__ void __launch_bounds__(NT, NT == kThreads3 ? AT_MIN_CTAS_3D : 2 * AT_MIN_CTAS_3D)
+template <typename T, int TC, int NF, bool SYS, bool ISO = false>
+__global__ void __launch_bounds__(kThreads3, AT_MIN_CTAS_3D)
     at_stepper3d(const Params3 p, const __grid_constant__ CUtensorMap tmap)
 {
     extern __shared__ __align__(128) unsigned char smem[];
@@ -239,7 +245,7 @@ __global__ void __launch_bounds__(NT, NT == kThreads3 ? AT_MIN_CTAS_3D : 2 * AT_
     T *u = reinterpret_cast<T *>(p.u);
     const long long field_words = p.n0 * p.n1 * p.n2;
 
-    constexpr int kWarps3 = NT / 32;
+    constexpr int kWarps3 = kThreads3 / 32;
     // per stage: warps done with its plane (the last one refills it), fills issued
     int *s_done = reinterpret_cast<int *>(bars + NS), *s_fills = s_done + NS;
     if (tid < NS) {
@@ -248,7 +254,7 @@ __global__ void __launch_bounds__(NT, NT == kThreads3 ? AT_MIN_CTAS_3D : 2 * AT_
         s_fills[tid] = 0;
     }
     if (tid == 0) { mbar_fence_init(); *s_flag = 0; }
-    for (int i = tid; i <= kMaxL; i += NT) hist[i] = 0u;
+    for (int i = tid; i <= kMaxL; i += kThreads3) hist[i] = 0u;
     __syncthreads();
 
     // word offset of the first point of subdomain `sub` in u
@@ -281,23 +287,20 @@ __global__ void __launch_bounds__(NT, NT == kThreads3 ? AT_MIN_CTAS_3D : 2 * AT_
     // faces touched (x: by the group's first / last column)
     int cx[TC], cy[TC], coff[TC], cface[TC];
     bool cv[TC];
-    const int GR = m0 / VW;                  // groups per row (the host checks VW | m0)
 #pragma unroll
     for (int q = 0; q < TC; ++q) {
-        const int c = tid + NT * q;
-        cv[q] = c < PW / VW;
-        cx[q] = cv[q] ? (c % GR) * VW : 0;
-        cy[q] = cv[q] ? c / GR : 0;
+        const int c = tid + kThreads3 * q;
+        cv[q] = c < PW;
+        cx[q] = cv[q] ? c % m0 : 0;
+        cy[q] = cv[q] ? c / m0 : 0;
         coff[q] = cy[q] * (int)p.n0 + cx[q];
-        cface[q] = (cx[q] == 0 ? 1 : 0) | (cx[q] + VW == m0 ? 2 : 0) | (cy[q] == 0 ? 4 : 0) | (cy[q] == m1 - 1 ? 8 : 0);
+        cface[q] = (cx[q] == 0 ? 1 : 0) | (cx[q] + 1 == m0 ? 2 : 0) | (cy[q] == 0 ? 4 : 0) | (cy[q] == m1 - 1 ? 8 : 0);
     }
-    T prev[NF][TC][VW], cur[NF][TC][VW];
+    T prev[NF][TC], cur[NF][TC];
 #pragma unroll
     for (int f = 0; f < NF; ++f)
 #pragma unroll
-        for (int q = 0; q < TC; ++q)
-#pragma unroll
-            for (int e = 0; e < VW; ++e) prev[f][q][e] = cur[f][q][e] = (T)0;
+        for (int q = 0; q < TC; ++q) prev[f][q] = cur[f][q] = (T)0;
 
     if (tid == 0)
         for (int st = 0; st < NS && st < Q; ++st) issue_plane(st, tx0, ty0, tz0 + st);
@@ -344,7 +347,7 @@ __global__ void __launch_bounds__(NT, NT == kThreads3 ? AT_MIN_CTAS_3D : 2 * AT_
         const long long base = tile_base(sub);
 #pragma unroll
         for (int f = 0; f < 6; ++f) rf[f] = ring_entry<T>(p, lv + 1, sub, f);
-        // warp w takes faces w, w + NT/32, ... (< 6): its lane 0 chooses the
+        // warp w takes faces w, w + kThreads3/32, ... (< 6): its lane 0 chooses the
         // delay and checks (or waits for) the neighbour's flag, then the warp
         // stages the face's halo plane -- the neighbour's facing ring
         // entries, extrapolated once with the delay (16-byte loads where aligned)
@@ -430,8 +433,8 @@ __global__ void __launch_bounds__(NT, NT == kThreads3 ? AT_MIN_CTAS_3D : 2 * AT_
 #pragma unroll
                 for (int q = 0; q < TC; ++q) {
                     if (!cv[q]) continue;
-                    lds<T, VW>(hz0 + f * hwz + cy[q] * m0 + cx[q], prev[f][q]);
-                    lds<T, VW>(st0 + f * PW + cy[q] * m0 + cx[q], cur[f][q]);
+                    prev[f][q] = hz0[f * hwz + cy[q] * m0 + cx[q]];
+                    cur[f][q] = st0[f * PW + cy[q] * m0 + cx[q]];
                 }
             }
         }
@@ -449,71 +452,48 @@ __global__ void __launch_bounds__(NT, NT == kThreads3 ? AT_MIN_CTAS_3D : 2 * AT_
             const int zy = z * m1, zx = z * m0;
 #pragma unroll
             for (int q = 0; q < TC; ++q) {
-                if (VW == 1 && !cv[q]) continue;            // groups of 4: every thread has one
+                if (!cv[q]) continue;
                 const int x = cx[q], y = cy[q], c = y * m0 + x;
                 const int fc = cface[q];
                 // advecting velocity at the points, level n (the system)
-                T Uv[VW], Vv[VW], Wv[VW];
-#pragma unroll
-                for (int e = 0; e < VW; ++e) {
-                    Uv[e] = SYS ? cur[0][q][e] : (T)0;
-                    Vv[e] = SYS ? cur[1 % NF][q][e] : (T)0;
-                    Wv[e] = SYS ? cur[2 % NF][q][e] : (T)0;
-                }
+                const T Uv = SYS ? cur[0][q] : (T)0, Vv = SYS ? cur[1 % NF][q] : (T)0, Wv = SYS ? cur[2 % NF][q] : (T)0;
 #pragma unroll
                 for (int f = 0; f < NF; ++f) {
                     const T *sf = st + f * PW;
-                    T ab[VW], ym[VW], yp[VW], un[VW];
-                    lds<T, VW>(top ? hz1 + f * hwz + c : stn + f * PW + c, ab);
-                    lds<T, VW>((fc & 4) ? hy0 + f * hwy + zx + x : sf + c - m0, ym);
-                    lds<T, VW>((fc & 8) ? hy1 + f * hwy + zx + x : sf + c + m0, yp);
-                    T xl, xr;
-                    if constexpr (VW == 4) {
-                        // a row is GR <= 32 consecutive lanes of one warp: the
-                        // words beyond the group are the neighbouring lanes'
-                        const T lft = __shfl_up_sync(0xffffffffu, cur[f][q][VW - 1], 1);
-                        const T rgt = __shfl_down_sync(0xffffffffu, cur[f][q][0], 1);
-                        xl = (fc & 1) ? hx0[f * hwx + zy + y] : lft;
-                        xr = (fc & 2) ? hx1[f * hwx + zy + y] : rgt;
+                    const T cc = cur[f][q], below = prev[f][q];
+                    const T above = top ? hz1[f * hwz + c] : stn[f * PW + c];
+                    const T ym = (fc & 4) ? hy0[f * hwy + zx + x] : sf[c - m0];
+                    const T yp = (fc & 8) ? hy1[f * hwy + zx + x] : sf[c + m0];
+                    const T xm = (fc & 1) ? hx0[f * hwx + zy + y] : sf[c - 1];
+                    const T xp = (fc & 2) ? hx1[f * hwx + zy + y] : sf[c + 1];
+                    T un;
+                    if constexpr (ISO && !SYS) {
+                        const T sum = ((xp + xm) + (yp + ym)) + (above + below);
+                        const T dif = ((xp - xm) + (yp - ym)) + (above - below);
+                        un = cc + (cB[f][0] * (sum - (T)6 * cc) - cc * (cA0 * dif));
                     } else {
-                        xl = (fc & 1) ? hx0[f * hwx + zy + y] : sf[c - 1];
-                        xr = (fc & 2) ? hx1[f * hwx + zy + y] : sf[c + VW];
-                    }
-#pragma unroll
-                    for (int e = 0; e < VW; ++e) {
-                        const T cc = cur[f][q][e], below = prev[f][q][e], above = ab[e];
-                        const T xm = e == 0 ? xl : cur[f][q][e > 0 ? e - 1 : 0];
-                        const T xp = e == VW - 1 ? xr : cur[f][q][e + 1 < VW ? e + 1 : e];
-                        const T d2 = cB[f][0] * ((xp + xm) - (T)2 * cc) + cB[f][1] * ((yp[e] + ym[e]) - (T)2 * cc) +
+                        const T d2 = cB[f][0] * ((xp + xm) - (T)2 * cc) + cB[f][1] * ((yp + ym) - (T)2 * cc) +
                                      cB[f][2] * ((above + below) - (T)2 * cc);
                         if constexpr (SYS) {
-                            const T adv = cA0 * Uv[e] * (xp - xm) + cA1 * Vv[e] * (yp[e] - ym[e]) +
-                                          cA2 * Wv[e] * (above - below);
-                            un[e] = cc + (d2 - adv);
-                        } else if constexpr (ISO) {
-                            const T sum = ((xp + xm) + (yp[e] + ym[e])) + (above + below);
-                            const T dif = ((xp - xm) + (yp[e] - ym[e])) + (above - below);
-                            un[e] = cc + (cB[f][0] * (sum - (T)6 * cc) - cc * (cA0 * dif));
+                            const T adv = cA0 * Uv * (xp - xm) + cA1 * Vv * (yp - ym) + cA2 * Wv * (above - below);
+                            un = cc + (d2 - adv);
                         } else {
-                            const T d1 = cA0 * (xp - xm) + cA1 * (yp[e] - ym[e]) + cA2 * (above - below);
-                            un[e] = cc + (d2 - cc * d1);
+                            const T d1 = cA0 * (xp - xm) + cA1 * (yp - ym) + cA2 * (above - below);
+                            un = cc + (d2 - cc * d1);
                         }
                     }
-                    stv<T, VW>(up + f * field_words + coff[q], un);
+                    up[f * field_words + coff[q]] = un;
                     // boundary values of the new level into the ring
                     if (fc) {
-                        if (fc & 1) rf[0][f * fw + zy + y] = un[0];
-                        if (fc & 2) rf[1][f * fw + zy + y] = un[VW - 1];
-                        if (fc & 4) stv<T, VW>(rf[2] + f * fw + zx + x, un);
-                        if (fc & 8) stv<T, VW>(rf[3] + f * fw + zx + x, un);
+                        if (fc & 1) rf[0][f * fw + zy + y] = un;
+                        if (fc & 2) rf[1][f * fw + zy + y] = un;
+                        if (fc & 4) rf[2][f * fw + zx + x] = un;
+                        if (fc & 8) rf[3][f * fw + zx + x] = un;
                     }
-                    if (z == 0) stv<T, VW>(rf[4] + f * fw + c, un);
-                    if (top) stv<T, VW>(rf[5] + f * fw + c, un);
-#pragma unroll
-                    for (int e = 0; e < VW; ++e) {
-                        prev[f][q][e] = cur[f][q][e];
-                        cur[f][q][e] = ab[e];
-                    }
+                    if (z == 0) rf[4][f * fw + c] = un;
+                    if (top) rf[5][f * fw + c] = un;
+                    prev[f][q] = cc;
+                    cur[f][q] = above;
                 }
             }
             // the next read of a plane written here is a bulk copy (async

@@ -67,11 +67,6 @@ __host__ __device__ inline Smem3b smem3b_layout(int m0, int m1, long long face_w
     return l;
 }
 
-template <int V>
-struct IntC {
-    static constexpr int value = V;
-};
-
 // levels of the pass that starts at level lv (the launch ends at level lev_end)
 __host__ __device__ inline long long pass_len3(long long lv, long long lev_end, int sb)
 {
