@@ -1,4 +1,4 @@
-// at_adjoint.cu -- instantiations of the adjoint interval kernel (float and
+// at_adjoint.cu -- instantiations of the adjoint interval kernels (float and
 // double state, stencil order 2 and 4).
 #include "at_adjoint.cuh"
 
@@ -10,11 +10,27 @@ __attribute__((visibility("hidden"))) void *atk_adjoint_kernel(int w, int order)
     return order == 2 ? (void *)atk::at_adjoint_interval<float, 2> : (void *)atk::at_adjoint_interval<float, 4>;
 }
 
-// The one-subdomain-per-block variant (see atk::at_adjoint_own), FP32 order 2
-// (where its per-thread data fits the registers; the host picks it only there).
-__attribute__((visibility("hidden"))) void *atk_adjoint_own_kernel(int w, int order)
+namespace {
+template <typename T, int ORDER, bool FULL>
+void *warp_gw(int gw)
 {
-    (void)w;
-    (void)order;
-    return (void *)atk::at_adjoint_own<float, 2>;
+    return gw == 1 ? (void *)atk::at_adjoint_warp<T, ORDER, 1, FULL>
+                   : gw == 2 ? (void *)atk::at_adjoint_warp<T, ORDER, 2, FULL>
+                   : gw == 4 ? (void *)atk::at_adjoint_warp<T, ORDER, 4, FULL>
+                             : (void *)atk::at_adjoint_warp<T, ORDER, 8, FULL>;
+}
+
+template <typename T>
+void *warp_kernel(int order, int gw, bool full)
+{
+    if (order == 2) return full ? warp_gw<T, 2, true>(gw) : warp_gw<T, 2, false>(gw);
+    return full ? warp_gw<T, 4, true>(gw) : warp_gw<T, 4, false>(gw);
+}
+}  // namespace
+
+// The one-subdomain-per-warp kernel for gw groups of 4 points per lane, whole
+// runs (full) or not.
+__attribute__((visibility("hidden"))) void *atk_adjoint_warp_kernel(int w, int order, int gw, bool full)
+{
+    return w == 8 ? warp_kernel<double>(order, gw, full) : warp_kernel<float>(order, gw, full);
 }

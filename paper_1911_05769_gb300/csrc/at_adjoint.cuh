@@ -26,7 +26,7 @@
 // word offsets of the levels read are computed on the host.
 #pragma once
 
-#include "at_device.cuh"
+#include "at_kernels.cuh"
 
 namespace atk {
 
@@ -37,7 +37,7 @@ struct AdjParams {
     long long Dl;
     void *lam_a, *lam_b;       // lambda, N words each: lambda^{n_hi} in lam_a, then alternating
     void *pend;                // [Tp][P][2][R] words: adjoint of boundary values at older levels
-    double *dnu_part;          // [gridDim.x * gridDim.y] running FP64 sums of dJ/dnu
+    double *dnu_part;          // running FP64 sums of dJ/dnu, one per block (at_adjoint_warp: per subdomain)
     const int8_t *delays;      // delays of level n at delays[(n - k_level) * P * 2 + p * 2 + face]
     long long k_level;         // level of the delays' first row
     long long N, P, M;
@@ -47,7 +47,10 @@ struct AdjParams {
     long long n_hi, n_lo;      // this launch: lambda^{n_hi} -> lambda^{n_lo}, n_hi > n_lo
     unsigned long long *bar;   // grid-barrier arrivals, zero at the launch
     int *ctrl;                 // the solver's control block (status, abort word)
-    long long timeout_ns;      // bound of each grid-barrier wait
+    long long timeout_ns;      // bound of each wait
+    // one subdomain per warp (at_adjoint_warp; lambda in lam_a only)
+    unsigned char *msg;        // messages between neighbours [kAdjMsgSlots][P][2], zero at the first launch
+    int gpl, swz_shift, swz_mask, stage_bytes;   // tile layout, as the stepper's
 };
 
 template <int ORDER>
@@ -387,277 +390,406 @@ __global__ void __launch_bounds__(kAdjThreads, ORDER == 2 ? 7 : 3) at_adjoint_in
 }
 
 // ---------------------------------------------------------------------------
-// The interval kernel for one subdomain per block (M <= kAdjOwnChunk points,
-// every subdomain's block resident): a block keeps its own lambda in
-// registers from level to level, and loads everything a level needs that does
-// not depend on lambda -- the delays, its points' stencil values, the pending
-// words its face threads will add to -- before the grid barrier that ends the
-// previous level, so that after the barrier a level waits for one round trip
-// at most (the neighbours' boundary lambdas and values, the pending words
-// addressed to this level; edge threads only).  Same arithmetic, in the same
-// order, as at_adjoint_interval.
-constexpr int kAdjOwnThreads = 128;
-constexpr int kAdjOwnPts = 8;                               // points per thread, kAdjOwnThreads apart
-constexpr int kAdjOwnChunk = kAdjOwnThreads * kAdjOwnPts;
+// The interval kernel for one subdomain per warp (every subdomain's warp
+// resident).  A level of at_adjoint_interval is a chain of a grid barrier, a
+// block barrier and dependent global round trips (9.2 us a level of 2^20 points
+// in 1024 subdomains when a block keeps its lambda in registers and prefetches
+// what it can).  Here a warp keeps its subdomain's lambda in registers for the
+// whole interval, in the stepper's lane-major layout, and the only thing it
+// hears from its neighbours is one message per face and level:
+//   * the adjoint of its halo values at level n (src: R words, from lambda^{n+1}
+//     and u^n at its own edge points) goes out at the start of the level, as one
+//     16-byte access with the level's tag (see EntryTag in at_kernels.cuh);
+//   * a warp that receives the message of level n adds w_m(k) src to its own
+//     pending words of level n - k - m, k the neighbour's delay (prescribed, so
+//     known to both sides): the pending ring is private, in shared memory;
+//   * level n waits for the neighbours' messages of level n only where their
+//     delay is 0, else for those of level n + 1 (one level of slack).
+// The stored levels do not depend on lambda: the subdomain's tile comes in
+// through a swizzled stage two levels ahead, the words its halos are
+// extrapolated from one level ahead, the delays eight levels at a time.
+// Same terms as at_adjoint_interval; the pending words are added last.
+// 2^20 points in 1024 subdomains of 1024, FP32, order 2: 9.25 us a level then,
+// 2.2 us so (6.7 warps per SM, so a level's latency, not its 27 instructions a
+// point, sets the pace); forward and backward over 200 levels 3.32 and 1.88 ms.
 
-template <typename T, int ORDER>
-__global__ void __launch_bounds__(kAdjOwnThreads, 7) at_adjoint_own(const AdjParams a)
+// Shared memory of a warp: `stages` tiles, the halo levels, the pending words.
+__host__ __device__ inline long long adjoint_warp_smem(long long stage_bytes, int stages, int R, int word, int Tp)
+{
+    return stages * stage_bytes + round_up(kRawBytes, 128) + round_up(2LL * Tp * R * word, 128);
+}
+constexpr int kAdjStages = 3;
+constexpr int kAdjMsgSlots = 8;      // levels of messages kept (a neighbour is at most 2 levels away)
+
+template <typename T, int ORDER, int GW, bool FULL>
+__global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? 3 : 2) at_adjoint_warp(const AdjParams a)
 {
     constexpr int R = ORDER / 2;
     constexpr int S_LEV = ORDER / 2 + 1;
-    constexpr int NT = kAdjOwnThreads, PTS = kAdjOwnPts;
-    __shared__ T s_c[2 * R + 1][kAdjOwnChunk];
-    __shared__ T red[NT / 32];
-    __shared__ long long s_off[2][kAdjMaxLevels];
-    __shared__ int s_ok;
-    const int tid = threadIdx.x, lane = tid & 31;
-    const int M = (int)a.M, P = (int)a.P;
-    const int p = blockIdx.x;
-    const int pl = p == 0 ? P - 1 : p - 1, pr = p == P - 1 ? 0 : p + 1;
-    const T dtdx2 = sizeof(T) == 4 ? (T)a.dtdx2f : (T)a.dtdx2;
-    // the face threads: point 0 (face 0) and point M-1 (face 1)
-    const bool own_f0 = tid == 0, own_f1 = tid == (M - 1) % NT;
-    const int kp_f1 = (M - 1) / NT;
+    constexpr unsigned kAll = 0xffffffffu;
+    constexpr int NH = entry_halves<T, ORDER, 0>();
+    constexpr int kEnt = kRingHalf * NH;
+    constexpr int CPG = (int)sizeof(T) / 4, WPC = 16 / (int)sizeof(T), NPT = 4 * GW, NCH = GW * CPG;
+    extern __shared__ __align__(128) unsigned char smem[];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int my_face = lane >> 4, my_m = lane & 15;
+    const int P = (int)a.P, M = (int)a.M;
+    const long long e = (long long)blockIdx.x * kWarps + w, E = (long long)gridDim.x * kWarps;
+    const int p = (int)(e * P / E);
+    if ((e + 1) * P / E == p) return;                    // (no subdomain)
+    const int nb = my_face ? (p == P - 1 ? 0 : p + 1) : (p == 0 ? P - 1 : p - 1);   // across this lane's face
+    unsigned char *base = smem + (size_t)w * adjoint_warp_smem(a.stage_bytes, kAdjStages, R, (int)sizeof(T), a.Tp);
+    unsigned char *raw = base + kAdjStages * a.stage_bytes;
+    T *pend = reinterpret_cast<T *>(raw + round_up(kRawBytes, 128));              // [Tp][2][R]
+    const int gpl = FULL ? GW : a.gpl;
+    const int NG = M / 4, lane_last = (NG - 1) / gpl, m_last = FULL ? GW - 1 : (NG - 1) - lane_last * gpl;
+    const bool is_first = lane == 0, is_last = lane == lane_last;
+    const Swizzle swz = FULL ? Swizzle::of(NCH) : Swizzle{a.swz_shift, a.swz_mask};
+    auto own_chunk = [&](int k) -> int { return FULL ? lane_chunk<NCH>(lane, k) : 16 * swz(gpl * CPG * lane + k); };
+    const T cA = sizeof(T) == 4 ? (T)a.cAf : (T)a.cA, cB = sizeof(T) == 4 ? (T)a.cBf : (T)a.cB;
+    const T *lev = reinterpret_cast<const T *>(a.levels);
+    const int Dl = (int)a.Dl;
+    const int n_lev = (int)(a.n_hi - a.n_lo);
+    const unsigned pmask = (unsigned)a.Tp - 1u;
 
-    auto set_off = [&](long long n, int b) {
-        if (tid < kAdjMaxLevels) s_off[b][tid] = (n - tid >= 0) ? ((n - tid) % a.Dl) * a.N : 0;
-    };
-    // extrapolation weights of a face with delay k
-    auto weights = [&](int k, T *w) {
-        if constexpr (S_LEV == 2) {
-            w[0] = (T)(k + 1);
-            w[1] = (T)(-k);
-        } else {
-            w[0] = (T)((k + 1) * (k + 2) / 2);
-            w[1] = (T)(-k * (k + 2));
-            w[2] = (T)(k * (k + 1) / 2);
-        }
-    };
-
-    // what a level needs that does not depend on lambda
-    T v[PTS][2 * R + 1];          // stencil values of this thread's points
-    int k0 = 0, k1 = 0, kl1 = 0, kr0 = 0;
-    T pold[2][S_LEV][R];          // face threads: current pending words of the levels they add to
-    // (lanes 0..3: the raw delays of level n: this subdomain's faces 0, 1,
-    // the left neighbour's face 1, the right neighbour's face 0 -- loaded a
-    // level ahead, so that the prefetch below does not wait for them)
-    auto load_delays = [&](long long n) -> int {
-        const AdjStep<T, ORDER> A(a, n, s_off[0], nullptr);
-        return lane < 4 ? A.delay(lane < 2 ? p : (lane == 2 ? pl : pr), lane < 2 ? lane : (lane == 2 ? 1 : 0)) : 0;
-    };
-    auto prefetch = [&](long long n, int b, int kk) {
-        const AdjStep<T, ORDER> A(a, n, s_off[b], nullptr);
-        k0 = __shfl_sync(0xffffffffu, kk, 0);
-        k1 = __shfl_sync(0xffffffffu, kk, 1);
-        kl1 = __shfl_sync(0xffffffffu, kk, 2);
-        kr0 = __shfl_sync(0xffffffffu, kk, 3);
-#pragma unroll
-        for (int kp = 0; kp < PTS; ++kp) {
-            const int loc = tid + kp * NT;
-            if (loc < M) A.values(p, loc, k0, k1, v[kp]);
-        }
-#pragma unroll
-        for (int f = 0; f < 2; ++f) {
-            const bool mine = f == 0 ? own_f0 : own_f1;
-            const int k = f == 0 ? k0 : k1;
-            const int q = f == 0 ? pl : pr;
-            T w[S_LEV];
-            weights(k, w);
-#pragma unroll
-            for (int m = 0; m < S_LEV; ++m)
-#pragma unroll
-                for (int r = 0; r < R; ++r)
-                    pold[f][m][r] = (mine && k + m != 0 && w[m] != (T)0) ? *A.pend(n - k - m, q, f == 0 ? 1 : 0, r)
-                                                                         : (T)0;
-        }
-    };
-
-    // lambda^{n_hi} of this block's points
-    T lamr[PTS];
-    {
-        const T *l0 = reinterpret_cast<const T *>(a.lam_a);
-#pragma unroll
-        for (int kp = 0; kp < PTS; ++kp) {
-            const int loc = tid + kp * NT;
-            lamr[kp] = loc < M ? l0[(size_t)p * M + loc] : (T)0;
-        }
+    // the pending words of this subdomain
+    T *pend_g = reinterpret_cast<T *>(a.pend);
+    for (int i = lane; i < 2 * a.Tp * R; i += 32) {
+        const int t = i / (2 * R), r = i - t * 2 * R;
+        pend[i] = pend_g[((size_t)t * P + p) * 2 * R + r];
     }
-    set_off(a.n_hi - 1, 0);
-    __syncthreads();
-    prefetch(a.n_hi - 1, 0, load_delays(a.n_hi - 1));
-    unsigned long long arrivals = 0;
-    for (long long n = a.n_hi - 1, it = 0; n >= a.n_lo; --n, ++it) {
-        const int b = (int)(it & 1);
-        // the next level's delays and level offsets, early
-        int kk_next = 0;
-        if (n > a.n_lo) {
-            kk_next = load_delays(n - 1);
-            set_off(n - 1, b ^ 1);
-        }
-        const T *lam_in = reinterpret_cast<const T *>((it & 1) ? a.lam_b : a.lam_a);
-        T *lam_out = reinterpret_cast<T *>((it & 1) ? a.lam_a : a.lam_b);
-        const AdjStep<T, ORDER> A(a, n, s_off[b], lam_in);
-        // the pending words addressed to this level (written by the
-        // neighbours' face threads at later levels), loaded before any store
-        // of the level: a thread holds at most one point within R of each face
-        // The neighbours' readers across the faces (their lambda^{n+1} and
-        // level-n values: an undelayed read lands on level n) likewise.
-        T pwL = (T)0, pwR = (T)0, eL = (T)0, eR = (T)0;
-        if (tid < R && tid < M) {
-            pwL = *A.pend(n, p, 0, tid);
-            if (kl1 == 0) {
+    // lambda^{n_hi}
+    T lam[NPT];
+    T *lg = reinterpret_cast<T *>(a.lam_a) + (size_t)p * M;
 #pragma unroll
-                for (int d = -R; d < 0; ++d) {
-                    const int rl = tid + d;
-                    if (rl >= 0) continue;
-                    T vv[2 * R + 1];
-                    A.values(pl, M + rl, -1, kl1, vv);
-                    eL += A.gbar(pl * M + M + rl, -d, vv);
+    for (int m = 0; m < GW; ++m) {
+        const int g = gpl * lane + m;
+        const bool live = m < gpl && g < NG;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) lam[4 * m + q] = live ? lg[4 * g + q] : (T)0;
+    }
+    // slot of level l of the stored levels, l = n_hi - 1 - i
+    const int slot_hi = (int)((a.n_hi - 1) % a.Dl);
+    auto level_slot = [&](int back) -> int {            // back: levels below n_hi - 1
+        int s = slot_hi - back % Dl;
+        return s < 0 ? s + Dl : s;
+    };
+    // --- the tile of level n_hi - 1 - i into its stage
+    const int nc = (int)((size_t)M * sizeof(T) / 16);
+    auto load_tile = [&](int i) {
+        if (i < n_lev) {
+            unsigned char *dst = base + (i % kAdjStages) * a.stage_bytes;
+            const unsigned char *src =
+                reinterpret_cast<const unsigned char *>(lev + (size_t)level_slot(i) * a.N + (size_t)p * M) + 16 * lane;
+#pragma unroll
+            for (int t = 0; t < NCH; ++t)
+                if (lane + 32 * t < nc) cp_async16(dst + swz.coalesced(lane, t), src + 512 * t);
+        }
+        cp_async_commit();
+    };
+    // --- delays: lane 4 i + b holds byte b of level n_hi - 1 - (t0 + i): the left
+    // neighbour's face 1, this subdomain's faces 0 and 1, the right neighbour's face 0
+    auto load_delays = [&](int t0) -> int {
+        const long long i = t0 + (lane >> 2);
+        if (i >= n_lev) return 0;
+        const int b = lane & 3;
+        const long long at = b == 0 ? (p == 0 ? 2LL * P - 1 : 2LL * p - 1)
+                                    : b == 3 ? (p == P - 1 ? 0 : 2LL * p + 2) : 2LL * p + b - 1;
+        const long long n = a.n_hi - 1 - i;
+        int k = a.delays[(n - a.k_level) * 2 * P + at];
+        // (clamped as the forward run clamps it)
+        long long kmax = n - S_LEV + 1;
+        kmax = kmax < 0 ? 0 : kmax > a.L ? a.L : kmax;
+        return k > kmax ? (int)kmax : k < 0 ? 0 : k;
+    };
+    int kb = load_delays(0), kb_next = load_delays(8);
+    auto delay = [&](int i, int b) -> int {               // of level n_hi - 1 - i, in the current batch
+        return __shfl_sync(kAll, kb, 4 * (i & 7) + b);
+    };
+    // --- the words this face's halo of level i is extrapolated from: lane m < s
+    // reads level n - k - m
+    T hw[R];
+    auto load_halo = [&](int i, int k) {
+        if (my_m < S_LEV && (my_m == 0 || k != 0)) {
+            const T *src = lev + (size_t)level_slot(i + k + my_m) * a.N + (size_t)nb * M + (my_face ? 0 : M - R);
+#pragma unroll
+            for (int q = 0; q < R; ++q) hw[q] = ld_cg(src + q);
+        }
+    };
+    // --- messages: the neighbour's facing one of level i
+    const unsigned char *msg_in = a.msg + ((size_t)nb * 2 + (1 - my_face)) * kEnt;
+    unsigned char *msg_out = a.msg + (size_t)p * 2 * kEnt;
+    const size_t msg_stride = (size_t)P * 2 * kEnt;
+    unsigned long long md[NH], mt[NH];
+    auto msg_tag = [&](int i) { return entry_tag(a.n_hi - 1 - i); };
+    auto read_msg = [&](bool on, int i) {
+        ld_tagged<NH>(on, msg_in + (size_t)((unsigned)(a.n_hi - 1 - i) & (kAdjMsgSlots - 1)) * msg_stride, md, mt);
+    };
+    auto msg_there = [&](int i) -> bool {
+        bool ok = true;
+#pragma unroll
+        for (int h = 0; h < NH; ++h) ok = ok && mt[h] == msg_tag(i);
+        return ok;
+    };
+    // adds the message of level i (this face's neighbour had delay k there) to
+    // the pending words: lane m < s the level n - k - m
+    auto apply_msg = [&](bool on, int i, int k) {
+        if (on && my_m < S_LEV) {
+            T wt;
+            if constexpr (S_LEV == 2) wt = my_m == 0 ? (T)(k + 1) : (T)(-k);
+            else wt = my_m == 0 ? (T)((k + 1) * (k + 2) / 2) : my_m == 1 ? (T)(-k * (k + 2)) : (T)(k * (k + 1) / 2);
+            if (wt != (T)0) {
+                T *d = pend + ((size_t)((unsigned)(a.n_hi - 1 - i - k - my_m) & pmask) * 2 + my_face) * R;
+                T s[R];
+                if constexpr (sizeof(T) == 8) {
+#pragma unroll
+                    for (int q = 0; q < R; ++q) s[q] = (T)__longlong_as_double((long long)md[q < NH ? q : 0]);
+                } else {
+#pragma unroll
+                    for (int q = 0; q < R; ++q) s[q] = (T)__uint_as_float((unsigned)(md[0] >> (32 * q)));
                 }
+#pragma unroll
+                for (int q = 0; q < R; ++q) d[q] += wt * s[q];
             }
         }
-        {
-            const int locR = tid + NT * ((M - 1 - tid) / NT);   // this thread's last point
-            if (tid <= M - 1 && locR >= M - R && locR >= R) {
-                pwR = *A.pend(n, p, 1, locR - (M - R));
-                if (kr0 == 0) {
-#pragma unroll
-                    for (int d = 1; d <= R; ++d) {
-                        const int rl = locR + d;
-                        if (rl < M) continue;
-                        T vv[2 * R + 1];
-                        A.values(pr, rl - M, kr0, -1, vv);
-                        eR += A.gbar(pr * M + (rl - M), -d, vv);
-                    }
-                }
-            }
-        }
-        // terms c_j = lambda^{n+1}_r d u^{n+1}_r / d v_j of this block's points
-        T nu_acc = (T)0;
-#pragma unroll
-        for (int kp = 0; kp < PTS; ++kp) {
-            const int loc = tid + kp * NT;
-            if (loc >= M) continue;
-            T av = (T)0, bv = (T)0;
-#pragma unroll
-            for (int q = -R; q <= R; ++q) {
-                av += (T)Coeffs<ORDER>::alpha(q) * v[kp][q + R];
-                bv += (T)Coeffs<ORDER>::beta(q) * v[kp][q + R];
-            }
-            const T g = lamr[kp];
-#pragma unroll
-            for (int j = -R; j <= R; ++j) {
-                T d = A.cB * (T)Coeffs<ORDER>::beta(j) - A.cA * v[kp][R] * (T)Coeffs<ORDER>::alpha(j);
-                if (j == 0) d += (T)1 - A.cA * av;
-                s_c[j + R][loc] = g * d;
-            }
-            nu_acc += g * bv;
-        }
-        __syncthreads();
-        // gather lambda^n_i; the neighbours' readers across the faces from
-        // their lambda^{n+1} and values (edge threads)
-#pragma unroll
-        for (int kp = 0; kp < PTS; ++kp) {
-            const int loc = tid + kp * NT;
-            if (loc >= M) continue;
-            const int i = p * M + loc;
-            T acc = (T)0;
-#pragma unroll
-            for (int d = -R; d <= R; ++d) {
-                const int rl = loc + d;
-                if (rl >= 0 && rl < M) acc += s_c[-d + R][rl];
-            }
-            // (the readers across the faces and the pending words, loaded
-            // above; the words are then cleared)
-            if (loc < R) acc += eL;
-            if (loc >= M - R && loc >= R) acc += eR;
-            if (loc < R) {
-                acc += pwL;
-                *A.pend(n, p, 0, loc) = (T)0;
-            } else if (loc >= M - R) {
-                acc += pwR;
-                *A.pend(n, p, 1, loc - (M - R)) = (T)0;
-            }
-            lam_out[i] = acc;
-            lamr[kp] = acc;
-        }
-        // this block's delayed reads across its faces, added to the
-        // neighbours' boundary words at older levels (the face threads)
-#pragma unroll
-        for (int f = 0; f < 2; ++f) {
-            if (!(f == 0 ? own_f0 : own_f1)) continue;
-            const int k = f == 0 ? k0 : k1;
-            const int q = f == 0 ? pl : pr;
-            const int off = f == 0 ? 0 : M - 1;
-            T w[S_LEV];
-            weights(k, w);
-            T src[R];
-#pragma unroll
-            for (int r = 0; r < R; ++r) src[r] = (T)0;
-#pragma unroll
-            for (int t = 0; t < R; ++t) {
-                const int rt = f == 0 ? off + t : off - t;
-#pragma unroll
-                for (int j = -R; j <= R; ++j) {
-                    const bool crosses = f == 0 ? (j <= -t - 1) : (j >= t + 1);
-                    if (!crosses) continue;
-                    src[f == 0 ? R + t + j : j - t - 1] += s_c[j + R][rt];
-                }
-            }
-#pragma unroll
-            for (int m = 0; m < S_LEV; ++m) {
-                if (k + m == 0 || w[m] == (T)0) continue;     // level n: gathered above
-#pragma unroll
-                for (int r = 0; r < R; ++r) *A.pend(n - k - m, q, f == 0 ? 1 : 0, r) = pold[f][m][r] + w[m] * src[r];
-            }
-        }
-        (void)kp_f1;
-        // dJ/dnu: warp sums in the state's precision; thread 0 adds the
-        // block's FP64 sum after the next block barrier
-        for (int o = 16; o > 0; o >>= 1) nu_acc += __shfl_xor_sync(0xffffffffu, nu_acc, o);
-        if (lane == 0) red[tid >> 5] = nu_acc;
-        // the next level's lambda-free data (its loads land during the barrier)
-        if (n > a.n_lo) prefetch(n - 1, b ^ 1, kk_next);
-        __syncthreads();
-        bool go = n > a.n_lo;
-        if (tid == 0) {
-            double sum = 0.0;
-            for (int w = 0; w < NT / 32; ++w) sum += (double)red[w] * (double)dtdx2;
-            atomicAdd(a.dnu_part + blockIdx.x, sum);
-            if (go) {
-                // grid barrier (bounded), as adjoint_grid_sync after its block barrier
-                arrivals += gridDim.x;
-                __threadfence();
-                atomicAdd(a.bar, 1ull);
-                bool ok = true;
-                if (ld_acquire(a.bar) < arrivals) {
-                    const unsigned long long t0 = global_ns();
-                    for (;;) {
-                        __nanosleep(32);
-                        if (ld_acquire(a.bar) >= arrivals) break;
-                        if (ld_relaxed(a.ctrl + kCtrlAbort)) { ok = false; break; }
-                        if ((long long)(global_ns() - t0) > a.timeout_ns) {
+        __syncwarp();
+    };
+    // Receives the message of level i where `want` (bounded wait); returns
+    // false on abort.  (md, mt: a read of it, perhaps too early)
+    auto receive = [&](bool want, int i, int k) -> bool {
+        if (!__all_sync(kAll, !want || msg_there(i))) {
+            const unsigned long long t0 = global_ns();
+            for (int polls = 0;; ++polls) {
+                const bool miss = want && !msg_there(i);
+                if (miss) read_msg(true, i);
+                if (__all_sync(kAll, !want || msg_there(i))) break;
+                if ((polls & 15) == 15) {
+                    const bool late = (long long)(global_ns() - t0) > a.timeout_ns;
+                    if (__any_sync(kAll, late || ld_relaxed(a.ctrl + kCtrlAbort) != 0)) {
+                        if (late && miss && my_m == 0) {
                             if (atomicCAS(a.ctrl + kCtrlStatus, 0, kStatusTimeout) == 0) {
                                 a.ctrl[kCtrlCta] = (int)blockIdx.x;
                                 a.ctrl[kCtrlWhere] = kWhereAdjoint;
-                                a.ctrl[kCtrlNb] = -1;
-                                a.ctrl[kCtrlStep] = (int)n;
+                                a.ctrl[kCtrlNb] = nb;
+                                a.ctrl[kCtrlStep] = (int)(a.n_hi - 1 - i);
                             }
                             atomicExch(a.ctrl + kCtrlAbort, 1);
-                            ok = false;
-                            break;
                         }
+                        return false;
                     }
+                    if (polls > 64) __nanosleep(64);
                 }
-                __threadfence();
-                s_ok = ok ? 1 : 0;
             }
         }
-        if (go) {
-            __syncthreads();
-            if (!s_ok) return;
+        apply_msg(want, i, k);
+        return true;
+    };
+
+    load_tile(0);
+    load_tile(1);
+    load_halo(0, delay(0, 1 + my_face));
+    double nu_sum = 0.0;
+    bool late_msg = false;              // this face's message of the level before is still to come
+    int k_late = 0;                     // the neighbour's delay there
+    bool ok = true;
+    for (int i = 0; i < n_lev; ++i) {
+        const long long n = a.n_hi - 1 - i;
+        if (i > 0 && (i & 7) == 0) {
+            kb = kb_next;
+            kb_next = load_delays(i + 8);
+        }
+        const int k_own = delay(i, 1 + my_face);         // of this face
+        const int k_nb = delay(i, my_face ? 3 : 0);      // of the neighbour's facing face
+        // --- u^n: tile and halos
+        load_tile(i + 2);
+        if (my_m < S_LEV) {
+            T *r = reinterpret_cast<T *>(raw + my_face * kRawFace + my_m * kRawEntry);
+#pragma unroll
+            for (int q = 0; q < R; ++q) r[q] = hw[q];
+        }
+        cp_async_wait(2);
+        __syncwarp();
+        T hv = (T)0;
+        if (my_m < R) hv = approx_halo<T, S_LEV>(raw + my_face * kRawFace, k_own, my_m);
+        const unsigned char *stage = base + (i % kAdjStages) * a.stage_bytes;
+        T u[NPT];
+#pragma unroll
+        for (int m = 0; m < GW; ++m) {
+            // (FULL: the stage has room for the lanes beyond the tile)
+            const bool has = FULL || (m < gpl && gpl * lane + m < NG);
+#pragma unroll
+            for (int h = 0; h < CPG; ++h) {
+                T *d = u + 4 * m + h * WPC;
+                if (has) lds<T, WPC>(reinterpret_cast<const T *>(stage + own_chunk(m * CPG + h)), d);
+                else
+#pragma unroll
+                    for (int q = 0; q < WPC; ++q) d[q] = (T)0;
+            }
+        }
+        // --- the words of u and lambda at the run's edges
+        T tu[R], tl[R];                                  // last words of the lane's run
+        T eu[R], el[R];                                  // last words of the tile (its owner's)
+#pragma unroll
+        for (int q = 0; q < R; ++q) {
+            tu[q] = eu[q] = u[NPT - R + q];
+            tl[q] = el[q] = lam[NPT - R + q];
+            if constexpr (!FULL) {
+#pragma unroll
+                for (int m = 0; m < GW; ++m) {
+                    if (m == gpl - 1) { tu[q] = u[4 * m + 4 - R + q]; tl[q] = lam[4 * m + 4 - R + q]; }
+                    if (m == m_last) { eu[q] = u[4 * m + 4 - R + q]; el[q] = lam[4 * m + 4 - R + q]; }
+                }
+            }
+        }
+        // --- the adjoint of this subdomain's halo values at level n, out to the
+        // neighbours: c_j = lambda (cB beta_j - cA u alpha_j) of the points next
+        // to each face
+        {
+            T s0[R], s1[R];
+            auto c = [&](T l, T uu, int j) -> T {
+                return l * (cB * (T)Coeffs<ORDER>::beta(j) - cA * uu * (T)Coeffs<ORDER>::alpha(j));
+            };
+            if constexpr (R == 1) {
+                s0[0] = c(lam[0], u[0], -1);
+                s1[0] = c(el[0], eu[0], 1);
+            } else {
+                s0[0] = c(lam[0], u[0], -2);
+                s0[R - 1] = c(lam[0], u[0], -1) + c(lam[1], u[1], -2);
+                s1[0] = c(el[R - 1], eu[R - 1], 1) + c(el[0], eu[0], 2);
+                s1[R - 1] = c(el[R - 1], eu[R - 1], 2);
+            }
+            unsigned char *o = msg_out + (size_t)((unsigned)n & (kAdjMsgSlots - 1)) * msg_stride;
+            st_entry<T, ORDER, 0>(is_first, o, s0, s0, msg_tag(i));
+            st_entry<T, ORDER, 0>(is_last, o + kEnt, s1, s1, msg_tag(i));
+        }
+        // --- the message of the level before, where the neighbour's delay let
+        // it come later; a first read of this level's
+        if (__any_sync(kAll, late_msg)) {
+            read_msg(late_msg, i - 1);
+            if (!receive(late_msg, i - 1, k_late)) { ok = false; break; }
+        }
+        read_msg(true, i);
+        if (i + 1 < n_lev) {
+            const int kx = __shfl_sync(kAll, ((i + 1) & 7) == 0 ? kb_next : kb, 4 * ((i + 1) & 7) + 1 + my_face);
+            load_halo(i + 1, kx);
+        }
+        // --- lambda^n inside the subdomain
+        T ul[R], ur[R], ll[R], lr[R], hr[R];
+#pragma unroll
+        for (int q = 0; q < R; ++q) {
+            const T h = __shfl_sync(kAll, hv, (is_first ? 0 : 16) + q);   // lane 0: left halo; others: right halo
+            hr[q] = __shfl_sync(kAll, hv, 16 + q);
+            ul[q] = __shfl_up_sync(kAll, tu[q], 1);
+            ur[q] = __shfl_down_sync(kAll, u[q], 1);
+            ll[q] = __shfl_up_sync(kAll, tl[q], 1);
+            lr[q] = __shfl_down_sync(kAll, lam[q], 1);
+            ul[q] = is_first ? h : ul[q];
+            ll[q] = is_first ? (T)0 : ll[q];
+            if constexpr (FULL) {
+                ur[q] = is_last ? hr[q] : ur[q];
+                lr[q] = is_last ? (T)0 : lr[q];
+            }
+        }
+        T nu_acc = (T)0;
+#pragma unroll
+        for (int m = 0; m < GW; ++m) {
+            if (!FULL && m >= gpl) break;
+            // u and lambda^{n+1} of the group and R points on either side
+            T U[4 + 2 * R], G[4 + 2 * R];
+#pragma unroll
+            for (int q = 0; q < R; ++q) {
+                U[q] = ul[q];
+                G[q] = ll[q];
+                U[R + 4 + q] = m + 1 < GW ? u[4 * (m + 1 < GW ? m + 1 : m) + q] : ur[q];
+                G[R + 4 + q] = m + 1 < GW ? lam[4 * (m + 1 < GW ? m + 1 : m) + q] : lr[q];
+                if constexpr (!FULL) {
+                    if (m >= m_last) {
+                        if (m == gpl - 1) { U[R + 4 + q] = ur[q]; G[R + 4 + q] = lr[q]; }
+                        if (m == m_last && is_last) { U[R + 4 + q] = hr[q]; G[R + 4 + q] = (T)0; }
+                    }
+                }
+                ul[q] = u[4 * m + 4 - R + q];
+                ll[q] = lam[4 * m + 4 - R + q];
+            }
+#pragma unroll
+            for (int q = 0; q < 4; ++q) { U[R + q] = u[4 * m + q]; G[R + q] = lam[4 * m + q]; }
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                T av = (T)0, bv = (T)0;
+#pragma unroll
+                for (int j = -R; j <= R; ++j) {
+                    if (j != 0) av += (T)Coeffs<ORDER>::alpha(j) * U[R + q + j];
+                    bv += (T)Coeffs<ORDER>::beta(j) * U[R + q + j];
+                }
+                T acc = (T)0;
+#pragma unroll
+                for (int d = -R; d <= R; ++d) {          // reader q + d, whose value j = -d this point is
+                    const int x = R + q + d;
+                    T t = cB * (T)Coeffs<ORDER>::beta(-d);
+                    if (d != 0) t -= cA * U[x] * (T)Coeffs<ORDER>::alpha(-d);
+                    else t += (T)1 - cA * av;
+                    acc += G[x] * t;
+                }
+                // (points beyond the tile stay 0)
+                const bool live = FULL || gpl * lane + m < NG;
+                if constexpr (!FULL) acc = live ? acc : (T)0;
+                nu_acc += live ? G[R + q] * bv : (T)0;
+                lam[4 * m + q] = acc;
+            }
+        }
+        nu_sum += lane <= lane_last ? (double)nu_acc : 0.0;
+        // --- this level's messages: where the neighbour's delay is 0, and
+        // where they are there already; then the pending words of level n
+        {
+            const bool here = msg_there(i);
+            const bool now = k_nb == 0 || here;
+            const unsigned bal = __ballot_sync(kAll, now);
+            // (one decision per face)
+            const bool want = ((bal >> (lane & 16)) & 0xffffu) == 0xffffu || k_nb == 0;
+            if (!receive(want, i, k_nb)) { ok = false; break; }
+            late_msg = !want;
+            k_late = k_nb;
+        }
+        {
+            T *pw = pend + (size_t)((unsigned)n & pmask) * 2 * R;
+            T p0[R], p1[R];
+#pragma unroll
+            for (int q = 0; q < R; ++q) { p0[q] = pw[q]; p1[q] = pw[R + q]; }
+            __syncwarp();
+            if (lane < 2 * R) pw[lane] = (T)0;
+            __syncwarp();
+#pragma unroll
+            for (int q = 0; q < R; ++q) {
+                if (is_first) lam[q] += p0[q];
+#pragma unroll
+                for (int m = 0; m < GW; ++m)
+                    if (FULL ? m == GW - 1 : m == m_last)
+                        if (is_last) lam[4 * m + 4 - R + q] += p1[q];
+            }
         }
     }
+    // the last level's messages belong to the pending words of the levels below
+    if (ok && __any_sync(kAll, late_msg)) {
+        read_msg(late_msg, n_lev - 1);
+        receive(late_msg, n_lev - 1, k_late);
+    }
+    cp_async_wait(0);
+    __syncwarp();
+    if (!ok) return;
+#pragma unroll
+    for (int m = 0; m < GW; ++m) {
+        const int g = gpl * lane + m;
+        // (word by word: the caller's array may start at any word)
+        if (m < gpl && g < NG)
+#pragma unroll
+            for (int q = 0; q < 4; ++q) lg[4 * g + q] = lam[4 * m + q];
+    }
+    for (int i = lane; i < 2 * a.Tp * R; i += 32) {
+        const int t = i / (2 * R), r = i - t * 2 * R;
+        pend_g[((size_t)t * P + p) * 2 * R + r] = pend[i];
+    }
+    for (int o = 16; o > 0; o >>= 1) nu_sum += __shfl_xor_sync(kAll, nu_sum, o);
+    if (lane == 0) a.dnu_part[p] += nu_sum * a.dtdx2;
 }
 
 }  // namespace atk

@@ -40,7 +40,7 @@ void *atk_batch_kernel_f32c(int order, int gw, bool full);
 void *atk_restore_kernel_f32(int order);
 void *atk_restore_kernel_f64(int order);
 void *atk_adjoint_kernel(int w, int order);
-void *atk_adjoint_own_kernel(int w, int order);
+void *atk_adjoint_warp_kernel(int w, int order, int gw, bool full);
 void *atk_stepper3d_kernel(int w, int tc);
 void *atk_stepper3d_iso_kernel(int w, int tc);
 void *atk_system3d_kernel(int w, int tc, int nf);
@@ -1474,9 +1474,11 @@ int64_t n_segments(int64_t n_steps, int64_t interval) { return n_steps <= 0 ? 1 
 int adj_grid_x(const at_solver *h) { return (int)(h->P < 16LL * h->sm_count ? h->P : 16LL * h->sm_count); }
 int adj_grid_y(const at_solver *h) { return (int)((h->M + atk::kAdjChunk - 1) / atk::kAdjChunk); }
 int adj_blocks(const at_solver *h) { return adj_grid_x(h) * adj_grid_y(h); }
+// partial sums of dJ/dnu: one per block, or per subdomain
+int64_t adj_sums(const at_solver *h) { return h->P > adj_blocks(h) ? h->P : adj_blocks(h); }
 
 struct AdjLayout {
-    size_t levels, lam, pend, dnu, bar, kbuf, total;
+    size_t levels, lam, pend, dnu, msg, bar, kbuf, total;
 };
 
 AdjLayout adj_layout(const at_solver *h, int64_t interval)
@@ -1486,7 +1488,9 @@ AdjLayout adj_layout(const at_solver *h, int64_t interval)
     l.levels = off; off = align_up(off + (size_t)(interval + ckpt_levels(h)) * h->N * h->w, 256);
     l.lam = off;    off = align_up(off + (size_t)h->N * h->w, 256);
     l.pend = off;   off = align_up(off + (size_t)h->T * h->P * 2 * h->R * h->w, 256);
-    l.dnu = off;    off = align_up(off + (size_t)adj_blocks(h) * 8, 256);
+    l.dnu = off;    off = align_up(off + (size_t)adj_sums(h) * 8, 256);
+    l.msg = off;
+    off = align_up(off + (size_t)atk::kAdjMsgSlots * h->P * 2 * atk::kRingHalf * entry_halves(h->w, h->R, false), 256);
     l.bar = off;    off = align_up(off + 8, 256);
     l.kbuf = off;   off = align_up(off + (size_t)interval * h->P * 2, 256);
     l.total = off;
@@ -1570,8 +1574,8 @@ int at_adjoint(at_solver *h, int64_t n_steps, int delay_mode, const int8_t *dela
     const size_t lvl = (size_t)h->N * h->w, seg_bytes = (size_t)Dc * lvl;
     unsigned char *ws = static_cast<unsigned char *>(adj_ws);
     const unsigned char *ck = static_cast<const unsigned char *>(ckpt);
-    const int G = adj_blocks(h);
-    cudaError_t e = cudaMemsetAsync(ws + al.pend, 0, al.dnu - al.pend + (size_t)G * 8, h->stream);
+    const int64_t G = adj_sums(h);
+    cudaError_t e = cudaMemsetAsync(ws + al.pend, 0, al.kbuf - al.pend, h->stream);
     if (e != cudaSuccess) return cuda_fail(e, "cudaMemsetAsync(adjoint)");
 
     atk::AdjParams a{};
@@ -1594,23 +1598,33 @@ int at_adjoint(at_solver *h, int64_t n_steps, int delay_mode, const int8_t *dela
         a.dtdx2 = h->dt / (12.0 * h->dx * h->dx);
     }
     a.cAf = (float)a.cA; a.cBf = (float)a.cB; a.dtdx2f = (float)a.dtdx2;
-    // one cooperative launch per interval: every block resident.  With one
-    // block per subdomain (M <= 1024 points, every subdomain's block
-    // resident) the variant that keeps lambda in registers and loads the next
-    // level's lambda-free data before the grid barrier; else blocks walk the
-    // subdomains
-    void *kern = atk_adjoint_own_kernel(h->w, h->order);
-    int threads = atk::kAdjOwnThreads;
+    a.msg = ws + al.msg;
+    a.gpl = run_groups(h->M);
+    const atk::Swizzle swz = atk::Swizzle::of(a.gpl * h->w / 4);
+    a.swz_shift = swz.shift;
+    a.swz_mask = swz.mask;
+    // one cooperative launch per interval.  With a warp per subdomain resident
+    // (M of 1024 points, FP32: up to 1824 subdomains on 152 SMs; shorter ones,
+    // more) the kernel that keeps lambda in registers, on as many CTAs as fit
+    // or there are subdomains; else blocks walk the subdomains
+    const int gw = groups_per_lane(h->M);
+    const bool full = full_runs(h->M, gw);
+    a.stage_bytes = (int)atk::round_up(atk::tile_points(h->M, gw, full) * h->w, 128);
+    void *kern = atk_adjoint_warp_kernel(h->w, h->order, gw, full);
+    int threads = atk::kThreads;
+    size_t smem = (size_t)atk::kWarps * atk::adjoint_warp_smem(a.stage_bytes, atk::kAdjStages, h->R, h->w, h->T);
+    e = allow_smem(kern, h->smem_optin);
+    if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute(adjoint)");
     int occ = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, threads, 0);
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, threads, smem);
     if (e != cudaSuccess) return cuda_fail(e, "cudaOccupancyMaxActiveBlocksPerMultiprocessor(adjoint)");
-    int gy = 1, gx = (int)h->P;
-    // (FP32, order 2: the variant's per-thread data fits its registers there)
-    const bool own = h->w == 4 && h->order == 2 && h->M <= atk::kAdjOwnChunk &&
-                     h->P <= (int64_t)occ * h->sm_count && h->P <= adj_blocks(h);
+    const int64_t fit = (int64_t)occ * h->sm_count;
+    int gy = 1, gx = (int)(fit < h->P ? fit : h->P);
+    const bool own = fit * atk::kWarps >= h->P;
     if (!own) {
         kern = atk_adjoint_kernel(h->w, h->order);
         threads = atk::kAdjThreads;
+        smem = 0;
         e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, threads, 0);
         if (e != cudaSuccess) return cuda_fail(e, "cudaOccupancyMaxActiveBlocksPerMultiprocessor(adjoint)");
         gy = adj_grid_y(h);
@@ -1648,6 +1662,7 @@ int at_adjoint(at_solver *h, int64_t n_steps, int delay_mode, const int8_t *dela
         cudaLaunchConfig_t cfg{};
         cfg.gridDim = dim3(gx, gy);
         cfg.blockDim = dim3(threads);
+        cfg.dynamicSmemBytes = smem;
         cfg.stream = h->stream;
         cudaLaunchAttribute attr[1];
         attr[0].id = cudaLaunchAttributeCooperative;
@@ -1657,7 +1672,7 @@ int at_adjoint(at_solver *h, int64_t n_steps, int delay_mode, const int8_t *dela
         void *args[] = {&a};
         e = cudaLaunchKernelExC(&cfg, kern, args);
         if (e != cudaSuccess) return cuda_fail(e, "cooperative launch of at_adjoint_interval");
-        if ((end - c) & 1) { unsigned char *t = cur; cur = other; other = t; }
+        if (!own && ((end - c) & 1)) { unsigned char *t = cur; cur = other; other = t; }
     }
     if (cur != lam) {
         e = cudaMemcpyAsync(lam, cur, lvl, cudaMemcpyDeviceToDevice, h->stream);
@@ -1669,7 +1684,7 @@ int at_adjoint(at_solver *h, int64_t n_steps, int delay_mode, const int8_t *dela
     rc = read_status(h);
     if (rc != AT_OK) return rc;
     double sum = 0.0;
-    for (int b = 0; b < G; ++b) sum += part[(size_t)b];
+    for (int64_t b = 0; b < G; ++b) sum += part[(size_t)b];
     if (dnu) *dnu = sum;
     return AT_OK;
 }

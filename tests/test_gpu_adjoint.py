@@ -218,3 +218,33 @@ def test_adjoint_workload_fp32_against_fp64():
     err = float((g32 - g64).norm() / g64.norm())
     assert err <= 1e-2, err
     assert abs(n32 - n64) <= 1e-2 * abs(n64), (n32, n64)
+
+
+@pytest.mark.parametrize("order,M,P", [(2, 4, 7), (4, 4, 7), (2, 100, 5), (4, 256, 1), (4, 400, 2), (2, 500, 9),
+                                       (4, 768, 3), (2, 1024, 4), (4, 1020, 3)])
+@pytest.mark.parametrize("dtype", ["f64", "f32"])
+def test_adjoint_tile_sizes(order, M, P, dtype):
+    """Subdomains in one lane, in partly filled and full warps, runs with a short
+    last one; one and two subdomains (a subdomain its own neighbour on both
+    sides); intervals of one level, shorter than the delay bound and odd."""
+    from paper_1911_05769_gb300 import AT_SEEDED
+    pr = problem(N=P * M, P=P, order=order, L=3, steps=23, nu=0.02 if P * M > 400 else 0.2, seed=M)
+    pr["dt"] *= 0.5
+    if dtype == "f32":
+        pr["u0"] = pr["u0"].astype(np.float32).astype(np.float64)
+        pr["lam_T"] = pr["lam_T"].astype(np.float32).astype(np.float64)
+    for interval in (1, 3, 11, 40):
+        uT, lam0, dnu, _ = gpu_adjoint(pr, mode=AT_SEEDED, interval=interval, dtype=dtype)
+        ouT, olam0, odnu = oracle_adjoint(pr, mode=oracle.SEEDED)
+        assert rel_linf(uT, ouT) <= TOL[dtype]
+        assert rel_linf(lam0, olam0) <= TOL[dtype]
+
+
+def test_adjoint_more_subdomains_than_resident_warps():
+    """Subdomains beyond the warps that can be resident: blocks walk them."""
+    from paper_1911_05769_gb300 import AT_SEEDED
+    pr = problem(N=4 * 20000, P=20000, order=2, L=2, steps=12, nu=0.02)
+    uT, lam0, dnu, _ = gpu_adjoint(pr, mode=AT_SEEDED, interval=5)
+    ouT, olam0, odnu = oracle_adjoint(pr, mode=oracle.SEEDED)
+    assert rel_linf(uT, ouT) <= TOL["f64"]
+    assert rel_linf(lam0, olam0) <= TOL["f64"]
