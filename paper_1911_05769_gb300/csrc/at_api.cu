@@ -22,6 +22,7 @@
 #include "at_kernels.cuh"
 #include "at_kernels3d_blk.cuh"
 #include "at_kernels3d_v4.cuh"
+#include "at_resident.cuh"
 
 void *atk_stepper_kernel_f32(int order, int gw, bool forced, bool full);
 void *atk_stepper_kernel_f32v(int order, int gw, bool forced, bool full);
@@ -40,6 +41,7 @@ void *atk_batch_kernel_f32c(int order, int gw, bool full);
 void *atk_restore_kernel_f32(int order);
 void *atk_restore_kernel_f64(int order);
 void *atk_adjoint_kernel(int w, int order);
+void *atk_resident_kernel(int w, int order, int ppl, bool forced);
 void *atk_adjoint_warp_kernel(int w, int order, int gw, bool full);
 void *atk_stepper3d_kernel(int w, int tc);
 void *atk_stepper3d_iso_kernel(int w, int tc);
@@ -420,6 +422,7 @@ struct at_solver {
     void *kernel_bs;           // the blocked synchronous mode's kernel (NULL: none)
     void *kernel_b3;           // 3D: the blocked free-running kernel (NULL: none)
     int G_b3, stages_b3, smem_b3;   // 3D: its CTAs, plane stages and shared memory
+    void *kernel_res;          // 1D: the one-subdomain-per-CTA kernel of prescribed delays (NULL: none)
     bool bs_ok;                // it can run in the launch shape chosen for `kernel`
     void *init_kernel;
 };
@@ -432,10 +435,15 @@ namespace {
 // may partition the subdomains into PEs differently from the one before.)
 cudaError_t launch_stepper(at_solver *h, atk::Params *p, void *kernel)
 {
+    const bool res = h->kernel_res && p->sb == 1 && (p->mode == AT_SEEDED || p->mode == AT_REPLAY);
+    if (res) {
+        kernel = h->kernel_res;
+        p->G = (int)h->P;
+    }
     cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3(h->G);
-    cfg.blockDim = dim3(atk::kThreads);
-    cfg.dynamicSmemBytes = (size_t)h->smem;
+    cfg.gridDim = dim3(p->G);
+    cfg.blockDim = dim3(res ? atk::resident_threads(h->M) : atk::kThreads);
+    cfg.dynamicSmemBytes = (size_t)(res ? 0 : h->smem);
     cfg.stream = h->stream;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeCooperative;
@@ -444,6 +452,25 @@ cudaError_t launch_stepper(at_solver *h, atk::Params *p, void *kernel)
     cfg.numAttrs = 1;
     void *args[] = {p};
     return cudaLaunchKernelExC(&cfg, kernel, args);
+}
+
+// The resident kernel (one subdomain per CTA, prescribed delays) serves a single
+// domain in plain precision whose subdomains find a resident CTA each and which
+// sets no CTA count of its own.
+// N = 4096 FP64 in 16 subdomains: 1.34 us a step here, 2.9 in the general
+// kernel; N = 1024, order 4, forced, in 16: 1.5 and 3.0.
+cudaError_t prepare_resident(at_solver *h)
+{
+    h->kernel_res = nullptr;
+    if (h->batch || h->comp || h->v64 || h->g.max_ctas > 0 || (h->g.flags & AT_FLAG_TEST_SKIP_PUBLISH)) return cudaSuccess;
+    const int ppt = atk::resident_points(h->M), threads = atk::resident_threads(h->M);
+    if (h->P > (int64_t)32 * h->sm_count) return cudaSuccess;
+    void *kern = atk_resident_kernel(h->w, h->order, ppt, h->g.forcing_amp != 0.0);
+    int occ = 0;
+    const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, threads, 0);
+    if (e != cudaSuccess) return e;
+    if ((int64_t)occ * h->sm_count >= h->P) h->kernel_res = kern;
+    return cudaSuccess;
 }
 
 // The blocked synchronous kernel runs in the launch shape chosen for the
@@ -832,6 +859,8 @@ int at_create(const at_grid *grid, int64_t P, int scheme_order, int L, double nu
                            stages, grid->stages > 0, sms, smem_optin, h->kernel, &h->G, &h->stages, &h->sl, &h->smem, &h->smax);
     if (rc2 != AT_OK) { delete h; return rc2; }
     prepare_bs(h);
+    e = prepare_resident(h);
+    if (e != cudaSuccess) { delete h; return cuda_fail(e, "cudaOccupancyMaxActiveBlocksPerMultiprocessor"); }
     h->sb = sb;
     h->step = 0;
     h->has_state = false;
@@ -1790,6 +1819,8 @@ extern "C" int at_step_noalloc(const at_grid *grid, int64_t P, int scheme_order,
                       grid->stages > 0, sms, smem_optin, h.kernel, &h.G, &h.stages, &h.sl, &h.smem, &h.smax);
     if (rc != AT_OK) return rc;
     h.sb = 1;
+    e = prepare_resident(&h);
+    if (e != cudaSuccess) return cuda_fail(e, "cudaOccupancyMaxActiveBlocksPerMultiprocessor");
 
     // Every call starts from zeroed ring buffers, flags, status and counters:
     // the array still holds whatever the previous call left in it.

@@ -379,26 +379,23 @@ __device__ __forceinline__ T forcing_point(T fs, T fc, T sv, T cv)
 
 // The forward-Euler update u += dt (-u u_x + nu u_xx) + F of a run of points,
 // as u += cA (cr b - u a + F / cA): cA = dt/(2dx) | dt/(12dx), cA cr = nu
-// dt/dx^2 | nu dt/(12dx^2), a and b the stencil's first and second difference.
-// The factors 1, cr, cA each ride in a fused multiply-add, so the increment,
-// formed apart from u, takes 3 operations beside a and b (6 when cB b - cA u a
-// + F + u is taken term by term): 10 a point at order 4, forcing included, 6 at
-// order 2.
-//   FP32: a and b value by value, a = 8 (u_1 - u_-1) - (u_2 - u_-2), b = 16 (u_1
-// + u_-1) - (u_2 + u_-2) - 30 u.
-//   FP64: from the first differences d_i = u_{i+1} - u_i and second ones e_i =
-// d_i - d_{i-1}, formed once for the points that share them: a = 6 (d_i +
-// d_{i-1}) - (e_{i+1} - e_{i-1}), b = 14 e_i - (e_{i+1} + e_{i-1}); the same 10
-// operations, but differences of nearby values are exact.  (FP32 keeps the
-// values' form: there the last addition's rounding decides, and over runs of
-// hundreds of steps the sums' own rounding breaks up its bias: error against 64
-// bits 2.2e-6 against 2.9e-6 with the exact differences.)
-//   Compensated state: the differences word by word, hi and lo, and the factors
-// as cB b - cA u a, each rounded once.
+// dt/dx^2 | nu dt/(12dx^2), a and b the stencil's first and second difference,
+// a = 8 (u_1 - u_-1) - (u_2 - u_-2), b = 16 (u_1 + u_-1) - (u_2 + u_-2) - 30 u
+// at order 4.  The factors 1, cr, cA each ride in a fused multiply-add, so the
+// increment, formed apart from u, takes 3 operations beside a and b (6 when cB
+// b - cA u a + F + u is taken term by term): 10 a point at order 4, forcing
+// included, 6 at order 2.  (Forming a and b from differences shared between
+// points takes as many.  In FP32 it loses: there the last addition's rounding
+// decides, and over runs of hundreds of steps the sums' own rounding breaks up
+// its bias -- error against 64 bits 2.2e-6 against 2.9e-6 with exact differences.)
+//   Compensated state: the differences word by word, hi and lo, first
+// differences d_i = u_{i+1} - u_i and second ones e_i = d_i - d_{i-1} formed once
+// for the points that share them: a = 6 (d_i + d_{i-1}) - (e_{i+1} - e_{i-1}), b =
+// 14 e_i - (e_{i+1} + e_{i-1}); the factors as cB b - cA u a, each rounded once.
 //
-// Every operation of the first two is written as the one instruction it is, so
-// that a point computed twice -- by its owner in group(), by a neighbour as a
-// ghost cell in point() -- is computed the same way twice.
+// Every operation is written as the one instruction it is, so that a point
+// computed twice -- by its owner in group(), by a neighbour as a ghost cell in
+// point() -- is computed the same way twice.
 //
 // PLAIN: the order-2 update as cB b - cA u a, 7 operations.  The unforced FP32
 // single domain keeps it: its trajectories feed the FP32 gradient, which
@@ -407,7 +404,7 @@ __device__ __forceinline__ T forcing_point(T fs, T fc, T sv, T cv)
 template <typename T, int ORDER, int PREC, bool PLAIN>
 struct StencilK {
     static constexpr int R = ORDER / 2;
-    static constexpr bool WINDOW = PREC == 1 || (PREC == 0 && sizeof(T) == 4);   // from the values of a window
+    static constexpr bool WINDOW = PREC != 2;   // from the values of a window
     T cA, cr, cB;
     double cB64;
     // (cr_: cr; a compensated state: cB)
@@ -419,8 +416,8 @@ struct StencilK {
     // what a lane carries from point to point
     struct Carry {
         T w[2];                        // WINDOW: the R words left of the point
-        T d0, d1, e0, e1;              // else d_{i-1}, d_i (order 2: d0 = d_{i-1}); e_{i-1}, e_i
-        T l0, l1, g0;                  // compensated state: the differences of the lo words; d_{i-1} + its lo
+        T d0, d1, e0, e1;              // else d_{i-1}, d_i (order 2: d0 = d_{i-1}) of the hi words; e_{i-1}, e_i
+        T l0, l1, g0;                  // the differences of the lo words; d_{i-1} + its lo
     };
 
     // cr b - u a + F / cA
@@ -458,29 +455,14 @@ struct StencilK {
             const T a = w[2] - w[0], b = (w[2] + w[0]) - (T)2 * cc;
             const T du = cB * b - cA * cc * a;
             return cc + du;
-        } else if constexpr (WINDOW && ORDER == 2) {
+        } else if constexpr (ORDER == 2) {
             const T a = w[2] - w[0], b = fma((T)-2, cc, w[2] + w[0]);
             return fma(cA, increment(cc, a, b, F, FORCED), cc);
-        } else if constexpr (WINDOW) {
+        } else {
             const T a = fma((T)8, w[2 * R - 1] - w[1], -(w[2 * R] - w[0]));
             const T b = fma((T)-30, cc, fma((T)16, w[2 * R - 1] + w[1], -(w[2 * R] + w[0])));
             return fma(cA, increment(cc, a, b, F, FORCED), cc);
-        } else if constexpr (ORDER == 2) {
-            const T d0 = cc - w[0], d1 = w[2] - cc;
-            return fma(cA, increment(cc, d1 + d0, d1 - d0, F, FORCED), cc);
-        } else {
-            const T d0 = w[1] - w[0], d1 = cc - w[1], d2 = w[2 * R - 1] - cc, d3 = w[2 * R] - w[2 * R - 1];
-            T a, b;
-            from_differences(d2 - d1, d1 - d0, d3 - d2, d2 + d1, a, b);
-            return fma(cA, increment(cc, a, b, F, FORCED), cc);
         }
-    }
-
-    // order 4: a and b from e_i, e_{i-1}, e_{i+1} and s = d_i + d_{i-1}
-    static __device__ __forceinline__ void from_differences(T e, T ep, T en, T s, T &a, T &b)
-    {
-        a = fma((T)6, s, -(en - ep));
-        b = fma((T)14, e, -(en + ep));
     }
 
     // the carry before the first point of a lane's run: lw the R words left of
@@ -492,25 +474,17 @@ struct StencilK {
             for (int q = 0; q < R; ++q) y.w[q] = lw[q];
         } else if constexpr (ORDER == 2) {
             y.d0 = c[0] - lw[0];
-            if constexpr (PREC == 2) {
-                y.l0 = cl[0] - lwl[0];
-                y.g0 = y.d0 + y.l0;
-            }
+            y.l0 = cl[0] - lwl[0];
+            y.g0 = y.d0 + y.l0;
         } else {
-            const T dm = lw[R - 1] - lw[0];
+            const T dm = lw[R - 1] - lw[0], lm = lwl[R - 1] - lwl[0];
             y.d0 = c[0] - lw[R - 1];
             y.d1 = c[1] - c[0];
-            if constexpr (PREC == 2) {
-                const T lm = lwl[R - 1] - lwl[0];
-                y.l0 = cl[0] - lwl[R - 1];
-                y.l1 = cl[1] - cl[0];
-                y.e0 = (y.d0 - dm) + (y.l0 - lm);
-                y.e1 = (y.d1 - y.d0) + (y.l1 - y.l0);
-                y.g0 = y.d0 + y.l0;
-            } else {
-                y.e0 = y.d0 - dm;
-                y.e1 = y.d1 - y.d0;
-            }
+            y.l0 = cl[0] - lwl[R - 1];
+            y.l1 = cl[1] - cl[0];
+            y.e0 = (y.d0 - dm) + (y.l0 - lm);
+            y.e1 = (y.d1 - y.d0) + (y.l1 - y.l0);
+            y.g0 = y.d0 + y.l0;
         }
     }
 
@@ -532,62 +506,43 @@ struct StencilK {
 #pragma unroll
             for (int e = 0; e < 4; ++e) c[e] = point<FORCED>(v + e, FORCED ? F[FORCED ? e : 0] : (T)0);
         } else {
-            T v[4 + R], vl[PREC == 2 ? 4 + R : 1];
+            T v[4 + R], vl[4 + R];
 #pragma unroll
             for (int e = 0; e < 4 + R; ++e) {
                 v[e] = e < 4 ? c[e < 4 ? e : 0] : nx[e >= 4 ? e - 4 : 0];
-                if constexpr (PREC == 2) vl[e] = e < 4 ? cl[e < 4 ? e : 0] : nxl[e >= 4 ? e - 4 : 0];
+                vl[e] = e < 4 ? cl[e < 4 ? e : 0] : nxl[e >= 4 ? e - 4 : 0];
             }
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
-                const T f = FORCED ? F[FORCED ? e : 0] : (T)0;
                 const T cc = v[e];
                 T a, b;
                 if constexpr (ORDER == 2) {
-                    const T dn = v[e + 1] - cc;
-                    if constexpr (PREC == 2) {
-                        const T ln = vl[e + 1] - vl[e];
-                        const T gn = dn + ln;
-                        b = (dn - y.d0) + (ln - y.l0);
-                        a = gn + y.g0;
-                        y.l0 = ln;
-                        y.g0 = gn;
-                    } else {
-                        a = dn + y.d0;
-                        b = dn - y.d0;
-                    }
+                    const T dn = v[e + 1] - cc, ln = vl[e + 1] - vl[e];
+                    const T gn = dn + ln;
+                    b = (dn - y.d0) + (ln - y.l0);
+                    a = gn + y.g0;
+                    y.l0 = ln;
+                    y.g0 = gn;
                     y.d0 = dn;
                 } else {
-                    const T dn = v[e + 2] - v[e + 1];
-                    T en, s;
-                    if constexpr (PREC == 2) {
-                        const T ln = vl[e + 2] - vl[e + 1];
-                        const T gn = y.d1 + y.l1;
-                        en = (dn - y.d1) + (ln - y.l1);
-                        s = gn + y.g0;
-                        y.l1 = ln;
-                        y.g0 = gn;
-                    } else {
-                        en = dn - y.d1;
-                        s = y.d1 + y.d0;
-                    }
-                    from_differences(y.e1, y.e0, en, s, a, b);
-                    y.d0 = y.d1;
+                    const T dn = v[e + 2] - v[e + 1], ln = vl[e + 2] - vl[e + 1];
+                    const T gn = y.d1 + y.l1, s = gn + y.g0;
+                    const T en = (dn - y.d1) + (ln - y.l1);
+                    a = fma((T)6, s, -(en - y.e0));
+                    b = fma((T)14, y.e1, -(en + y.e0));
+                    y.l1 = ln;
+                    y.g0 = gn;
                     y.d1 = dn;
                     y.e0 = y.e1;
                     y.e1 = en;
                 }
-                if constexpr (PREC == 2) {
-                    // two-sum of hi and (increment + lo): exact sum t + err
-                    T yy = fma(-(cA * cc), a, fma(cB, b, vl[e]));
-                    if constexpr (FORCED) yy = yy + f;
-                    const T t = cc + yy;
-                    const T z = t - cc;
-                    cl[e] = (cc - (t - z)) + (yy - z);
-                    c[e] = t;
-                } else {
-                    c[e] = fma(cA, increment(cc, a, b, f, FORCED), cc);
-                }
+                // two-sum of hi and (increment + lo): exact sum t + err
+                T yy = fma(-(cA * cc), a, fma(cB, b, vl[e]));
+                if constexpr (FORCED) yy = yy + F[FORCED ? e : 0];
+                const T t = cc + yy;
+                const T z = t - cc;
+                cl[e] = (cc - (t - z)) + (yy - z);
+                c[e] = t;
             }
         }
     }
