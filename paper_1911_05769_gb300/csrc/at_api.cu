@@ -924,7 +924,6 @@ static atk::Params make_params(const at_solver *h)
     p.tab_words = (int)atk::tile_points(h->M, gw, full_runs(h->M, gw));
     p.tab_off = h->sl.tab_off;
     p.sb = 1;
-    p.alt = 0;
     p.timeout_ns = h->g.timeout_ns;
     p.skip_publish = (h->g.flags & AT_FLAG_TEST_SKIP_PUBLISH) ? 1 : 0;
     p.skip_step = h->g.test_skip_step;
@@ -1022,9 +1021,6 @@ static int step_impl(at_solver *h, int64_t n_steps, int delay_mode, int8_t *dela
     p.delays = delays;
     p.n_steps = n_steps;
     p.sb = levels ? 1 : delay_mode == AT_FREE ? h->sb : (delay_mode == AT_SYNC && h->bs_ok) ? sync_pass_len(h) : 1;
-    // blocked free-running passes alternate their sweep direction; the
-    // blocked synchronous passes (a grid barrier before each) need not
-    p.alt = (p.sb > 1 && delay_mode == AT_FREE) ? 1 : 0;
     p.strip_words = strip_words(h, p.sb);
     if (h->batch && h->K > 1 && (delay_mode == AT_FREE || delay_mode == AT_SYNC)) {
         // multi-subdomain tiles (the faces between a tile's subdomains at delay 0)

@@ -190,7 +190,6 @@ struct Params {
     long long n_steps;
     int sb;                    // most levels per pass (temporal blocking: free mode, and the blocked
                                // synchronous mode, where k = 0 and the ghost cells are recomputed)
-    int alt;                   // sweep direction alternates from pass to pass (blocked free mode)
     unsigned long long seed;
     double cA, cB, cr;         // dt/(2dx) | dt/(12dx);  nu dt/dx^2 | nu dt/(12dx^2);  cB / cA
     double fX;                 // forcing factor: A dt (FP64 viscous term, compensated state), else A dt / cA
@@ -584,13 +583,17 @@ static __device__ __noinline__ bool cta_grid_sync(const Params &p, int *s_count,
 // smallest delay bound of its subdomains): a PE's halo waits only need its
 // neighbours' per-level flags, whatever their pass boundaries.
 //
-// alt: the sweep direction alternates from pass to pass (lo..hi-1, then
+// The sweep direction alternates from pass to pass (lo..hi-1, then
 // hi-1..lo, ...).  A pass of L+1 levels must start from its edge neighbours'
 // level n exactly (delay 0); in a one-way sweep the first tile of a pass
 // needs the left neighbour PE's last tile of the previous pass, so every PE
 // waits on its neighbour at each pass start.  Alternating, each edge tile
-// needs a tile its neighbour finished about a pass earlier; and the tile at
-// the turn is the same subdomain twice in a row, continued in registers.
+// needs a tile its neighbour finished about a pass earlier; the tile at
+// the turn is the same subdomain twice in a row, continued in registers; and
+// the tiles next to it are still in the L2 cache, which is what passes of one
+// level over a state about its size gain from: seeded delays, 2^25 FP32
+// points, 100 levels, take 5.02 ms one way and 3.95 ms alternating (free
+// delays on 2^26 points 4.27 ms before and 4.12 ms since).
 //
 // single: passes of one level while the level is below s-1 (the AT halos need
 // s levels); the synchronous modes read level n only and have none.
@@ -599,12 +602,11 @@ struct Sweep {
     int n_steps;               // levels of the launch (the host keeps it below 2^30)
     int sb;
     int single;                // the first `single` levels take one-level passes (start-up)
-    bool alt;
 };
 
 // Position of a tile in a PE's sweep: the pass's first level n relative to n0,
-// tile j (relative to the PE's first), the pass length, (alternating sweeps)
-// the direction of the pass, and the index of the pass within the launch.
+// tile j (relative to the PE's first), the pass length, the direction of the
+// pass, and the index of the pass within the launch.
 struct Cursor {
     int n, j, len, pass;
     bool rev;
@@ -629,9 +631,8 @@ __device__ __forceinline__ void advance(const Sweep &sw, Cursor &c, int S)
     if (c.j != end) {
         c.j += c.rev ? -1 : 1;
     } else {
-        // the next pass: from the first tile, or (alternating) back from the same one
-        if (sw.alt) c.rev = !c.rev;
-        else c.j = 0;
+        // the next pass: back from the same tile
+        c.rev = !c.rev;
         c.n += c.len;
         c.len = pass_len(sw, c.n);
         ++c.pass;
@@ -785,10 +786,10 @@ __device__ void run_pe(const Params &p, const Sweep &sw, long long lo, int S, un
         else return f == 0 ? t == 0 : t == S - 1;
     };
     const int NS = p.stages;
-    // tiles loaded ahead; an alternating sweep revisits the subdomain of
-    // position i after a turn 2i+1 tiles later, so at most 2 ahead there
+    // tiles loaded ahead; the sweep revisits the subdomain of position i
+    // after a turn 2i+1 tiles later, so at most 2 ahead
     int D = S - 1 < NS - 1 ? S - 1 : NS - 1;
-    if (sw.alt && D > 2) D = 2;
+    if (D > 2) D = 2;
     // groups of the tile, owner of the last one (FULL: every lane's run is
     // full, so the last group is the last of its lane)
     const int M = (int)p.M;
@@ -835,10 +836,12 @@ __device__ void run_pe(const Params &p, const Sweep &sw, long long lo, int S, un
         // prescribed modes draw 16 tiles' delays at once (one per lane)
         const unsigned t0 = t & ~15u;
         if (t0 != kb_t0) {
-            // (n, j) of tile t0 + lane/2, stepping from c (tile t) back or forth
-            int jj = c.j - (int)(t - t0) + (lane >> 1), nn = c.n;
+            // (n, j) of tile t0 + lane/2: its place in the sweep from that of c
+            // (tile t), passes of one level, every other one reversed
+            int jj = (c.rev ? S - 1 - c.j : c.j) - (int)(t - t0) + (lane >> 1), nn = c.n;
             while (jj < 0) { jj += S; --nn; }
             while (jj >= S) { jj -= S; ++nn; }
+            if (((nn ^ c.n) & 1) != (c.rev ? 1 : 0)) jj = S - 1 - jj;
             int k = 0;
             if (nn >= 0 && nn < sw.n_steps) {
                 // (prescribed delays: tiles of one subdomain)
@@ -1039,9 +1042,9 @@ __device__ void run_pe(const Params &p, const Sweep &sw, long long lo, int S, un
     int sl = 0;                        // stage of the next load
     int sr = 0;                        // stage of the next loaded tile to use
     unsigned char *stage = stages;     // stage of the tile last read: its way back
-    // after a load: move to the next tile that is loaded (a turn tile of an
-    // alternating sweep is not: it continues in registers; nor is any later
-    // tile of a PE with one subdomain)
+    // after a load: move to the next tile that is loaded (a turn tile is not:
+    // it continues in registers; nor is any later tile of a PE with one
+    // subdomain)
     auto load_next = [&]() {
         issue_load(sl, L.j);
         const int jj = L.j;
@@ -1049,7 +1052,7 @@ __device__ void run_pe(const Params &p, const Sweep &sw, long long lo, int S, un
         ++lead;
         if (S == 1) {
             L.n = sw.n_steps;
-        } else if (sw.alt && L.j == jj) {
+        } else if (L.j == jj) {
             advance(sw, L, S);
             ++lead;
         }
@@ -1081,6 +1084,7 @@ __device__ void run_pe(const Params &p, const Sweep &sw, long long lo, int S, un
         __syncwarp();
     }
     while (lead < D && L.n < sw.n_steps) load_next();
+    int bar_pass = 0;                  // synchronous modes: the pass the grid barrier has admitted
     bool prepared = false;             // the halo of tile r has been prepared
     bool turn = false;                 // tile r continues tile r-1 in registers
     T c[NPT];                          // this lane's points
@@ -1094,7 +1098,8 @@ __device__ void run_pe(const Params &p, const Sweep &sw, long long lo, int S, un
         // synchronous algorithm: before the first tile of a pass (a step when
         // unblocked), all PEs have finished the previous pass (grid barrier,
         // Algorithm 1)
-        if (sync_mode && C.pass > 0 && C.j == 0) {
+        if (sync_mode && C.pass > bar_pass) {
+            bar_pass = C.pass;
             if (!cta_grid_sync(p, s_count, s_epoch, C.pass + ep_off, true)) { ok = false; break; }
             __syncwarp();
         }
@@ -1105,7 +1110,7 @@ __device__ void run_pe(const Params &p, const Sweep &sw, long long lo, int S, un
         const int kf0 = kcur;
         // read the entries of tile r + 1 (in AT_SYNC not across the grid
         // barrier)
-        prepared = N.n < sw.n_steps && !(sync_mode && N.j == 0);
+        prepared = N.n < sw.n_steps && !(sync_mode && N.pass != C.pass);
         if (prepared) prep(r + 1, N);
         const int n = C.n, len = C.len;                   // level at the pass start
         const int s0 = ti.s0, s1 = ti.s0 + ti.cnt - 1;    // its first and last subdomain
@@ -1506,7 +1511,6 @@ __global__ void __launch_bounds__(kThreads, AT_MIN_CTAS_PER_SM) at_stepper(const
     sw.n0 = *reinterpret_cast<const volatile long long *>(p.ctrl + kCtrlN0);
     sw.n_steps = (int)p.n_steps;
     sw.sb = p.sb;
-    sw.alt = p.alt != 0;
     sw.single = (p.mode != kModeSync && sw.n0 < ORDER / 2) ? ORDER / 2 - (int)sw.n0 : 0;
 
     __shared__ int s_count;                   // grid-barrier arrivals of this CTA's warps

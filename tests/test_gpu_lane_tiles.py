@@ -76,3 +76,29 @@ def test_free_running_delay_bounds_beyond_one_read(require_gpu, L):
         ref, hist = oracle_run(u0, mode="replay", delays=g["rec"], **kw)
         assert rel_linf(g["u"], ref) <= TOL["f64"]
         assert np.array_equal(g["hist"], hist)
+
+
+@pytest.mark.parametrize("stages", [2, 3, 4])
+@pytest.mark.parametrize("per_pe", [2, 3, 5, 15, 16, 17, 35])
+def test_one_level_passes_turn(require_gpu, per_pe, stages):
+    """Passes of one level alternate their direction too: the delays drawn 16
+    tiles at a time follow the turns (blocks that end at, before and after a
+    turn, and that hold several), the grid barrier of the synchronous mode
+    stands before a turn tile, and every call starts forward again."""
+    import paper_1911_05769_gb300 as at
+    P, M, L = 8 * per_pe, 64, 3
+    u0, dt = _turn_setup(P * M)
+    kw = dict(P=P, order=4, L=L, nu=0.02, dt=dt, steps=31, forcing=0.1)
+    for mode, name in ((at.AT_SEEDED, "seeded"), (at.AT_SYNC, "sync")):
+        g = gpu_run(u0, mode=mode, seed=11, max_ctas=2, stages=stages, record=True, calls=[1, 17, 13],
+                    steps_per_pass=1, **kw)
+        ref, hist = oracle_run(u0, mode=name, seed=11, **kw)
+        assert g["info"].ctas == 2
+        assert rel_linf(g["u"], ref) <= TOL["f64"], name
+        assert np.array_equal(g["hist"], hist), name
+
+
+def _turn_setup(N):
+    u0 = W.u0_fourier(N, modes=8, seed=N)
+    _, dx = W.grid(N)
+    return u0, 0.5 * W.dt_rule(u0, dx, 0.02)
