@@ -939,9 +939,9 @@ int at_set_state(at_solver *h, const void *u)
     if (h->dim == 3) {
         atk::Params3 p = make_params3(h);
         void *args[] = {&p};
-        const long long work = h->P * 6 * h->nf * h->d3.face_words;
-        const int blocks = (int)((work + 255) / 256 < 4096 ? (work + 255) / 256 : 4096);
-        e = cudaLaunchKernel(h->init_kernel, dim3(blocks), dim3(256), args, 0, h->stream);
+        const long long items = h->P * h->nf;
+        const int blocks = (int)(items < 16384 ? items : 16384);
+        e = cudaLaunchKernel(h->init_kernel, dim3(blocks), dim3(atk::kThreads3), args, 0, h->stream);
         if (e != cudaSuccess) return cuda_fail(e, "launch at_init3d");
         h->step = 0;
             h->has_state = true;

@@ -560,34 +560,59 @@ __global__ void __launch_bounds__(kThreads3, AT_MIN_CTAS_3D)
 }
 
 // level-0 ring entries of every face, flags and control block
-template <typename T>
-__global__ void at_init3d(const Params3 p)
+// Groups of VW columns of two opposite faces: rows `row_a`, `row_b` of `cols`
+// columns and their `rows` successors `stride` words on, to ring planes a, b.
+template <typename T, int VW>
+__device__ __forceinline__ void init_rows(const T *row_a, const T *row_b, unsigned cols, unsigned rows, size_t stride,
+                                          T *a, T *b)
 {
-    const int PWmax = (int)p.face_words;
-    const long long stride = (long long)gridDim.x * blockDim.x;
-    const long long total = p.P * 6 * p.nf * PWmax;
-    const long long field_words = p.n0 * p.n1 * p.n2;
-    for (long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x; t < total; t += stride) {
-        const long long sub = t / (6 * p.nf * PWmax);
-        const int f = (int)((t / ((long long)p.nf * PWmax)) % 6);
-        const int fld = (int)((t / PWmax) % p.nf);
-        const int e = (int)(t % PWmax);
-        const T *u = reinterpret_cast<const T *>(p.u) + (size_t)fld * field_words;
-        const long long s0 = sub % p.P0, s1 = (sub / p.P0) % p.P1, s2 = sub / (p.P0 * p.P1);
-        int x, y, z;
-        if (f < 2) {            // [z][y]
-            if (e >= p.m1 * p.m2) continue;
-            z = e / p.m1; y = e % p.m1; x = f == 0 ? 0 : p.m0 - 1;
-        } else if (f < 4) {     // [z][x]
-            if (e >= p.m0 * p.m2) continue;
-            z = e / p.m0; x = e % p.m0; y = f == 2 ? 0 : p.m1 - 1;
-        } else {                // [y][x]
-            if (e >= p.m0 * p.m1) continue;
-            y = e / p.m0; x = e % p.m0; z = f == 4 ? 0 : p.m2 - 1;
+    const unsigned groups = cols / VW;
+#pragma unroll 4
+    for (unsigned e = threadIdx.x; e < groups * rows; e += kThreads3) {
+        const unsigned r = e / groups, x = (e - r * groups) * VW;
+        T va[VW], vb[VW];
+        lds<T, VW>(row_a + r * stride + x, va);              // (16-byte generic loads of global memory)
+        lds<T, VW>(row_b + r * stride + x, vb);
+        stv<T, VW>(a + r * cols + x, va);
+        stv<T, VW>(b + r * cols + x, vb);
+    }
+}
+
+// A block takes one field of one subdomain at a time and copies its faces in
+// pairs, x faces word by word, y and z faces in 16-byte groups where rows allow.
+// Bound by memory: the x faces touch half the state's sectors.  (One thread per
+// word with its place from 64-bit divisions was bound by those: 512^3 FP32 points
+// in 32^3 subdomains took 313 us; set_state, 24 levels and the state back 5.87 ms
+// then, 5.68 so; five fields of 256^3, 16 levels, 4.64 and 4.40 ms.)
+template <typename T>
+__global__ void __launch_bounds__(kThreads3) at_init3d(const Params3 p)
+{
+    const unsigned m0 = p.m0, m1 = p.m1, m2 = p.m2, nf = p.nf;
+    const size_t row = (size_t)p.n0, plane = (size_t)(p.n0 * p.n1);
+    const unsigned uP0 = (unsigned)p.P0, uP1 = (unsigned)p.P1;
+    const bool groups = m0 % 4 == 0;                         // (then n0 and every array's words are multiples of 4)
+    for (long long item = blockIdx.x; item < p.P * (int)nf; item += gridDim.x) {
+        const unsigned sub = (unsigned)(item / nf), fld = (unsigned)(item - (long long)sub * nf);
+        const unsigned q1 = sub / uP0, s0 = sub - q1 * uP0, s2 = q1 / uP1, s1 = q1 - s2 * uP1;
+        const T *u = reinterpret_cast<const T *>(p.u) + (size_t)fld * plane * (size_t)p.n2 +
+                     (size_t)s2 * m2 * plane + (size_t)s1 * m1 * row + (size_t)s0 * m0;
+        auto face = [&](int f) -> T * { return ring_entry<T>(p, 0, sub, f) + (size_t)fld * p.face_words; };
+        T *const x0 = face(0), *const x1 = face(1);
+#pragma unroll 4
+        for (unsigned e = threadIdx.x; e < m1 * m2; e += kThreads3) {
+            const unsigned z = e / m1, y = e - z * m1;
+            const T *r = u + z * plane + y * row;
+            x0[e] = r[0];
+            x1[e] = r[m0 - 1];
         }
-        const size_t gi = ((size_t)(s2 * p.m2 + z) * p.n1 + (size_t)(s1 * p.m1 + y)) * p.n0 + (size_t)(s0 * p.m0 + x);
-        ring_entry<T>(p, 0, sub, f)[(size_t)fld * PWmax + e] = u[gi];
-        if (e == 0 && fld == 0) p.flag[sub * 6 + f] = 0ull;
+        if (groups) {
+            init_rows<T, 4>(u, u + (m1 - 1) * row, m0, m2, plane, face(2), face(3));
+            init_rows<T, 4>(u, u + (m2 - 1) * plane, m0, m1, row, face(4), face(5));
+        } else {
+            init_rows<T, 1>(u, u + (m1 - 1) * row, m0, m2, plane, face(2), face(3));
+            init_rows<T, 1>(u, u + (m2 - 1) * plane, m0, m1, row, face(4), face(5));
+        }
+        if (fld == 0 && threadIdx.x < 6) p.flag[(size_t)sub * 6 + threadIdx.x] = 0ull;
     }
     if (blockIdx.x == 0) {
         if (threadIdx.x < kCtrlWords) p.ctrl[threadIdx.x] = 0;
