@@ -1496,9 +1496,8 @@ __global__ void __launch_bounds__(kThreads, AT_MIN_CTAS_PER_SM) at_stepper(const
 {
     extern __shared__ __align__(128) unsigned char smem[];
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const long long e = (long long)blockIdx.x * kWarps + w;     // this warp's PE
-    const long long lo = e * p.ntiles / p.E;                  // this PE's tiles
-    const long long hi = (e + 1) * p.ntiles / p.E;
+    const ItemRange own = item_range(p.ntiles, p.E, (long long)blockIdx.x * kWarps + w);   // this warp's tiles
+    const long long lo = own.lo, hi = own.hi;
     const long long S = hi - lo;
     unsigned char *raw = smem + p.raw_off + (size_t)w * kRawBytes;
     unsigned char *stages = smem + p.stage_off + (size_t)w * p.stages * p.stage_bytes;

@@ -224,7 +224,8 @@ __global__ void __launch_bounds__(kThreads3, AT_MIN_CTAS_3D)
     const long long fw = p.face_words;
 
     const int tid = threadIdx.x, lane = tid & 31;
-    const long long lo = (long long)blockIdx.x * p.P / p.G, hi = (long long)(blockIdx.x + 1) * p.P / p.G;
+    const ItemRange own = item_range(p.P, p.G, blockIdx.x);
+    const long long lo = own.lo, hi = own.hi;
     const long long S = hi - lo;
     const long long lev0 = *reinterpret_cast<const volatile long long *>(p.ctrl + kCtrlN0);
     const int NS = p.stages;

@@ -97,7 +97,8 @@ __global__ void __launch_bounds__(kThreads3b, sizeof(T) == 4 ? 2 : 1)
     const int fw = MS ? MS * MS : (int)p.face_words;
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const long long lo = (long long)blockIdx.x * p.P / p.G, hi = (long long)(blockIdx.x + 1) * p.P / p.G;
+    const ItemRange own = item_range(p.P, p.G, blockIdx.x);
+    const long long lo = own.lo, hi = own.hi;
     const long long S = hi - lo;
     const long long lev0 = *reinterpret_cast<const volatile long long *>(p.ctrl + kCtrlN0);
     const long long lev_end = lev0 + p.n_steps;

@@ -127,8 +127,9 @@ __global__ void __launch_bounds__(NT * TEAMS, v4_min_ctas(NF, NT * TEAMS))
     const unsigned tx_bytes = (unsigned)(NF * bp);                           // one box: a plane of every field
 
     const int tid = (int)threadIdx.x - team * NT, lane = tid & 31, warp = tid >> 5;   // within the team
-    const long long pe = (long long)blockIdx.x * TEAMS + team, npes = (long long)p.G * TEAMS;
-    const long long lo = pe * p.P / npes, hi = (pe + 1) * p.P / npes;
+    const long long npes = (long long)p.G * TEAMS;
+    const ItemRange own = item_range(p.P, npes, (long long)blockIdx.x * TEAMS + team);
+    const long long lo = own.lo, hi = own.hi;
     const long long S = hi - lo;
     const long long lev0 = *reinterpret_cast<const volatile long long *>(p.ctrl + kCtrlN0);
     const long long Q = p.n_steps * S * m2;                                  // planes this team sweeps
