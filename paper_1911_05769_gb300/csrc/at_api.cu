@@ -266,6 +266,58 @@ void pick_kernels(int w, int order, int64_t M, bool forced, bool v64, bool comp,
     if (stepper_bs) *stepper_bs = bs;
 }
 
+// The tiles of an ensemble whose passes have one length: first tile in the list
+// and cost of a tile and level.
+struct TileGroup {
+    int64_t first, tiles;
+    double cost;
+};
+using TileGroups = std::vector<TileGroup>;
+
+// Shares G CTAs out among the groups so that the slowest takes least (none:
+// fewer CTAs than groups; one group).  *most: most tiles of a PE.
+//   A pass costs as much as `c` levels besides its levels, so a tile in passes
+// of 2 levels takes longer per level than one in passes of 4: 1.58, 1.21 and 1.03
+// us for 2, 3 and 4 (1824 PEs, tiles of 1024 FP32 points, order 2, c = 4.6).  With
+// one tile count for all, the PEs of the short passes were last (2048 instances,
+// 100 steps 3.20 ms, now 2.92).
+atk::TileSplit split_tiles(const TileGroups &gr, int G, int64_t *most)
+{
+    atk::TileSplit sp{};
+    *most = 0;
+    if (gr.size() < 2 || (int64_t)gr.size() > G) return sp;
+    const int n = (int)gr.size();
+    auto ctas = [&](double limit, int g) -> int64_t {
+        const int64_t per = (int64_t)(limit / gr[(size_t)g].cost) * atk::kWarps;      // tiles of a CTA
+        return per < 1 ? (int64_t)G + 1 : (gr[(size_t)g].tiles + per - 1) / per;
+    };
+    auto fits = [&](double limit) -> bool {
+        int64_t sum = 0;
+        for (int g = 0; g < n && sum <= G; ++g) sum += ctas(limit, g);
+        return sum <= G;
+    };
+    double lo = 0.0, hi = 0.0;                 // (hi: a CTA for each group is enough)
+    for (const TileGroup &t : gr) hi += (double)(t.tiles + 1) * t.cost;
+    for (int it = 0; it < 60; ++it) {
+        const double mid = 0.5 * (lo + hi);
+        if (fits(mid)) hi = mid;
+        else lo = mid;
+    }
+    int64_t left = G;
+    for (int g = 0; g < n; ++g) left -= ctas(hi, g);
+    for (int g = 0; g < n; ++g) {
+        // (CTAs left over: to the groups in turn)
+        const int64_t c = ctas(hi, g) + left / n + (g < left % n ? 1 : 0);
+        const int64_t per = (gr[(size_t)g].tiles + c * atk::kWarps - 1) / (c * atk::kWarps);
+        sp.tile[g] = gr[(size_t)g].first;
+        sp.cta[g + 1] = sp.cta[g] + (int)c;
+        if (per > *most) *most = per;
+    }
+    sp.tile[n] = gr.back().first + gr.back().tiles;
+    sp.groups = n;
+    return sp;
+}
+
 // Shared-memory table of a CTA: `fixed` bytes plus `per_sub` bytes per
 // subdomain of each of its PEs and `extra` more subdomains per PE (forcing:
 // sin/cos tables, which also cover the PE's two outer neighbours; ensembles:
@@ -276,6 +328,7 @@ struct TabSize {
     int extra;
     int64_t ntk;     // ensembles: tiles of the multi-subdomain list (0: single domain)
     int k;           // ensembles: most subdomains per tile
+    const TileGroups *groups = nullptr;   // ensembles: the list's groups of one pass length
 };
 
 TabSize tab_size(int64_t M, int w, bool forced, bool batch, bool comp = false, int64_t ntk = 0, int k = 1)
@@ -314,6 +367,11 @@ int launch_shape(int64_t M, int w, int64_t P, TabSize tsz, int max_ctas, int sta
         if (tsz.ntk > 0 && tsz.k > 1) {
             const long long sk = (tsz.ntk + E - 1) / E * tsz.k;
             if (sk > *smax) *smax = sk;
+        }
+        if (tsz.groups) {
+            int64_t most = 0;
+            split_tiles(*tsz.groups, G, &most);
+            if (most * tsz.k > *smax) *smax = most * tsz.k;
         }
         const long long tab = tsz.fixed + (long long)atk::kWarps * (*smax + tsz.extra) * tsz.per_sub;
         const int gw = groups_per_lane(M);
@@ -416,6 +474,7 @@ struct at_solver {
     int lmin;                  // smallest delay bound (ensembles), else L
     int K;                     // ensembles: subdomains per tile of the AT_FREE / AT_SYNC list
     int64_t ntiles_k;          // ensembles: tiles of that list
+    atk::TileSplit split{};    // ensembles: the CTAs' shares of the tiles in AT_FREE passes
     std::vector<atk::BatchSub> bsub_host;   // ensembles: the subdomain records (tile planning)
     std::vector<at_instance> inst_host;     // ensembles: the instances
     void *kernel;
@@ -543,6 +602,33 @@ void plan_tiles(const std::vector<atk::BatchSub> &sub, int64_t n_inst, const at_
             d.z = cnt | (link << 16);
         }
     }
+}
+
+// The groups of the list of K subdomains per tile for passes of at most sb levels
+// (instances in the order of the lists).
+TileGroups tile_groups(const at_solver *h, int K, int sb)
+{
+    TileGroups gr;
+    if (sb < 2) return gr;
+    std::vector<int64_t> idx((size_t)h->n_inst);
+    for (int64_t j = 0; j < h->n_inst; ++j) idx[(size_t)j] = j;
+    std::stable_sort(idx.begin(), idx.end(),
+                     [&](int64_t a, int64_t b) { return h->inst_host[(size_t)a].L < h->inst_host[(size_t)b].L; });
+    // levels that a pass costs besides its own (see split_tiles; measured at
+    // order 2, elsewhere by the operations of a level)
+    const double c = h->w == 8 ? 0.4 : h->comp ? 2.0 : h->order == 4 ? 3.0 : 4.6;
+    int last = -1;
+    int64_t at = 0;
+    for (int64_t j : idx) {
+        const at_instance &a = h->inst_host[(size_t)j];
+        const int len = a.L + 1 < sb ? a.L + 1 : sb;
+        if (len != last) gr.push_back({at, 0, 1.0 + c / len});
+        last = len;
+        const int64_t n = (a.n / h->M + K - 1) / K;
+        gr.back().tiles += n;
+        at += n;
+    }
+    return gr;
 }
 
 // Ensembles: plans the tile lists for K subdomains per tile, copies them to
@@ -1027,6 +1113,7 @@ static int step_impl(at_solver *h, int64_t n_steps, int delay_mode, int8_t *dela
         p.tiles = reinterpret_cast<const int4 *>(h->ws + h->lay.tiles) + h->P;
         p.ntiles = h->ntiles_k;
     }
+    if (h->batch && delay_mode == AT_FREE) p.split = h->split;
     p.levels = levels;
     p.levels_depth = depth;
     // (the kernel counts the levels of a launch in 32 bits)
@@ -1351,11 +1438,15 @@ int at_create_batch(const at_grid *grid, int64_t n_inst, const at_instance *inst
     h->init_kernel = w == 8 ? atk_init_kernel_f64(scheme_order) : atk_init_kernel_f32(scheme_order);
     int stages = grid->stages > 0 ? grid->stages : 3;
     if (stages < atk::kMinStages) stages = atk::kMinStages;
-    rc = launch_shape((int64_t)h->K * M, w, d.P, tab_size(M, w, false, true, comp, h->ntiles_k, h->K), grid->max_ctas,
-                      stages, grid->stages > 0, sms, smem_optin, h->kernel, &h->G, &h->stages, &h->sl, &h->smem, &h->smax);
+    h->sb = grid->steps_per_pass > 0 ? grid->steps_per_pass : 1;
+    const TileGroups groups = tile_groups(h, h->K, h->sb);
+    TabSize tsz = tab_size(M, w, false, true, comp, h->ntiles_k, h->K);
+    tsz.groups = &groups;
+    rc = launch_shape((int64_t)h->K * M, w, d.P, tsz, grid->max_ctas, stages, grid->stages > 0, sms, smem_optin, h->kernel, &h->G, &h->stages, &h->sl, &h->smem, &h->smax);
     if (rc != AT_OK) { delete h; return rc; }
     prepare_bs(h);
-    h->sb = grid->steps_per_pass > 0 ? grid->steps_per_pass : 1;
+    int64_t most = 0;
+    h->split = split_tiles(groups, h->G, &most);
     h->step = 0;
     h->has_state = false;
     *out = h;
@@ -1398,7 +1489,9 @@ int at_tune(at_solver *h, int64_t n_steps, int delay_mode, at_tune_result *res)
         }
         // (a tile is one subdomain, except in an ensemble of K-subdomain tiles)
         const int kt = h->batch ? h->K : 1;
-        const TabSize tsz = tab_size(h->M, h->w, h->g.forcing_amp != 0.0, h->batch, h->comp, h->ntiles_k, kt);
+        TabSize tsz = tab_size(h->M, h->w, h->g.forcing_amp != 0.0, h->batch, h->comp, h->ntiles_k, kt);
+        const TileGroups groups = h->batch ? tile_groups(h, kt, sh.sb) : TileGroups{};
+        tsz.groups = &groups;
         int G = 0, st = 0, smem = 0;
         long long smax = 0;
         atk::SmemLayout sl{};
@@ -1407,6 +1500,8 @@ int at_tune(at_solver *h, int64_t n_steps, int delay_mode, at_tune_result *res)
         if (r != AT_OK) return r;
         if (st != sh.stages) return AT_ERR_RESIDENCY;   // did not fit as asked
         h->G = G; h->stages = st; h->sl = sl; h->smem = smem; h->smax = smax; h->sb = sh.sb;
+        int64_t most = 0;
+        h->split = split_tiles(groups, G, &most);
         prepare_bs(h);
         return AT_OK;
     };

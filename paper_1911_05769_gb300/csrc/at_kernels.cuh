@@ -166,6 +166,15 @@ struct TileInfo {
     int s0, rec, cnt, link;
 };
 
+// Ensembles in passes of several levels: the CTAs from cta[g] to cta[g + 1] own
+// the tiles from tile[g] to tile[g + 1], whose instances have one pass length
+// (0 groups: all CTAs own all tiles).
+struct TileSplit {
+    int groups;
+    int cta[kMaxL + 2];
+    long long tile[kMaxL + 2];
+};
+
 struct Params {
     void *u;                   // state, N words, updated in place
     unsigned char *ring;       // [T][P][2] entries (see entry_halves)
@@ -178,6 +187,7 @@ struct Params {
     const BatchInst *binst;    // ensembles: instance records (else NULL)
     const int4 *tiles;         // ensembles: the launch's tile list [ntiles] (see TileInfo)
     const int *sub_order;      // ensembles: subdomain at each place of the tile lists' enumeration [P]
+    TileSplit split;
     long long ntiles;          // tiles of the launch (single domain: P, tile j = subdomain j)
     int ktile;                 // most subdomains per tile
     void *ur;                  // compensated state: the rounding error of every point (N words)
@@ -1496,8 +1506,18 @@ __global__ void __launch_bounds__(kThreads, AT_MIN_CTAS_PER_SM) at_stepper(const
 {
     extern __shared__ __align__(128) unsigned char smem[];
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const ItemRange own = item_range(p.ntiles, p.E, (long long)blockIdx.x * kWarps + w);   // this warp's tiles
-    const long long lo = own.lo, hi = own.hi;
+    // this warp's tiles (an ensemble: of its CTA's group)
+    int g0 = 0, g1 = p.G;
+    long long t0 = 0, t1 = p.ntiles;
+    if constexpr (BATCH) {
+        for (int g = 0; g < p.split.groups; ++g) {
+            if ((int)blockIdx.x < p.split.cta[g]) break;
+            g0 = p.split.cta[g]; g1 = p.split.cta[g + 1];
+            t0 = p.split.tile[g]; t1 = p.split.tile[g + 1];
+        }
+    }
+    const ItemRange own = item_range(t1 - t0, (long long)(g1 - g0) * kWarps, (long long)((int)blockIdx.x - g0) * kWarps + w);
+    const long long lo = t0 + own.lo, hi = t0 + own.hi;
     const long long S = hi - lo;
     unsigned char *raw = smem + p.raw_off + (size_t)w * kRawBytes;
     unsigned char *stages = smem + p.stage_off + (size_t)w * p.stages * p.stage_bytes;
