@@ -41,7 +41,7 @@ void *atk_batch_kernel_f32c(int order, int gw, bool full);
 void *atk_restore_kernel_f32(int order);
 void *atk_restore_kernel_f64(int order);
 void *atk_adjoint_kernel(int w, int order);
-void *atk_resident_kernel(int w, int order, int ppl, bool forced);
+void *atk_resident_kernel(int w, int order, int ppl, bool forced, bool cluster);
 void *atk_adjoint_warp_kernel(int w, int order, int gw, bool full);
 void *atk_stepper3d_kernel(int w, int tc);
 void *atk_stepper3d_iso_kernel(int w, int tc);
@@ -482,11 +482,22 @@ struct at_solver {
     void *kernel_b3;           // 3D: the blocked free-running kernel (NULL: none)
     int G_b3, stages_b3, smem_b3;   // 3D: its CTAs, plane stages and shared memory
     void *kernel_res;          // 1D: the one-subdomain-per-CTA kernel of prescribed delays (NULL: none)
+    bool res_cluster = false;  // ... whose CTAs are one cluster
     bool bs_ok;                // it can run in the launch shape chosen for `kernel`
     void *init_kernel;
 };
 
 namespace {
+
+// one cluster of n CTAs
+cudaLaunchAttribute cluster_attr(int n)
+{
+    cudaLaunchAttribute a{};
+    a.id = cudaLaunchAttributeClusterDimension;
+    a.val.clusterDim.x = (unsigned)n;
+    a.val.clusterDim.y = a.val.clusterDim.z = 1;
+    return a;
+}
 
 // One launch of the persistent stepper: cooperative, so that every CTA is
 // resident; cudaLaunchKernelExC with the cooperative attribute may be
@@ -505,8 +516,12 @@ cudaError_t launch_stepper(at_solver *h, atk::Params *p, void *kernel)
     cfg.dynamicSmemBytes = (size_t)(res ? 0 : h->smem);
     cfg.stream = h->stream;
     cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeCooperative;
-    attr[0].val.cooperative = 1;
+    if (res && h->res_cluster) {
+        attr[0] = cluster_attr((int)h->P);               // (co-resident by itself)
+    } else {
+        attr[0].id = cudaLaunchAttributeCooperative;
+        attr[0].val.cooperative = 1;
+    }
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     void *args[] = {p};
@@ -521,14 +536,34 @@ cudaError_t launch_stepper(at_solver *h, atk::Params *p, void *kernel)
 cudaError_t prepare_resident(at_solver *h)
 {
     h->kernel_res = nullptr;
+    h->res_cluster = false;
     if (h->batch || h->comp || h->v64 || h->g.max_ctas > 0 || (h->g.flags & AT_FLAG_TEST_SKIP_PUBLISH)) return cudaSuccess;
     const int ppt = atk::resident_points(h->M), threads = atk::resident_threads(h->M);
     if (h->P > (int64_t)32 * h->sm_count) return cudaSuccess;
-    void *kern = atk_resident_kernel(h->w, h->order, ppt, h->g.forcing_amp != 0.0);
+    void *kern = atk_resident_kernel(h->w, h->order, ppt, h->g.forcing_amp != 0.0, false);
     int occ = 0;
     const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, threads, 0);
     if (e != cudaSuccess) return e;
     if ((int64_t)occ * h->sm_count >= h->P) h->kernel_res = kern;
+    // up to kMaxCluster subdomains, the largest cluster there is: the cluster variant,
+    // if the device has room for one of that size (times of both at kMaxCluster)
+    if (h->P <= atk::kMaxCluster && h->T <= atk::kClusterSlots) {
+        kern = atk_resident_kernel(h->w, h->order, ppt, h->g.forcing_amp != 0.0, true);
+        cudaLaunchAttribute attr = cluster_attr((int)h->P);
+        cudaLaunchConfig_t cfg{};
+        cfg.gridDim = dim3((unsigned)h->P);
+        cfg.blockDim = dim3(threads);
+        cfg.attrs = &attr;
+        cfg.numAttrs = 1;
+        int clusters = 0;
+        if (cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
+            cudaOccupancyMaxActiveClusters(&clusters, kern, &cfg) == cudaSuccess && clusters > 0) {
+            h->kernel_res = kern;
+            h->res_cluster = true;
+        } else {
+            cudaGetLastError();
+        }
+    }
     return cudaSuccess;
 }
 
