@@ -1945,7 +1945,8 @@ extern "C" int at_step_noalloc(const at_grid *grid, int64_t P, int scheme_order,
                       grid->stages > 0, sms, smem_optin, h.kernel, &h.G, &h.stages, &h.sl, &h.smem, &h.smax);
     if (rc != AT_OK) return rc;
     h.sb = 1;
-    e = prepare_resident(&h);
+    // (the other modes never take it)
+    if (delay_mode == AT_SEEDED || delay_mode == AT_REPLAY) e = prepare_resident(&h);
     if (e != cudaSuccess) return cuda_fail(e, "cudaOccupancyMaxActiveBlocksPerMultiprocessor");
 
     // Every call starts from zeroed ring buffers, flags, status and counters:
