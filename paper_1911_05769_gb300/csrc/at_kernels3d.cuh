@@ -325,6 +325,9 @@ __global__ void __launch_bounds__(kThreads3, AT_MIN_CTAS_3D)
     // Every warp runs the same number of tiles and meets the same CTA
     // barriers; a failed wait inside a tile only skips that warp's remaining
     // planes, and all threads leave together after the next tile-start barrier.
+    // (decided by the barrier itself: a word tested behind a plain barrier may
+    // have been set since by a warp that is already past it)
+    auto aborted = [&]() -> bool { return __syncthreads_or(*reinterpret_cast<volatile int *>(s_flag) == -1) != 0; };
     bool ok = true;
     long long lv = lev0, sub = lo;
     long long g = 0;                         // plane of the sweep being computed (0 .. Q-1)
@@ -334,8 +337,7 @@ __global__ void __launch_bounds__(kThreads3, AT_MIN_CTAS_3D)
     for (long long t = 0; t < n_tiles; ++t) {
         // ---- tile start (two CTA barriers): release the previous tile's
         // flags, grid barrier (synchronous mode), delays, halos
-        __syncthreads();
-        if (*s_flag == -1) { ok = false; break; }
+        if (aborted()) { ok = false; break; }
         if (tid == 0 && prev_sub >= 0 && !(p.skip_publish && blockIdx.x == 0 && prev_new > p.skip_step)) {
             __threadfence();
             for (int f = 0; f < 6; ++f) st_release(p.flag + prev_sub * 6 + f, (unsigned long long)prev_new);
@@ -423,8 +425,7 @@ __global__ void __launch_bounds__(kThreads3, AT_MIN_CTAS_3D)
             }
         }
         if (tid == 0 && p.mode == kModeSync) __threadfence();
-        __syncthreads();
-        if (*s_flag == -1) { ok = false; break; }
+        if (aborted()) { ok = false; break; }
         // plane z = -1 (the -z halo) and plane 0
         if (!wait_plane(gs, gp)) { ok = false; }
         {
@@ -528,7 +529,7 @@ __global__ void __launch_bounds__(kThreads3, AT_MIN_CTAS_3D)
         tx0 = nx0; ty0 = ny0; tz0 = nz0;
         tile_coords(sub + 1 == hi ? lo : sub + 1, &nx0, &ny0, &nz0);
     }
-    __syncthreads();
+    if (aborted()) ok = false;
     if (tid == 0 && ok && prev_sub >= 0 && !(p.skip_publish && blockIdx.x == 0 && prev_new > p.skip_step)) {
         __threadfence();
         for (int f = 0; f < 6; ++f) st_release(p.flag + prev_sub * 6 + f, (unsigned long long)prev_new);

@@ -54,8 +54,9 @@ constexpr long long kGraceNs = 20000;
 
 // grid barrier before level `step` (1-based within the launch), one arrival per
 // team that has subdomains (npe of them); bounded.  Returns false on abort.
-template <int NT, typename Sync>
-__device__ bool team_grid_sync(const Params3 &p, long long step, long long npe, int ttid, volatile int *s_flag, Sync sync)
+template <typename Sync, typename Any>
+__device__ bool team_grid_sync(const Params3 &p, long long step, long long npe, int ttid, volatile int *s_flag, Sync sync,
+                               Any any)
 {
     sync();
     if (ttid == 0) {
@@ -69,8 +70,7 @@ __device__ bool team_grid_sync(const Params3 &p, long long step, long long npe, 
         }
         __threadfence();
     }
-    sync();
-    return *s_flag != -1;
+    return !any(*s_flag == -1);
 }
 
 // Shared memory of a team: stage barriers and counters, delay counters, the
@@ -112,6 +112,20 @@ __global__ void __launch_bounds__(NT * TEAMS, v4_min_ctas(NF, NT * TEAMS))
     auto sync = [&]() {
         if constexpr (TEAMS == 1) __syncthreads();
         else asm volatile("bar.sync %0, %1;" ::"r"(team + 1), "n"(NT) : "memory");
+    };
+    // the same, and whether `x` holds for any of them: the whole team leaves or
+    // stays together (a word tested after a plain barrier may have been set
+    // since by a thread that is already past it)
+    auto any = [&](bool x) -> bool {
+        if constexpr (TEAMS == 1) {
+            return __syncthreads_or(x) != 0;
+        } else {
+            int r;
+            asm volatile("{\n\t.reg .pred a, b;\n\tsetp.ne.s32 a, %1, 0;\n\t"
+                         "barrier.cta.red.or.pred b, %2, %3, a;\n\tselp.s32 %0, 1, 0, b;\n\t}"
+                         : "=r"(r) : "r"((int)x), "r"(team + 1), "n"(NT) : "memory");
+            return r != 0;
+        }
     };
     uint64_t *bars = reinterpret_cast<uint64_t *>(smem);
     unsigned *hist = reinterpret_cast<unsigned *>(smem + sl.hist_off);
@@ -195,7 +209,7 @@ __global__ void __launch_bounds__(NT * TEAMS, v4_min_ctas(NF, NT * TEAMS))
     int gs = 0;                              // stage and fill parity of the current plane
     unsigned gp = 0;
     // every lane tests the stage's barrier; a wait that runs out is recorded in
-    // s_flag, on which all threads act at the next barrier of a tile start
+    // s_flag, on which the team acts as one at the next barrier of a tile start
     auto wait_plane = [&](int st, unsigned par) -> bool {
         bool good = mbar_try_wait(&bars[st], par);
         if (!good) {
@@ -243,8 +257,7 @@ __global__ void __launch_bounds__(NT * TEAMS, v4_min_ctas(NF, NT * TEAMS))
     for (long long t = 0; t < n_tiles; ++t) {
         // ---- tile start: the previous tile's faces to the ring, grid barrier
         // (synchronous mode), delays, halos
-        sync();
-        if (*reinterpret_cast<volatile int *>(s_flag) == -1) { ok = false; break; }
+        if (any(*reinterpret_cast<volatile int *>(s_flag) == -1)) { ok = false; break; }
         // (released before this tile waits for other teams' flags)
         if (prev_sub >= 0) {
             faces_out(prev_sub, prev_new);
@@ -252,7 +265,7 @@ __global__ void __launch_bounds__(NT * TEAMS, v4_min_ctas(NF, NT * TEAMS))
             release(prev_sub, prev_new);
         }
         if (p.mode == kModeSync && sub == lo && lv > lev0) {
-            if (!team_grid_sync<NT>(p, lv - lev0, p.P < npes ? p.P : npes, tid, s_flag, sync)) { ok = false; break; }
+            if (!team_grid_sync(p, lv - lev0, p.P < npes ? p.P : npes, tid, s_flag, sync, any)) { ok = false; break; }
         }
         const unsigned us = (unsigned)sub, us2 = us / uP01, usr = us - us2 * uP01, us1 = usr / uP0;
         const long long s0 = usr - us1 * uP0, s1 = us1, s2 = us2;
@@ -295,8 +308,7 @@ __global__ void __launch_bounds__(NT * TEAMS, v4_min_ctas(NF, NT * TEAMS))
             s_k[f] = (int)k;
             __threadfence();
         }
-        sync();
-        if (*reinterpret_cast<volatile int *>(s_flag) == -1) { ok = false; break; }
+        if (any(*reinterpret_cast<volatile int *>(s_flag) == -1)) { ok = false; break; }
         // halos, (k+1) f0 - k f1 in Newton form f0 + k (f0 - f1): the z faces of
         // this thread's columns into registers, the x and y faces into shared
         // memory; the loads of two faces in flight together
@@ -578,8 +590,7 @@ __global__ void __launch_bounds__(NT * TEAMS, v4_min_ctas(NF, NT * TEAMS))
         tx0 = nx0; ty0 = ny0; tz0 = nz0;
         tile_coords(sub + 1 == hi ? lo : sub + 1, &nx0, &ny0, &nz0);
     }
-    sync();
-    if (*reinterpret_cast<volatile int *>(s_flag) == -1) ok = false;
+    if (any(*reinterpret_cast<volatile int *>(s_flag) == -1)) ok = false;
     if (ok && prev_sub >= 0) {
         faces_out(prev_sub, prev_new);
         sync();

@@ -1,0 +1,41 @@
+"""Bounded waits of the steppers that run out: the first CTA stops publishing
+(test knob), every kernel form returns with AT_ERR_TIMEOUT latched, and the
+next run on the context is right."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from gpu_util import TOL, rel_linf
+from test_gpu_3d_groups import box
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("sub,dtype", [((8, 8, 4), "f32"), ((16, 16, 4), "f32"), ((32, 16, 4), "f32"),
+                                       ((32, 32, 4), "f32"), ((12, 8, 4), "f32"), ((16, 8, 4), "f64")])
+@pytest.mark.parametrize("mode_name", ["seeded", "free"])
+@pytest.mark.parametrize("skip", [0, 5])
+def test_3d_teams_leave_together(sub, dtype, mode_name, skip):
+    """Planes of 64 to 1024 points (CTAs of 8, 4, 2 and 1 teams, and the kernel
+    of single columns); the knob acts from the first level on, so that the
+    first tiles' waits run out, or after some."""
+    import paper_1911_05769_gb300 as at
+    mode = at.AT_SEEDED if mode_name == "seeded" else at.AT_FREE
+    n = (4 * sub[0], 4 * sub[1], 6 * sub[2])
+    u0 = box(n, 9)[0]
+    length = tuple(0.3 * k for k in n)
+    for flags in (at.AT_FLAG_TEST_SKIP_PUBLISH, 0):
+        s = at.Solver3D(n, sub, 2, 0.2, 0.04, dtype=dtype, length=length, seed=3, max_ctas=3, flags=flags,
+                        test_skip_step=skip, timeout_ns=20_000_000 if flags else 0)
+        s.set_state(torch.from_numpy(np.ascontiguousarray(u0)).ravel())
+        s.step(15, mode if flags else at.AT_SEEDED)
+        if flags:
+            assert s.status() == at.AT_ERR_TIMEOUT
+            assert "timed out" in at.at_last_error()
+        else:
+            out = s.state().double().cpu().numpy().reshape(u0.shape)
+        s.close()
+    ref, _ = oracle.run3d(u0, delay_mode=oracle.SEEDED, seed=3, P=(4, 4, 6), n_steps=15, L=2, nu=0.2, dt=0.04,
+                          dx=tuple(length[a] / n[a] for a in range(3)))
+    assert rel_linf(out, ref) <= TOL[dtype]
