@@ -537,7 +537,7 @@ cudaError_t prepare_resident(at_solver *h)
 {
     h->kernel_res = nullptr;
     h->res_cluster = false;
-    if (h->batch || h->comp || h->v64 || h->g.max_ctas > 0 || (h->g.flags & AT_FLAG_TEST_SKIP_PUBLISH)) return cudaSuccess;
+    if (h->batch || h->comp || h->v64 || h->g.max_ctas > 0) return cudaSuccess;
     const int ppt = atk::resident_points(h->M), threads = atk::resident_threads(h->M);
     if (h->P > (int64_t)32 * h->sm_count) return cudaSuccess;
     void *kern = atk_resident_kernel(h->w, h->order, ppt, h->g.forcing_amp != 0.0, false);

@@ -5,8 +5,9 @@ import numpy as np
 import pytest
 import torch
 
+import at_workloads as W
 import oracle
-from gpu_util import TOL, rel_linf
+from gpu_util import TOL, gpu_run, oracle_run, rel_linf
 from test_gpu_3d_groups import box
 
 pytestmark = pytest.mark.gpu
@@ -39,3 +40,24 @@ def test_3d_teams_leave_together(sub, dtype, mode_name, skip):
     ref, _ = oracle.run3d(u0, delay_mode=oracle.SEEDED, seed=3, P=(4, 4, 6), n_steps=15, L=2, nu=0.2, dt=0.04,
                           dx=tuple(length[a] / n[a] for a in range(3)))
     assert rel_linf(out, ref) <= TOL[dtype]
+
+
+@pytest.mark.parametrize("P", [2, 5, 16, 17, 200])
+@pytest.mark.parametrize("M,order,dtype", [(32, 2, "f64"), (64, 4, "f64"), (100, 4, "f32"), (256, 2, "f64"), (1024, 4, "f32")])
+@pytest.mark.parametrize("skip", [0, 7])
+def test_one_subdomain_per_cta_leaves_together(P, M, order, dtype, skip):
+    """Prescribed delays with a CTA per subdomain, of one to eight warps, through
+    a cluster (P <= 16) and through the ring."""
+    import paper_1911_05769_gb300 as at
+    u0 = W.u0_two_modes(P * M)
+    u0 = u0.astype(np.float32 if dtype == "f32" else np.float64).astype(np.float64)
+    _, dx = W.grid(P * M)
+    kw = dict(P=P, order=order, L=2, nu=0.02, dt=0.1 * W.dt_rule(u0, dx, 0.02), steps=80, seed=3)
+    g = gpu_run(u0, mode=at.AT_SEEDED, dtype=dtype, flags=at.AT_FLAG_TEST_SKIP_PUBLISH, test_skip_step=skip,
+                timeout_ns=20_000_000, check=False, **kw)
+    assert g["rc"] == at.AT_ERR_TIMEOUT
+    # levels up to the one published run
+    g = gpu_run(u0, mode=at.AT_SEEDED, dtype=dtype, flags=at.AT_FLAG_TEST_SKIP_PUBLISH, test_skip_step=80, **kw)
+    ref, hist = oracle_run(u0, mode="seeded", **kw)
+    assert rel_linf(g["u"], ref) <= TOL[dtype]
+    assert np.array_equal(g["hist"], hist)
