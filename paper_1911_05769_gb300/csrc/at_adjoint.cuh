@@ -51,6 +51,7 @@ struct AdjParams {
     // one subdomain per warp (at_adjoint_warp; lambda in lam_a only)
     unsigned char *msg;        // messages between neighbours [kAdjMsgSlots][P][2], zero at the first launch
     int gpl, swz_shift, swz_mask, stage_bytes;   // tile layout, as the stepper's
+    long long stop_below;      // test knob: subdomain 0 takes no step to a level below (0: every step)
 };
 
 template <int ORDER>
@@ -450,6 +451,8 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? 3 : 2) at_adjoint_w
     const T *lev = reinterpret_cast<const T *>(a.levels);
     const int Dl = (int)a.Dl;
     const int n_lev = (int)(a.n_hi - a.n_lo);
+    const long long n_end = p == 0 && a.stop_below > a.n_lo ? a.stop_below : a.n_lo;
+    const int n_run = n_end < a.n_hi ? (int)(a.n_hi - n_end) : 0;       // steps this warp takes
     const unsigned pmask = (unsigned)a.Tp - 1u;
 
     // the pending words of this subdomain
@@ -566,7 +569,8 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? 3 : 2) at_adjoint_w
                 if ((polls & 15) == 15) {
                     const bool late = (long long)(global_ns() - t0) > a.timeout_ns;
                     if (__any_sync(kAll, late || ld_relaxed(a.ctrl + kCtrlAbort) != 0)) {
-                        if (late && miss && my_m == 0) {
+                        // (any lane that misses it reports it: each reads for itself)
+                        if (__any_sync(kAll, late) && miss) {
                             if (atomicCAS(a.ctrl + kCtrlStatus, 0, kStatusTimeout) == 0) {
                                 a.ctrl[kCtrlCta] = (int)blockIdx.x;
                                 a.ctrl[kCtrlWhere] = kWhereAdjoint;
@@ -592,7 +596,7 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? 3 : 2) at_adjoint_w
     bool late_msg = false;              // this face's message of the level before is still to come
     int k_late = 0;                     // the neighbour's delay there
     bool ok = true;
-    for (int i = 0; i < n_lev; ++i) {
+    for (int i = 0; i < n_run; ++i) {
         const long long n = a.n_hi - 1 - i;
         if (i > 0 && (i & 7) == 0) {
             kb = kb_next;
@@ -770,8 +774,8 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? 3 : 2) at_adjoint_w
     }
     // the last level's messages belong to the pending words of the levels below
     if (ok && __any_sync(kAll, late_msg)) {
-        read_msg(late_msg, n_lev - 1);
-        receive(late_msg, n_lev - 1, k_late);
+        read_msg(late_msg, n_run - 1);
+        receive(late_msg, n_run - 1, k_late);
     }
     cp_async_wait(0);
     __syncwarp();

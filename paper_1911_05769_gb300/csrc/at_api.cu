@@ -1741,6 +1741,7 @@ int at_adjoint(at_solver *h, int64_t n_steps, int delay_mode, const int8_t *dela
     a.bar = reinterpret_cast<unsigned long long *>(ws + al.bar);
     a.ctrl = reinterpret_cast<int *>(h->ws + h->lay.ctrl);
     a.timeout_ns = h->g.timeout_ns;
+    if (h->g.flags & AT_FLAG_TEST_SKIP_PUBLISH) a.stop_below = 2 * n_steps - h->g.test_skip_step;
     a.N = h->N; a.P = h->P; a.M = h->M;
     a.L = h->L; a.Tp = h->T;
     if (h->order == 2) {

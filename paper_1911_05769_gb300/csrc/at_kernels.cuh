@@ -982,7 +982,7 @@ __device__ void run_pe(const Params &p, const Sweep &sw, long long lo, int S, un
                 const bool late = (long long)(global_ns() - t0) > p.timeout_ns;
                 if (__any_sync(kAll, late || ld_relaxed(p.ctrl + kCtrlAbort) != 0)) {
                     // (the first lane of a face that is not there reports it)
-                    if (late && !ready && my_m == 0) raise_timeout(p, kWhereFlag, sw.n0 + c.n, h_nb);
+                    if (__any_sync(kAll, late) && !ready && my_m == 0) raise_timeout(p, kWhereFlag, sw.n0 + c.n, h_nb);
                     return false;
                 }
                 if (polls > 64) __nanosleep(64);

@@ -222,7 +222,9 @@ __global__ void __launch_bounds__(256) at_resident(const Params p)
             if ((polls & 15) == 15) {
                 const bool late = (long long)(global_ns() - t0) > p.timeout_ns;
                 if (__any_sync(kAll, late || ld_relaxed(p.ctrl + kCtrlAbort) != 0)) {
-                    if (late && miss && hc == 0) raise_timeout(p, kWhereFlag, n0 + i, nb);
+                    // (any lane that misses its words reports it: the newest
+                    // level may be there and another's half be missing)
+                    if (__any_sync(kAll, late) && miss) raise_timeout(p, kWhereFlag, n0 + i, nb);
                     return false;
                 }
                 if (polls > 256) __nanosleep(64);

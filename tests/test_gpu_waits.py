@@ -61,3 +61,35 @@ def test_one_subdomain_per_cta_leaves_together(P, M, order, dtype, skip):
     ref, hist = oracle_run(u0, mode="seeded", **kw)
     assert rel_linf(g["u"], ref) <= TOL[dtype]
     assert np.array_equal(g["hist"], hist)
+
+
+@pytest.mark.parametrize("P,M,order,dtype", [(2, 64, 2, "f64"), (5, 100, 4, "f64"), (16, 1024, 2, "f32"), (300, 64, 4, "f32")])
+@pytest.mark.parametrize("back", [0, 1, 9])
+def test_adjoint_messages_time_out(P, M, order, dtype, back):
+    """Subdomain 0 stops after `back` backward steps: its neighbours' waits for
+    its messages run out, whether they are due at once (delay 0) or a level
+    later; without the knob the gradient is the oracle's."""
+    from paper_1911_05769_gb300 import AT_ERR_TIMEOUT, AT_FLAG_TEST_SKIP_PUBLISH, AT_OK, AT_SEEDED, Solver, binding as B
+    from test_gpu_adjoint import oracle_adjoint, problem
+    pr = problem(N=P * M, P=P, order=order, L=2, steps=24, nu=0.02 if P * M > 400 else 0.2)
+    pr["dt"] *= 0.5
+    if dtype == "f32":
+        for k in ("u0", "lam_T"):
+            pr[k] = pr[k].astype(np.float32).astype(np.float64)
+    tdt = torch.float64 if dtype == "f64" else torch.float32
+    n, interval = pr["steps"], 10
+    for flags in (AT_FLAG_TEST_SKIP_PUBLISH, 0):
+        s = Solver(pr["N"], P, order, 2, pr["nu"], pr["dt"], dtype=dtype, seed=pr["seed"], flags=flags,
+                   test_skip_step=n + back, timeout_ns=20_000_000 if flags else 0)
+        s.set_state(pr["u0"])
+        ckpt = torch.empty(B.at_checkpoint_bytes(s.h, n, interval), dtype=torch.uint8, device="cuda")
+        assert B.at_step_checkpointed(s.h, n, AT_SEEDED, None, interval, ckpt.data_ptr()) == AT_OK
+        assert s.status() == AT_OK
+        lam = torch.from_numpy(pr["lam_T"]).to(tdt).cuda()
+        nb = B.at_adjoint_workspace_bytes(s.h, interval)
+        ws = torch.empty(nb, dtype=torch.uint8, device="cuda")
+        rc, _ = B.at_adjoint(s.h, n, AT_SEEDED, None, interval, ckpt.data_ptr(), ws.data_ptr(), nb, lam.data_ptr())
+        assert rc == (AT_ERR_TIMEOUT if flags else AT_OK)
+        s.close()
+    _, olam0, _ = oracle_adjoint(pr, mode=oracle.SEEDED)
+    assert rel_linf(lam.double().cpu().numpy(), olam0) <= TOL[dtype]
