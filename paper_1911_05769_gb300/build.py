@@ -25,7 +25,7 @@ SOURCES = [os.path.join(CSRC, f) for f in (
     "at_kernels_f32v.cu", "at_kernels_f32c.cu", "at_batch_f32c.cu", "at_sync_f32.cu", "at_sync_f32v.cu", "at_sync_batch_f32.cu",
     "at_sync_f64.cu", "at_kernels3d.cu", "at_kernels3d_iso.cu", "at_kernels3d_blk.cu", "at_kernels3d_blk32.cu",
     "at_kernels3d_v4.cu", "at_system3d.cu", "at_resident.cu")]
-DEPS = SOURCES + [os.path.join(CSRC, f) for f in ("at_kernels.cuh", "at_device.cuh", "at_adjoint.cuh",
+DEPS = SOURCES + [os.path.join(CSRC, f) for f in ("at_kernels.cuh", "at_device.cuh", "at_items.cuh", "at_adjoint.cuh",
                                                  "at_kernels3d.cuh", "at_kernels3d_blk.cuh", "at_kernels3d_v4.cuh", "at_resident.cuh")] + [
     os.path.join(INCLUDE, "at.h")]
 

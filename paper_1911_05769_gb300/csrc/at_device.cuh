@@ -10,6 +10,8 @@
 
 #include <cstdint>
 
+#include "at_items.cuh"
+
 namespace atk {
 
 // Control block words (the solver's workspace).  kCtrlN0 (64-bit, words 8-9)
@@ -205,25 +207,6 @@ __device__ __forceinline__ void ld_tagged(bool on, const unsigned char *e, unsig
 }
 
 // a word from the L2 cache
-// The contiguous run of `total` items that processor e of n owns: runs differ by
-// one item at most, the last processors have the longer ones.  The CTAs that share
-// an SM are 148 apart in the launch order, but for the first 4 x occupancy of
-// them, which fill 4 SMs by themselves (measured); so consecutive CTAs with one
-// item more land on different SMs, if they are not the first ones.  Cut at
-// e total / n instead, the CTAs of an SM nearly all had the longer run or none of
-// them.  Before and now: 384 x 256 x 288 in 864 subdomains on 608 CTAs, 40 seeded
-// levels 2748 -> 2655 us; 2^22 FP64 points in 4096 subdomains on 1216 warps, 40
-// levels 3632 -> 3544; with the first processors longer 2872 and 4010.
-struct ItemRange {
-    long long lo, hi;
-};
-
-__device__ __forceinline__ ItemRange item_range(long long total, long long n, long long e)
-{
-    const long long q = total / n, few = n - (total - q * n);      // processors with q items
-    return ItemRange{e * q + (e > few ? e - few : 0), (e + 1) * q + (e + 1 > few ? e + 1 - few : 0)};
-}
-
 __device__ __forceinline__ float ld_cg(const float *p) { return __ldcg(p); }
 __device__ __forceinline__ double ld_cg(const double *p) { return __ldcg(p); }
 

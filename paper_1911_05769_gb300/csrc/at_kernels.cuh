@@ -1516,7 +1516,7 @@ __global__ void __launch_bounds__(kThreads, AT_MIN_CTAS_PER_SM) at_stepper(const
             t0 = p.split.tile[g]; t1 = p.split.tile[g + 1];
         }
     }
-    const ItemRange own = item_range(t1 - t0, (long long)(g1 - g0) * kWarps, (long long)((int)blockIdx.x - g0) * kWarps + w);
+    const ItemRange own = cta_items(t1 - t0, g1 - g0, kWarps, (int)blockIdx.x - g0, w);
     const long long lo = t0 + own.lo, hi = t0 + own.hi;
     const long long S = hi - lo;
     unsigned char *raw = smem + p.raw_off + (size_t)w * kRawBytes;

@@ -142,7 +142,7 @@ __global__ void __launch_bounds__(NT * TEAMS, v4_min_ctas(NF, NT * TEAMS))
 
     const int tid = (int)threadIdx.x - team * NT, lane = tid & 31, warp = tid >> 5;   // within the team
     const long long npes = (long long)p.G * TEAMS;
-    const ItemRange own = item_range(p.P, npes, (long long)blockIdx.x * TEAMS + team);
+    const ItemRange own = cta_items(p.P, p.G, TEAMS, blockIdx.x, team);
     const long long lo = own.lo, hi = own.hi;
     const long long S = hi - lo;
     const long long lev0 = *reinterpret_cast<const volatile long long *>(p.ctrl + kCtrlN0);
