@@ -75,8 +75,9 @@ extern "C" {
                                           elements after level test_skip_step, so
                                           that its neighbours' waits time out
                                           (1D: its first warp; 3D: its subdomains;
-                                          at_adjoint: its step to level n is level
-                                          2 n_steps - n of the run) */
+                                          at_adjoint, whose step from level n is level
+                                          2 n_steps - n of the run: subdomain 0 leaves
+                                          out the intervals that start after it) */
 #define AT_FLAG_VISCOUS_FP64        8  /* FP32 state: form the viscous term nu dt D2 u
                                           and add it to u in FP64 (one rounding per
                                           update).  Chosen automatically when

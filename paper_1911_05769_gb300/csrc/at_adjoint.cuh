@@ -51,7 +51,7 @@ struct AdjParams {
     // one subdomain per warp (at_adjoint_warp; lambda in lam_a only)
     unsigned char *msg;        // messages between neighbours [kAdjMsgSlots][P][2], zero at the first launch
     int gpl, swz_shift, swz_mask, stage_bytes;   // tile layout, as the stepper's
-    long long stop_below;      // test knob: subdomain 0 takes no step to a level below (0: every step)
+    long long stop_below;      // test knob: subdomain 0 leaves out intervals that start at or below it (0: none)
 };
 
 template <int ORDER>
@@ -438,6 +438,7 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? 3 : 2) at_adjoint_w
     const long long e = (long long)blockIdx.x * kWarps + w, E = (long long)gridDim.x * kWarps;
     const int p = (int)(e * P / E);
     if ((e + 1) * P / E == p) return;                    // (no subdomain)
+    if (p == 0 && a.n_hi <= a.stop_below) return;
     const int nb = my_face ? (p == P - 1 ? 0 : p + 1) : (p == 0 ? P - 1 : p - 1);   // across this lane's face
     unsigned char *base = smem + (size_t)w * adjoint_warp_smem(a.stage_bytes, kAdjStages, R, (int)sizeof(T), a.Tp);
     unsigned char *raw = base + kAdjStages * a.stage_bytes;
@@ -451,8 +452,6 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? 3 : 2) at_adjoint_w
     const T *lev = reinterpret_cast<const T *>(a.levels);
     const int Dl = (int)a.Dl;
     const int n_lev = (int)(a.n_hi - a.n_lo);
-    const long long n_end = p == 0 && a.stop_below > a.n_lo ? a.stop_below : a.n_lo;
-    const int n_run = n_end < a.n_hi ? (int)(a.n_hi - n_end) : 0;       // steps this warp takes
     const unsigned pmask = (unsigned)a.Tp - 1u;
 
     // the pending words of this subdomain
@@ -596,7 +595,7 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? 3 : 2) at_adjoint_w
     bool late_msg = false;              // this face's message of the level before is still to come
     int k_late = 0;                     // the neighbour's delay there
     bool ok = true;
-    for (int i = 0; i < n_run; ++i) {
+    for (int i = 0; i < n_lev; ++i) {
         const long long n = a.n_hi - 1 - i;
         if (i > 0 && (i & 7) == 0) {
             kb = kb_next;
@@ -774,8 +773,8 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? 3 : 2) at_adjoint_w
     }
     // the last level's messages belong to the pending words of the levels below
     if (ok && __any_sync(kAll, late_msg)) {
-        read_msg(late_msg, n_run - 1);
-        receive(late_msg, n_run - 1, k_late);
+        read_msg(late_msg, n_lev - 1);
+        receive(late_msg, n_lev - 1, k_late);
     }
     cp_async_wait(0);
     __syncwarp();

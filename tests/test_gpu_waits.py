@@ -66,9 +66,9 @@ def test_one_subdomain_per_cta_leaves_together(P, M, order, dtype, skip):
 @pytest.mark.parametrize("P,M,order,dtype", [(2, 64, 2, "f64"), (5, 100, 4, "f64"), (16, 1024, 2, "f32"), (300, 64, 4, "f32")])
 @pytest.mark.parametrize("back", [0, 1, 9])
 def test_adjoint_messages_time_out(P, M, order, dtype, back):
-    """Subdomain 0 stops after `back` backward steps: its neighbours' waits for
-    its messages run out, whether they are due at once (delay 0) or a level
-    later; without the knob the gradient is the oracle's."""
+    """Subdomain 0 leaves out the intervals of 10 levels that start `back` or
+    more backward steps in: its neighbours' waits for its messages run out;
+    without the knob the gradient is the oracle's."""
     from paper_1911_05769_gb300 import AT_ERR_TIMEOUT, AT_FLAG_TEST_SKIP_PUBLISH, AT_OK, AT_SEEDED, Solver, binding as B
     from test_gpu_adjoint import oracle_adjoint, problem
     pr = problem(N=P * M, P=P, order=order, L=2, steps=24, nu=0.02 if P * M > 400 else 0.2)
