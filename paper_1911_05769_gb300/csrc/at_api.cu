@@ -46,7 +46,7 @@ void *atk_adjoint_warp_kernel(int w, int order, int gw, bool full);
 void *atk_stepper3d_kernel(int w, int tc);
 void *atk_stepper3d_iso_kernel(int w, int tc);
 void *atk_system3d_kernel(int w, int tc, int nf);
-void *atk_stepper3d_v4_kernel(int nf, int nt, int tc, int iso);
+void *atk_stepper3d_v4_kernel(int nf, int nt, int tc, int teams, int iso);
 void *atk_init3d_kernel(int w);
 void *atk_stepper3d_blk_kernel(int w, int sb, int iso);
 void *atk_stepper3d_blk32_kernel(int w, int sb, int iso);
@@ -462,7 +462,6 @@ struct at_solver {
     bool has_state;
     int dim;                   // 1 or 3
     Dims3 d3;                  // 3D: extents, subdomains, ring entry size
-    int tc;                    // 3D: columns per thread
     int nt3;                   // 3D: threads per CTA
     CUtensorMap tmap;          // 3D: tensor map of the state (planes of a subdomain, all fields)
     int nf;                    // 3D: fields (1: the scalar equation; 3..5: the system)
@@ -755,45 +754,63 @@ static int create3d(const at_grid *grid, int64_t P, int L, int nf, const double 
     cudaDeviceGetAttribute(&smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
     if (!coop) return fail(AT_ERR_RESIDENCY, "device does not support cooperative launch");
 
-    // FP32 with rows of a power of two of 4-point groups (a row lies in one
-    // warp): the kernel with one or two groups of 4 consecutive columns per
-    // thread, CTAs as small as the plane allows; else 256 threads of 1, 2 or 4
-    // single columns
     const int pw = d.m[0] * d.m[1];
-    const bool v4 = w == 4 && d.m[0] <= 128 && (d.m[0] & (d.m[0] - 1)) == 0;
-    const int groups = pw / 4;
-    const int nt = !v4 ? atk::kThreads3 : groups <= 32 ? 32 : groups <= 64 ? 64 : (groups <= 128 || nf == 1) ? 128 : 256;
-    const int teams = (v4 && nf == 1 && groups <= nt) ? atk::kThreads3 / nt : 1;   // (see at_stepper3d_v4)
-    const int tc = v4 ? (groups > nt ? 2 : 1) : pw <= atk::kThreads3 ? 1 : pw <= 2 * atk::kThreads3 ? 2 : 4;
-    if (nf > 1 && !v4 && tc > 2) return fail(AT_ERR_ARG, "the 3D system needs sub[0] * sub[1] <= 512 (or 1024, FP32)");
     const int sb = grid->steps_per_pass > 0 ? grid->steps_per_pass : 1;
     if (nf > 1 && sb > 1) return fail(AT_ERR_ARG, "the 3D system takes one level per pass");
     // (the scalar equation with equal spacing on the three axes: one
     // coefficient pair, the neighbours summed first)
     const int iso = dx[0] == dx[1] && dx[1] == dx[2];
-    void *kern = v4 ? atk_stepper3d_v4_kernel(nf, nt, tc, iso)
-                 : nf == 1 ? (iso ? atk_stepper3d_iso_kernel(w, tc) : atk_stepper3d_kernel(w, tc))
-                           : atk_system3d_kernel(w, tc, nf);
     // plane buffers: at least 3 (planes z and z+1 in use, one arriving), at most sub[2]
-    int stages = grid->stages > 0 ? grid->stages : 4;
-    if (stages < 3) stages = 3;
-    if (stages > d.m[2]) stages = d.m[2];
-    auto smem_for = [&](int st) {
-        return v4 ? teams * atk::smem3v4_layout(d.m[0], d.m[1], d.m[2], st, nf).total
-                  : atk::smem3_layout(d.m[0], d.m[1], d.m[2], w, st, nf).total;
-    };
-    while (smem_for(stages) > smem_optin && stages > 3) --stages;
-    const long long smem = smem_for(stages);
-    if (smem > smem_optin) return fail(AT_ERR_RESIDENCY, "shared memory %lld exceeds %d", smem, smem_optin);
-    e = allow_smem(kern, smem_optin);
-    if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute");
-    int occ = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, nt * teams, (size_t)smem);
-    if (e != cudaSuccess) return cuda_fail(e, "cudaOccupancyMaxActiveBlocksPerMultiprocessor");
-    int64_t G = grid->max_ctas > 0 ? grid->max_ctas : (int64_t)occ * sms;
-    if (G > P) G = P;
-    if (occ < 1 || (int64_t)occ * sms < G)
-        return fail(AT_ERR_RESIDENCY, "%lld CTAs cannot be co-resident (occupancy %d per SM)", (long long)G, occ);
+    int stages0 = grid->stages > 0 ? grid->stages : 4;
+    if (stages0 < 3) stages0 = 3;
+    if (stages0 > d.m[2]) stages0 = d.m[2];
+
+    // FP32 with rows of a power of two of 4-point groups (a row lies in one
+    // warp): the kernel with one or two groups of 4 consecutive columns per
+    // thread, in CTAs of as many teams as 256 threads hold (see at_stepper3d_v4);
+    // fewer teams where their halos do not fit one CTA (a team's x and y halos grow
+    // with sub[2]: 16 x 16 columns of more than 214 planes) or the caller's CTA
+    // count does not fit the SMs (one team needs no more shared memory than the
+    // other kernel).  Else 256 threads of 1, 2 or 4 single columns (teams 0).
+    const bool v4 = w == 4 && d.m[0] <= 128 && (d.m[0] & (d.m[0] - 1)) == 0;
+    const int groups = pw / 4;
+    const int nt4 = groups <= 32 ? 32 : groups <= 64 ? 64 : (groups <= 128 || nf == 1) ? 128 : 256;
+    const int tc4 = groups > nt4 ? 2 : 1, tc1 = pw <= atk::kThreads3 ? 1 : pw <= 2 * atk::kThreads3 ? 2 : 4;
+    if (nf > 1 && !v4 && tc1 > 2) return fail(AT_ERR_ARG, "the 3D system needs sub[0] * sub[1] <= 512 (or 1024, FP32)");
+    void *kern = nullptr;
+    int nt = 0, stages = 0, occ = 0;
+    int64_t G = 0;
+    long long smem = 0;
+    rc = AT_ERR_RESIDENCY;
+    for (int teams = !v4 ? 0 : (nf == 1 && tc4 == 1) ? atk::kThreads3 / nt4 : 1; rc != AT_OK; teams /= 2) {
+        kern = teams ? atk_stepper3d_v4_kernel(nf, nt4, tc4, teams, iso)
+                     : nf == 1 ? (iso ? atk_stepper3d_iso_kernel(w, tc1) : atk_stepper3d_kernel(w, tc1))
+                               : atk_system3d_kernel(w, tc1, nf);
+        nt = teams ? nt4 * teams : atk::kThreads3;
+        auto smem_for = [&](int st) {
+            return teams ? teams * atk::smem3v4_layout(d.m[0], d.m[1], d.m[2], st, nf).total
+                         : atk::smem3_layout(d.m[0], d.m[1], d.m[2], w, st, nf).total;
+        };
+        stages = stages0;
+        while (smem_for(stages) > smem_optin && stages > 3) --stages;
+        smem = smem_for(stages);
+        if (smem > smem_optin) {
+            rc = fail(AT_ERR_RESIDENCY, "shared memory %lld exceeds %d", smem, smem_optin);
+        } else {
+            e = allow_smem(kern, smem_optin);
+            if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute");
+            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, nt, (size_t)smem);
+            if (e != cudaSuccess) return cuda_fail(e, "cudaOccupancyMaxActiveBlocksPerMultiprocessor");
+            G = grid->max_ctas > 0 ? grid->max_ctas : (int64_t)occ * sms;
+            if (G > P) G = P;
+            rc = occ >= 1 && (int64_t)occ * sms >= G
+                     ? AT_OK
+                     : fail(AT_ERR_RESIDENCY, "%lld CTAs cannot be co-resident (occupancy %d per SM)", (long long)G, occ);
+        }
+        if (teams <= 1) break;
+    }
+    if (rc != AT_OK) return rc;
+    g_err[0] = 0;
 
     at_solver *h = new (std::nothrow) at_solver();
     if (!h) return fail(AT_ERR_ARG, "out of host memory");
@@ -801,8 +818,7 @@ static int create3d(const at_grid *grid, int64_t P, int L, int nf, const double 
     if (h->g.timeout_ns <= 0) h->g.timeout_ns = 1000000000ll;
     h->dim = 3;
     h->d3 = d;
-    h->tc = tc;
-    h->nt3 = nt * teams;
+    h->nt3 = nt;
     h->nf = nf;
     for (int f = 0; f < nf; ++f) h->kappa[f] = kappa[f];
     h->N = (int64_t)nf * d.n[0] * d.n[1] * d.n[2];   // words of the state (all fields)

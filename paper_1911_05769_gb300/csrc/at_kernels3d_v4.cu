@@ -20,11 +20,22 @@ void *v4_system(int nf)
 }
 }  // namespace
 
-// nf fields (1: the scalar equation), teams of nt threads (32, 64, 128, 256; the
-// scalar equation with tc = 2 groups per thread: 128, one team per CTA).
-__attribute__((visibility("hidden"))) void *atk_stepper3d_v4_kernel(int nf, int nt, int tc, int iso)
+// nf fields (1: the scalar equation), CTAs of `teams` teams of nt threads (32, 64,
+// 128, 256; the scalar equation: 1 to 256 / nt teams, with tc = 2 groups per thread
+// one team of 128; the system: one team).
+__attribute__((visibility("hidden"))) void *atk_stepper3d_v4_kernel(int nf, int nt, int tc, int teams, int iso)
 {
     if (nf > 1) return nt == 32 ? v4_system<32>(nf) : nt == 64 ? v4_system<64>(nf) : nt == 128 ? v4_system<128>(nf) : v4_system<256>(nf);
     if (tc == 2) return v4_scalar<128, 2, 1>(iso);
-    return nt == 32 ? v4_scalar<32, 1, 8>(iso) : nt == 64 ? v4_scalar<64, 1, 4>(iso) : v4_scalar<128, 1, 2>(iso);
+    switch (nt * 16 + teams) {
+    case 32 * 16 + 8: return v4_scalar<32, 1, 8>(iso);
+    case 32 * 16 + 4: return v4_scalar<32, 1, 4>(iso);
+    case 32 * 16 + 2: return v4_scalar<32, 1, 2>(iso);
+    case 32 * 16 + 1: return v4_scalar<32, 1, 1>(iso);
+    case 64 * 16 + 4: return v4_scalar<64, 1, 4>(iso);
+    case 64 * 16 + 2: return v4_scalar<64, 1, 2>(iso);
+    case 64 * 16 + 1: return v4_scalar<64, 1, 1>(iso);
+    case 128 * 16 + 2: return v4_scalar<128, 1, 2>(iso);
+    default: return v4_scalar<128, 1, 1>(iso);
+    }
 }

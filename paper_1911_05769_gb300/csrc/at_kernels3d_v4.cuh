@@ -24,8 +24,8 @@
 // The arithmetic is at_stepper3d's, operation by operation.
 //
 // A processing element is a team of NT threads; scalar CTAs hold 256 / NT teams
-// (planes of 1024 points: one of 128), each with its own subdomains, shared
-// memory and named barrier, the system's CTAs one (their shared memory is what
+// (planes of 1024 points: one of 128; long columns fewer, as their halos fit),
+// each with its own subdomains, shared memory and named barrier, the system's CTAs one (their shared memory is what
 // limits them, and it comes in smaller pieces so).
 //
 // Pass times before and after (at_stepper3d, this kernel): 5-field system on
