@@ -771,7 +771,8 @@ static int create3d(const at_grid *grid, int64_t P, int L, int nf, const double 
     // fewer teams where their halos do not fit one CTA (a team's x and y halos grow
     // with sub[2]: 16 x 16 columns of more than 214 planes) or the caller's CTA
     // count does not fit the SMs (one team needs no more shared memory than the
-    // other kernel).  Else 256 threads of 1, 2 or 4 single columns (teams 0).
+    // other kernel; the system's kernel of 256 threads then takes 128 registers, 80 to
+    // 196 bytes spilled, in place of up to 249).  Else 256 threads of 1, 2 or 4 single columns (teams 0).
     const bool v4 = w == 4 && d.m[0] <= 128 && (d.m[0] & (d.m[0] - 1)) == 0;
     const int groups = pw / 4;
     const int nt4 = groups <= 32 ? 32 : groups <= 64 ? 64 : (groups <= 128 || nf == 1) ? 128 : 256;
@@ -781,9 +782,9 @@ static int create3d(const at_grid *grid, int64_t P, int L, int nf, const double 
     int nt = 0, stages = 0, occ = 0;
     int64_t G = 0;
     long long smem = 0;
-    rc = AT_ERR_RESIDENCY;
-    for (int teams = !v4 ? 0 : (nf == 1 && tc4 == 1) ? atk::kThreads3 / nt4 : 1; rc != AT_OK; teams /= 2) {
-        kern = teams ? atk_stepper3d_v4_kernel(nf, nt4, tc4, teams, iso)
+    bool two = false;          // the system's 256-thread kernel in 128 registers: two CTAs an SM
+    for (int teams = !v4 ? 0 : (nf == 1 && tc4 == 1) ? atk::kThreads3 / nt4 : 1;;) {
+        kern = teams ? atk_stepper3d_v4_kernel(nf, nt4, tc4, two ? 2 : teams, iso)
                      : nf == 1 ? (iso ? atk_stepper3d_iso_kernel(w, tc1) : atk_stepper3d_kernel(w, tc1))
                                : atk_system3d_kernel(w, tc1, nf);
         nt = teams ? nt4 * teams : atk::kThreads3;
@@ -807,7 +808,10 @@ static int create3d(const at_grid *grid, int64_t P, int L, int nf, const double 
                      ? AT_OK
                      : fail(AT_ERR_RESIDENCY, "%lld CTAs cannot be co-resident (occupancy %d per SM)", (long long)G, occ);
         }
-        if (teams <= 1) break;
+        if (rc == AT_OK) break;
+        if (teams > 1) teams /= 2;
+        else if (teams && nf > 1 && nt4 == 256 && !two) two = true;
+        else break;
     }
     if (rc != AT_OK) return rc;
     g_err[0] = 0;

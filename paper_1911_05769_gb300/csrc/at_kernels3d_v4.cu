@@ -11,21 +11,23 @@ void *v4_scalar(bool iso)
                : (void *)atk::at_stepper3d_v4<1, false, NT, TC, false, TEAMS>;
 }
 
-template <int NT>
+template <int NT, int CTAS = atk::v4_min_ctas(3, NT)>
 void *v4_system(int nf)
 {
-    return nf == 3 ? (void *)atk::at_stepper3d_v4<3, true, NT, 1, false, 1>
-                   : nf == 4 ? (void *)atk::at_stepper3d_v4<4, true, NT, 1, false, 1>
-                             : (void *)atk::at_stepper3d_v4<5, true, NT, 1, false, 1>;
+    return nf == 3 ? (void *)atk::at_stepper3d_v4<3, true, NT, 1, false, 1, CTAS>
+                   : nf == 4 ? (void *)atk::at_stepper3d_v4<4, true, NT, 1, false, 1, CTAS>
+                             : (void *)atk::at_stepper3d_v4<5, true, NT, 1, false, 1, CTAS>;
 }
 }  // namespace
 
 // nf fields (1: the scalar equation), CTAs of `teams` teams of nt threads (32, 64,
 // 128, 256; the scalar equation: 1 to 256 / nt teams, with tc = 2 groups per thread
-// one team of 128; the system: one team).
+// one team of 128; the system: one team, or with teams = 2 the 256-thread kernel
+// compiled for two CTAs an SM).
 __attribute__((visibility("hidden"))) void *atk_stepper3d_v4_kernel(int nf, int nt, int tc, int teams, int iso)
 {
-    if (nf > 1) return nt == 32 ? v4_system<32>(nf) : nt == 64 ? v4_system<64>(nf) : nt == 128 ? v4_system<128>(nf) : v4_system<256>(nf);
+    if (nf > 1) return nt == 32 ? v4_system<32>(nf) : nt == 64 ? v4_system<64>(nf) : nt == 128 ? v4_system<128>(nf)
+                                : teams == 1 ? v4_system<256>(nf) : v4_system<256, 2>(nf);
     if (tc == 2) return v4_scalar<128, 2, 1>(iso);
     switch (nt * 16 + teams) {
     case 32 * 16 + 8: return v4_scalar<32, 1, 8>(iso);

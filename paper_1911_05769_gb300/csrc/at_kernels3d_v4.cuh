@@ -97,8 +97,8 @@ __host__ __device__ inline Smem3v4 smem3v4_layout(int m0, int m1, int m2, int st
     return l;
 }
 
-template <int NF, bool SYS, int NT, int TC, bool ISO, int TEAMS>
-__global__ void __launch_bounds__(NT * TEAMS, v4_min_ctas(NF, NT * TEAMS))
+template <int NF, bool SYS, int NT, int TC, bool ISO, int TEAMS, int CTAS = v4_min_ctas(NF, NT * TEAMS)>
+__global__ void __launch_bounds__(NT * TEAMS, CTAS)
     at_stepper3d_v4(const Params3 p, const __grid_constant__ CUtensorMap tmap)
 {
     using T = float;

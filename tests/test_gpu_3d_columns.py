@@ -42,3 +42,22 @@ def test_cta_count_of_the_caller():
     s = at.Solver3D((384, 96, 513), (32, 8, 171), 2, 0.1, 1e-7, max_ctas=304)
     assert s.info().ctas == 304
     s.close()
+
+
+@pytest.mark.parametrize("nf", [3, 4, 5])
+def test_two_ctas_of_the_system_to_an_sm(nf):
+    """Planes of 1024 points, more CTAs than SMs."""
+    import paper_1911_05769_gb300 as at
+    from test_gpu_system3d import gpu_system
+    n, sub = (256, 64, 120), (128, 8, 3)
+    q0 = box(n, 5, nf)
+    dx = tuple(2 * np.pi / k for k in n)
+    kappa = [0.05, 0.05, 0.05, 0.02, 0.08][:nf]
+    dt = 0.2 / (2 * 0.08 * sum(1 / d ** 2 for d in dx))
+    kw = dict(L=2, kappa=kappa, dt=dt)
+    s = at.System3D(n, sub, 2, kappa, dt)
+    sms = s.info().sm_count
+    s.close()
+    g = gpu_system(q0, sub=sub, steps=6, dtype="f32", mode=at.AT_SEEDED, seed=7, max_ctas=2 * sms, **kw)
+    ref, _ = oracle.run3d_system(q0, delay_mode=oracle.SEEDED, seed=7, P=(2, 8, 40), n_steps=6, dx=dx, **kw)
+    assert rel_linf(g["q"], ref) <= TOL["f32"]
