@@ -772,12 +772,14 @@ static int create3d(const at_grid *grid, int64_t P, int L, int nf, const double 
     // with sub[2]: 16 x 16 columns of more than 214 planes) or the caller's CTA
     // count does not fit the SMs (one team needs no more shared memory than the
     // other kernel; the system's kernel of 256 threads then takes 128 registers, 80 to
-    // 196 bytes spilled, in place of up to 249).  Else 256 threads of 1, 2 or 4 single columns (teams 0).
+    // 196 bytes spilled, in place of up to 249).  Else 256 threads of 1, 2 or 4
+    // single columns (teams 0).
     const bool v4 = w == 4 && d.m[0] <= 128 && (d.m[0] & (d.m[0] - 1)) == 0;
     const int groups = pw / 4;
     const int nt4 = groups <= 32 ? 32 : groups <= 64 ? 64 : (groups <= 128 || nf == 1) ? 128 : 256;
     const int tc4 = groups > nt4 ? 2 : 1, tc1 = pw <= atk::kThreads3 ? 1 : pw <= 2 * atk::kThreads3 ? 2 : 4;
-    if (nf > 1 && !v4 && tc1 > 2) return fail(AT_ERR_ARG, "the 3D system needs sub[0] * sub[1] <= 512 (or 1024, FP32)");
+    if (nf > 1 && pw > 512 && !(v4 && pw == 1024))
+        return fail(AT_ERR_ARG, "the 3D system needs sub[0] * sub[1] <= 512 (or 1024, FP32)");
     void *kern = nullptr;
     int nt = 0, stages = 0, occ = 0;
     int64_t G = 0;
