@@ -115,8 +115,9 @@ typedef struct at_grid {
   void    *stream;          /* cudaStream_t (NULL = legacy default stream)         */
   int64_t  timeout_ns;      /* bound of every device wait; 0 = 1 s                 */
   int32_t  max_ctas;        /* CTAs: 0 = all that can be resident at once (capped */
-                            /* at P); else this many (AT_ERR_RESIDENCY if they    */
-                            /* cannot all be resident)                            */
+                            /* at P); else this many, or P, or in 1D as many of   */
+                            /* them as can be resident if every subdomain then    */
+                            /* has a warp (else AT_ERR_RESIDENCY)                 */
   int32_t  stages;          /* tile buffers per warp: 0 = 3; at least 2; fewer if */
                             /* shared memory cannot hold them                     */
   int64_t  test_skip_step;  /* level after which AT_FLAG_TEST_SKIP_PUBLISH acts    */

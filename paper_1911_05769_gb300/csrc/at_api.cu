@@ -433,6 +433,24 @@ int launch_shape(int64_t M, int w, int64_t P, TabSize tsz, int max_ctas, int sta
         e = occupancy(sl.total, &occ);
         if (e != cudaSuccess) return cuda_fail(e, "cudaOccupancyMaxActiveBlocksPerMultiprocessor");
     }
+    // a count of the caller's that cannot be resident: as many as can, if they give
+    // every subdomain a warp of its own (more would only spread them further);
+    // else with fewer tile buffers
+    const int asked = G;
+    while (max_ctas > 0 && (int64_t)occ * sms < G) {
+        const int64_t fit = (int64_t)occ * sms;
+        if (occ > 0 && G == asked && fit * atk::kWarps >= P) {
+            G = (int)fit;
+        } else if (stages > atk::kMinStages) {
+            --stages;
+            G = asked;
+        } else {
+            break;
+        }
+        sl = layout_for(G, stages, &smax);
+        e = occupancy(sl.total, &occ);
+        if (e != cudaSuccess) return cuda_fail(e, "cudaOccupancyMaxActiveBlocksPerMultiprocessor");
+    }
     if (occ < 1 || (int64_t)occ * sms < G)
         return fail(AT_ERR_RESIDENCY, "%d CTAs cannot be co-resident (occupancy %d per SM)", G, occ);
     *G_out = G;
