@@ -568,8 +568,9 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? 3 : 2) at_adjoint_w
                 if ((polls & 15) == 15) {
                     const bool late = (long long)(global_ns() - t0) > a.timeout_ns;
                     if (__any_sync(kAll, late || ld_relaxed(a.ctrl + kCtrlAbort) != 0)) {
-                        // (any lane that misses it reports it: each reads for itself)
-                        if (__any_sync(kAll, late) && miss) {
+                        // (any lane that misses it reports it: each reads for itself;
+                        // the first report stands)
+                        if (miss) {
                             if (atomicCAS(a.ctrl + kCtrlStatus, 0, kStatusTimeout) == 0) {
                                 a.ctrl[kCtrlCta] = (int)blockIdx.x;
                                 a.ctrl[kCtrlWhere] = kWhereAdjoint;

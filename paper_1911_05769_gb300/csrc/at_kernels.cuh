@@ -981,8 +981,9 @@ __device__ void run_pe(const Params &p, const Sweep &sw, long long lo, int S, un
             if ((polls & 15) == 15) {
                 const bool late = (long long)(global_ns() - t0) > p.timeout_ns;
                 if (__any_sync(kAll, late || ld_relaxed(p.ctrl + kCtrlAbort) != 0)) {
-                    // (the first lane of a face that is not there reports it)
-                    if (__any_sync(kAll, late) && !ready && my_m == 0) raise_timeout(p, kWhereFlag, sw.n0 + c.n, h_nb);
+                    // (the first lane of a face that is not there reports it; the
+                    // first report stands)
+                    if (!ready && my_m == 0) raise_timeout(p, kWhereFlag, sw.n0 + c.n, h_nb);
                     return false;
                 }
                 if (polls > 64) __nanosleep(64);

@@ -92,11 +92,10 @@ __global__ void __launch_bounds__(256) at_resident(const Params p)
     constexpr int kEnt = kRingHalf * NH;
     constexpr bool PLAIN = sizeof(T) == 4 && ORDER == 2 && !FORCED;     // (as the general stepper)
     __shared__ T s_edge[2][8][2][R];           // [level parity][warp][first | last R words]
-    // [level parity] a wait of the level ran out.  (Two words: with one, a warp
-    // past the level's barrier could set it for the next level before a slower
-    // warp has read it for this one; that warp would leave a barrier early, for
-    // the last ones, which are not bounded.)
-    __shared__ int s_abort[2];
+    // level whose wait ran out.  (With a mere flag, a warp past a level's barrier could
+    // set it for the next level before a slower warp has read it for this one; that
+    // warp would leave a barrier early, for the last ones, which are not bounded.)
+    __shared__ int s_abort;
     __shared__ T s_kt[kMaxL + 1][2];           // k and k (k + 1) / 2 in the state's type
     __shared__ ulonglong2 s_ring[CL ? kClusterSlots * 2 * NH : 1];      // [slot][face][half]: the neighbours' words
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
@@ -126,10 +125,6 @@ __global__ void __launch_bounds__(256) at_resident(const Params p)
     const T cA = sizeof(T) == 4 ? (T)p.cA32 : (T)p.cA, cr = sizeof(T) == 4 ? (T)p.cr32 : (T)p.cr;
     const StencilK<T, ORDER, 0, PLAIN> K(cA, cr, p);
 
-    // (test knob: CTA 0 stops, and so stops publishing, after level skip_step)
-    const long long most = p.skip_publish && pj == 0 ? p.skip_step - n0 : (long long)n_steps;
-    const int n_run = most < 0 ? 0 : most < n_steps ? (int)most : n_steps;
-
     // the state, and the forcing of this thread's points
     T v[PPT], F[FORCED ? PPT : 1];
     T *ug = reinterpret_cast<T *>(p.u) + (size_t)pj * M + tid * PPT;
@@ -153,7 +148,7 @@ __global__ void __launch_bounds__(256) at_resident(const Params p)
         s_kt[tid][0] = (T)tid;
         s_kt[tid][1] = (T)(tid * (tid + 1) / 2);
     }
-    if (tid < 2) s_abort[tid] = 0;
+    if (tid == 0) s_abort = 0x7fffffff;
     if constexpr (CL) {
         // the levels a halo may use that are there already, from the global ring
         // (unread ones empty), before any neighbour stores into this one
@@ -223,8 +218,9 @@ __global__ void __launch_bounds__(256) at_resident(const Params p)
                 const bool late = (long long)(global_ns() - t0) > p.timeout_ns;
                 if (__any_sync(kAll, late || ld_relaxed(p.ctrl + kCtrlAbort) != 0)) {
                     // (any lane that misses its words reports it: the newest
-                    // level may be there and another's half be missing)
-                    if (__any_sync(kAll, late) && miss) raise_timeout(p, kWhereFlag, n0 + i, nb);
+                    // level may be there and another's half be missing; the first
+                    // report stands)
+                    if (miss) raise_timeout(p, kWhereFlag, n0 + i, nb);
                     return false;
                 }
                 if (polls > 256) __nanosleep(64);
@@ -251,8 +247,10 @@ __global__ void __launch_bounds__(256) at_resident(const Params p)
     }
     if (n_warps > 1) put_edges(0);
     __syncthreads();
-    bool ok = true;
-    for (int i = 0; i < n_run; ++i) {
+    // (test knob: CTA 0 takes no part in a launch that goes beyond level skip_step)
+    bool ok = !(p.skip_publish && pj == 0 && n0 + n_steps > p.skip_step);
+    if (ok)
+    for (int i = 0; i < n_steps; ++i) {
         const int par = i & 1;
         // the R words left and right of the warp's run
         T lw[R], rw[R];
@@ -261,8 +259,7 @@ __global__ void __launch_bounds__(256) at_resident(const Params p)
             if ((i & 15) == 8) kb_next = draw((i & ~15) + 16);
             const int k = h_k;
             if (!__all_sync(kAll, !h_act || ht == h_tag)) {
-                ok = wait_entries(i);
-                if (!ok && lane == 0) *reinterpret_cast<volatile int *>(&s_abort[par]) = 1;
+                if (!wait_entries(i)) { ok = false; if (lane == 0) *reinterpret_cast<volatile int *>(&s_abort) = i; }
             }
             if (f == 0 ? w_first : w_last) {
                 cnt_k += hc == k ? 1u : 0u;
@@ -292,7 +289,7 @@ __global__ void __launch_bounds__(256) at_resident(const Params p)
         }
         if (n_warps > 1) {
             __syncthreads();
-            if (*reinterpret_cast<volatile int *>(&s_abort[par])) { ok = false; break; }
+            if (*reinterpret_cast<volatile int *>(&s_abort) <= i) { ok = false; break; }
 #pragma unroll
             for (int q = 0; q < R; ++q) {
                 if (!w_first) lw[q] = s_edge[par][w - 1][1][q];
