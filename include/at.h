@@ -74,7 +74,9 @@ extern "C" {
 #define AT_FLAG_TEST_SKIP_PUBLISH   4  /* test only: CTA 0 stops publishing to other
                                           elements after level test_skip_step, so
                                           that its neighbours' waits time out
-                                          (1D: its first warp; 3D: its subdomains;
+                                          (1D: the element of subdomain 0, with a CTA
+                                          per subdomain it takes no part in launches
+                                          that go beyond; 3D: its subdomains;
                                           at_adjoint, whose step from level n is level
                                           2 n_steps - n of the run: subdomain 0 leaves
                                           out the intervals that start after it) */

@@ -377,10 +377,8 @@ int launch_shape(int64_t M, int w, int64_t P, TabSize tsz, int max_ctas, int sta
         const int gw = groups_per_lane(M);
         return atk::smem_layout(atk::tile_points(M, gw, full_runs(M, gw)), w, st, tab, tsz.comp);
     };
-    // at most one CTA per subdomain: with few subdomains every CTA holds one
-    // (spread over the SMs, so that the subdomains share no SM's pipes) instead
-    // of kWarps (16 subdomains of 256 FP64 points: 0.5 us of FP64 pipe a step
-    // on 16 SMs, 2 us on 4).
+    // at most one CTA per subdomain (FP64: 16 subdomains of 256 points take 0.5 us of
+    // FP64 pipe a step on 16 SMs, 2 us on 4)
     const int gmax = (int)(P < (1LL << 30) ? P : (1LL << 30));
     int G = max_ctas > 0 ? max_ctas : sms;
     if (G > gmax) G = gmax;
@@ -429,6 +427,15 @@ int launch_shape(int64_t M, int w, int64_t P, TabSize tsz, int max_ctas, int sta
         }
         if (e != cudaSuccess) return cuda_fail(e, "cudaOccupancyMaxActiveBlocksPerMultiprocessor");
         if (Gs > 0) G = Gs;
+        // FP64, one subdomain per warp at most: no more CTAs than give every subdomain a
+        // warp with the SMs evenly loaded.  More of them cost a forced run its start, in
+        // which each forms its sin/cos tables (600 subdomains of 1024 points on 304 and
+        // 152 CTAs: 39.1 and 31.0 us for one level, 882 and 868 for 64; 1000 of 256 on 250
+        // and 304: 18.7 us both, 430 and 378).  (FP32 leaves the spare CTAs empty, see
+        // at_stepper.)
+        const int64_t sm_warps = (int64_t)atk::kWarps * sms;
+        if (w == 8 && !tsz.ntk && P <= (int64_t)G * atk::kWarps && (P + sm_warps - 1) / sm_warps * sms < G)
+            G = (int)((P + sm_warps - 1) / sm_warps * sms);
         sl = layout_for(G, stages, &smax);
         e = occupancy(sl.total, &occ);
         if (e != cudaSuccess) return cuda_fail(e, "cudaOccupancyMaxActiveBlocksPerMultiprocessor");
@@ -516,13 +523,32 @@ cudaLaunchAttribute cluster_attr(int n)
     return a;
 }
 
+// Whether a launch of n_steps levels goes to the resident kernel, where there is one
+// (see prepare_resident).  A forced run's CTAs form the sin/cos of their points when
+// they start, and the resident kernel has a CTA per subdomain, R of them to an SM:
+// 8 ns a point and CTA more than the general kernel's, made up for by 0.3 us a level
+// in FP32 and in FP64 by 1.4 us or more, unless R is large.  1000 subdomains of 1024
+// FP32 points: 67.8 us for one level and 135 for 64, in the general kernel 26.9 and
+// 112.9; 300 of 1024: 24.8 and 76.2, 17.3 and 92.1; 600 of 64: 10.5 and 58.0, 8.6 and
+// 84.8.  FP64, 600 of 1024: 53.5 and 864, 31.0 and 845; 300 of 256: 14.4 and 161, 13.3
+// and 264.  (Both kernels give the same bits and may take turns.)
+bool takes_resident(const at_solver *h, const atk::Params *p)
+{
+    if (!h->kernel_res || p->sb != 1 || (p->mode != AT_SEEDED && p->mode != AT_REPLAY)) return false;
+    if (h->g.forcing_amp == 0.0) return true;
+    const int64_t sms = h->sm_count, filled = (h->P + atk::kWarps - 1) / atk::kWarps;
+    const int64_t R = (h->P + sms - 1) / sms, general = ((filled < h->G ? filled : h->G) + sms - 1) / sms;
+    return p->n_steps >= (h->w == 4 ? h->M * (R - general) / 37 : h->M * (R - 2) / 176);
+}
+
 // One launch of the persistent stepper: cooperative, so that every CTA is
 // resident; cudaLaunchKernelExC with the cooperative attribute may be
 // captured into a CUDA graph.  (Ring entries carry their levels, so a launch
 // may partition the subdomains into PEs differently from the one before.)
 cudaError_t launch_stepper(at_solver *h, atk::Params *p, void *kernel)
 {
-    const bool res = h->kernel_res && p->sb == 1 && (p->mode == AT_SEEDED || p->mode == AT_REPLAY);
+    const bool res = takes_resident(h, p);
+    p->G = h->G;
     if (res) {
         kernel = h->kernel_res;
         p->G = (int)h->P;

@@ -810,7 +810,7 @@ __device__ void run_pe(const Params &p, const Sweep &sw, long long lo, int S, un
     const unsigned tmask = (unsigned)p.T - 1u;
     const unsigned n0lo = (unsigned)sw.n0;
     const unsigned long long tag0 = entry_tag(sw.n0);    // tag of relative level 0
-    const bool stop_pub = p.skip_publish && blockIdx.x == 0 && threadIdx.x < 32;   // (test knob)
+    const bool stop_pub = p.skip_publish && lo == 0;   // (test knob: the first tile's owner)
     const T fX = sizeof(T) == 4 ? (T)p.fX32 : (T)p.fX;
     const int err_off = p.stage_bytes / 2;               // (compensated state: the error words of a tile)
     const Swizzle swz = FULL ? Swizzle::of(NCH) : Swizzle{p.swz_shift, p.swz_mask};
@@ -1517,7 +1517,12 @@ __global__ void __launch_bounds__(kThreads, AT_MIN_CTAS_PER_SM) at_stepper(const
             t0 = p.split.tile[g]; t1 = p.split.tile[g + 1];
         }
     }
-    const ItemRange own = cta_items(t1 - t0, g1 - g0, kWarps, (int)blockIdx.x - g0, w);
+    // (fewer tiles than warps: FP64 spreads them over the CTAs, whose SMs' pipes set its
+    // pace; FP32 fills the last CTAs with them, whose neighbours are then near.  100
+    // subdomains of 256 points in passes of 4: FP32 0.45 us a level on 25 SMs, 0.54 on
+    // 100; FP64, 600 of 1000: 23.8 us a level on 75 SMs, 12.8 on 152.)
+    const long long G = g1 - g0, g = (int)blockIdx.x - g0;
+    const ItemRange own = sizeof(T) == 8 ? cta_items(t1 - t0, G, kWarps, g, w) : item_range(t1 - t0, G * kWarps, g * kWarps + w);
     const long long lo = t0 + own.lo, hi = t0 + own.hi;
     const long long S = hi - lo;
     unsigned char *raw = smem + p.raw_off + (size_t)w * kRawBytes;
@@ -1536,7 +1541,8 @@ __global__ void __launch_bounds__(kThreads, AT_MIN_CTAS_PER_SM) at_stepper(const
     __shared__ int s_count;                   // grid-barrier arrivals of this CTA's warps
     __shared__ long long s_epoch;             // last grid barrier this CTA passed
     if (threadIdx.x == 0) { s_count = 0; s_epoch = 0; }
-    if (FORCED) {
+    // (a CTA without subdomains forms no tables: 8 us of an SM's FP64 pipe at M = 1024)
+    if (FORCED && __syncthreads_or(S > 0)) {
         // sin/cos of the offsets j dx within a subdomain and of the subdomain
         // origins x0 + p M dx (FP64), so that A sin(x_i) needs two FMAs
         for (long long i = threadIdx.x; i < p.M; i += blockDim.x) {

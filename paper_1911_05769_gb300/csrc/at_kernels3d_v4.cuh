@@ -54,9 +54,10 @@ constexpr long long kGraceNs = 20000;
 
 // grid barrier before level `step` (1-based within the launch), one arrival per
 // team that has subdomains (npe of them); bounded.  Returns false on abort.
-template <typename Sync, typename Any>
-__device__ bool team_grid_sync(const Params3 &p, long long step, long long npe, int ttid, volatile int *s_flag, Sync sync,
-                               Any any)
+// (The flag may be tested behind the last barrier here: a synchronous run sets it
+// again only behind the tile's next one.)
+template <typename Sync>
+__device__ bool team_grid_sync(const Params3 &p, long long step, long long npe, int ttid, volatile int *s_flag, Sync sync)
 {
     sync();
     if (ttid == 0) {
@@ -70,7 +71,8 @@ __device__ bool team_grid_sync(const Params3 &p, long long step, long long npe, 
         }
         __threadfence();
     }
-    return !any(*s_flag == -1);
+    sync();
+    return *s_flag != -1;
 }
 
 // Shared memory of a team: stage barriers and counters, delay counters, the
@@ -265,7 +267,7 @@ __global__ void __launch_bounds__(NT * TEAMS, CTAS)
             release(prev_sub, prev_new);
         }
         if (p.mode == kModeSync && sub == lo && lv > lev0) {
-            if (!team_grid_sync(p, lv - lev0, p.P < npes ? p.P : npes, tid, s_flag, sync, any)) { ok = false; break; }
+            if (!team_grid_sync(p, lv - lev0, p.P < npes ? p.P : npes, tid, s_flag, sync)) { ok = false; break; }
         }
         const unsigned us = (unsigned)sub, us2 = us / uP01, usr = us - us2 * uP01, us1 = usr / uP0;
         const long long s0 = usr - us1 * uP0, s1 = us1, s2 = us2;

@@ -1,7 +1,6 @@
-"""Fewer subdomains than processing elements: the first CTA has a subdomain like
-every other (it is the one whose elements stop publishing under the failure
-knob, so that its neighbours' bounded waits run out), and runs agree with the
-oracle."""
+"""Fewer subdomains than processing elements: the failure knob finds the element of
+the first one (in 3D: the first CTA has a subdomain like every other), so that
+its neighbours' bounded waits run out, and runs agree with the oracle."""
 import numpy as np
 import pytest
 import torch
@@ -17,7 +16,7 @@ pytestmark = pytest.mark.gpu
 
 @pytest.mark.parametrize("P,M,dtype", [(2, 64, "f64"), (16, 256, "f64"), (150, 64, "f32"), (600, 64, "f64")])
 @pytest.mark.parametrize("spp", [1, 3])
-def test_first_cta_takes_part(P, M, dtype, spp):
+def test_first_element_is_found(P, M, dtype, spp):
     import paper_1911_05769_gb300 as at
     u0 = W.u0_two_modes(P * M)
     _, dx = W.grid(P * M)
