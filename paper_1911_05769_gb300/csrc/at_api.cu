@@ -1087,13 +1087,12 @@ static atk::Params make_params(const at_solver *h)
         p.cB = h->nu * h->dt / (12.0 * h->dx * h->dx);
     }
     p.cr = (h->order == 2 ? 2.0 : 1.0) * h->nu / h->dx;
-    const bool dtA = h->v64 || h->comp;
-    p.fX = dtA ? h->dt * h->g.forcing_amp : (h->order == 2 ? 2.0 : 12.0) * h->dx * h->g.forcing_amp;
+    p.fX = h->v64 ? h->dt * h->g.forcing_amp : (h->order == 2 ? 2.0 : 12.0) * h->dx * h->g.forcing_amp;
     p.cA32 = (float)p.cA;
     p.cB32 = (float)p.cB;
     // (the factors of the rounded cA: their products with it are rounded once)
     p.cr32 = (float)(p.cB / (double)p.cA32);
-    p.fX32 = (float)(dtA ? p.fX : h->dt * h->g.forcing_amp / (double)p.cA32);
+    p.fX32 = (float)(h->v64 ? p.fX : h->dt * h->g.forcing_amp / (double)p.cA32);
     p.gpl = h->gpl;
     const atk::Swizzle swz = atk::Swizzle::of(h->gpl * h->w / 4);
     p.swz_shift = swz.shift;
@@ -1497,9 +1496,9 @@ int at_create_batch(const at_grid *grid, int64_t n_inst, const at_instance *inst
             b = atk::BatchSub{};
             const double cB = a.nu * a.dt / ((scheme_order == 2 ? 1.0 : 12.0) * dx * dx);
             b.cA = a.dt / ((scheme_order == 2 ? 2.0 : 12.0) * dx);
-            b.cr = comp ? cB : (scheme_order == 2 ? 2.0 : 1.0) * a.nu / dx;
+            b.cr = (scheme_order == 2 ? 2.0 : 1.0) * a.nu / dx;
             b.cA32 = (float)b.cA;
-            b.cr32 = (float)(comp ? cB : cB / (double)b.cA32);
+            b.cr32 = (float)(cB / (double)b.cA32);
             b.seed = a.seed;
             b.L = a.L;
             b.lp = (int)lp;

@@ -135,7 +135,7 @@ __host__ __device__ inline unsigned long long entry_tag(long long level) { retur
 // One record per subdomain (built on the host, copied to shared memory by the
 // PE that owns it) and one per problem instance.
 struct BatchSub {
-    double cA, cr;             // stencil factors of the instance (as Params::cA, cr; compensated state: cA, cB)
+    double cA, cr;             // stencil factors of the instance (as Params::cA, cr)
     unsigned long long seed;   // AT_SEEDED seed of the instance
     int L;                     // delay bound of the instance
     int lp;                    // index of the subdomain within its instance
@@ -202,7 +202,7 @@ struct Params {
                                // synchronous mode, where k = 0 and the ghost cells are recomputed)
     unsigned long long seed;
     double cA, cB, cr;         // dt/(2dx) | dt/(12dx);  nu dt/dx^2 | nu dt/(12dx^2);  cB / cA
-    double fX;                 // forcing factor: A dt (FP64 viscous term, compensated state), else A dt / cA
+    double fX;                 // forcing factor: A dt (FP64 viscous term), else A dt / cA
     float cA32, cB32, cr32, fX32;   // the same in FP32 (no conversion per tile)
     double x0, dx;
     int G;                     // CTAs
@@ -397,10 +397,16 @@ __device__ __forceinline__ T forcing_point(T fs, T fc, T sv, T cv)
 // points takes as many.  In FP32 it loses: there the last addition's rounding
 // decides, and over runs of hundreds of steps the sums' own rounding breaks up
 // its bias -- error against 64 bits 2.2e-6 against 2.9e-6 with exact differences.)
-//   Compensated state: the differences word by word, hi and lo, first
-// differences d_i = u_{i+1} - u_i and second ones e_i = d_i - d_{i-1} formed once
-// for the points that share them: a = 6 (d_i + d_{i-1}) - (e_{i+1} - e_{i-1}), b =
-// 14 e_i - (e_{i+1} + e_{i-1}); the factors as cB b - cA u a, each rounded once.
+//   Compensated state: the differences word by word, first differences d_i = u_{i+1}
+// - u_i and second ones e_i = d_i - d_{i-1} formed once for the points that share
+// them: a = 6 (d_i + d_{i-1}) - (e_{i+1} - e_{i-1}), b = 14 e_i - (e_{i+1} + e_{i-1}).
+// Those of the hi words are exact, and stay apart from those of the lo words until the
+// last fused multiply-adds (joined before, the sums' roundings counted 6- and 14-fold:
+// RMS error up to 1.7 times this one at order 4 and steps of 3e-8 to 1e-7).  The
+// increment is formed apart from lo and meets it in one rounding, by the last factor's
+// multiply-add: increments are often smaller than lo there, and added to it term by
+// term they were rounded at its magnitude two or three times (1.02 to 2 times the
+// error at steps of 1e-8 and less).
 //
 // Every operation is written as the one instruction it is, so that a point
 // computed twice -- by its owner in group(), by a neighbour as a ghost cell in
@@ -416,17 +422,16 @@ struct StencilK {
     static constexpr bool WINDOW = PREC != 2;   // from the values of a window
     T cA, cr, cB;
     double cB64;
-    // (cr_: cr; a compensated state: cB)
     __device__ __forceinline__ StencilK(T cA_, T cr_, const Params &p)
-        : cA(cA_), cr(cr_), cB(PREC == 2 ? cr_ : (T)p.cB32), cB64(p.cB)
+        : cA(cA_), cr(cr_), cB((T)p.cB32), cB64(p.cB)
     {
     }
 
     // what a lane carries from point to point
     struct Carry {
         T w[2];                        // WINDOW: the R words left of the point
-        T d0, d1, e0, e1;              // else d_{i-1}, d_i (order 2: d0 = d_{i-1}) of the hi words; e_{i-1}, e_i
-        T l0, l1, g0;                  // the differences of the lo words; d_{i-1} + its lo
+        T d0, d1, l0, l1;              // else d_{i-1}, d_i of the hi words and of the lo words (order 2: d_{i-1})
+        T eh, el, e0, e1;              // e_i of the hi words, of the lo words; e_{i-1}, e_i (their sums)
     };
 
     // cr b - u a + F / cA
@@ -484,7 +489,6 @@ struct StencilK {
         } else if constexpr (ORDER == 2) {
             y.d0 = c[0] - lw[0];
             y.l0 = cl[0] - lwl[0];
-            y.g0 = y.d0 + y.l0;
         } else {
             const T dm = lw[R - 1] - lw[0], lm = lwl[R - 1] - lwl[0];
             y.d0 = c[0] - lw[R - 1];
@@ -492,8 +496,9 @@ struct StencilK {
             y.l0 = cl[0] - lwl[R - 1];
             y.l1 = cl[1] - cl[0];
             y.e0 = (y.d0 - dm) + (y.l0 - lm);
-            y.e1 = (y.d1 - y.d0) + (y.l1 - y.l0);
-            y.g0 = y.d0 + y.l0;
+            y.eh = y.d1 - y.d0;
+            y.el = y.l1 - y.l0;
+            y.e1 = y.eh + y.el;
         }
     }
 
@@ -527,27 +532,26 @@ struct StencilK {
                 T a, b;
                 if constexpr (ORDER == 2) {
                     const T dn = v[e + 1] - cc, ln = vl[e + 1] - vl[e];
-                    const T gn = dn + ln;
                     b = (dn - y.d0) + (ln - y.l0);
-                    a = gn + y.g0;
-                    y.l0 = ln;
-                    y.g0 = gn;
+                    a = (dn + y.d0) + (ln + y.l0);
                     y.d0 = dn;
+                    y.l0 = ln;
                 } else {
                     const T dn = v[e + 2] - v[e + 1], ln = vl[e + 2] - vl[e + 1];
-                    const T gn = y.d1 + y.l1, s = gn + y.g0;
-                    const T en = (dn - y.d1) + (ln - y.l1);
-                    a = fma((T)6, s, -(en - y.e0));
-                    b = fma((T)14, y.e1, -(en + y.e0));
-                    y.l1 = ln;
-                    y.g0 = gn;
+                    const T hn = dn - y.d1, kn = ln - y.l1, en = hn + kn;
+                    a = fma((T)6, y.d1 + y.d0, fma((T)6, y.l1 + y.l0, -(en - y.e0)));
+                    b = fma((T)14, y.eh, fma((T)14, y.el, -(en + y.e0)));
+                    y.d0 = y.d1;
                     y.d1 = dn;
+                    y.l0 = y.l1;
+                    y.l1 = ln;
+                    y.eh = hn;
+                    y.el = kn;
                     y.e0 = y.e1;
                     y.e1 = en;
                 }
                 // two-sum of hi and (increment + lo): exact sum t + err
-                T yy = fma(-(cA * cc), a, fma(cB, b, vl[e]));
-                if constexpr (FORCED) yy = yy + F[FORCED ? e : 0];
+                const T yy = fma(cA, increment(cc, a, b, FORCED ? F[FORCED ? e : 0] : (T)0, FORCED), vl[e]);
                 const T t = cc + yy;
                 const T z = t - cc;
                 cl[e] = (cc - (t - z)) + (yy - z);
@@ -1100,7 +1104,7 @@ __device__ void run_pe(const Params &p, const Sweep &sw, long long lo, int S, un
     bool turn = false;                 // tile r continues tile r-1 in registers
     T c[NPT];                          // this lane's points
     T er[COMP ? NPT : 1];              // compensated state: carried rounding errors
-    T F[FORCED ? NPT : 1];             // forcing (PREC 0: dt A sin x / cA; else dt A sin x)
+    T F[FORCED ? NPT : 1];             // forcing (PREC 1: dt A sin x; else dt A sin x / cA)
 
     for (unsigned r = 0; C.n < sw.n_steps && ok; ++r) {
         // state copy of tile r + D (stage of tile r - 1, written back)
@@ -1126,7 +1130,7 @@ __device__ void run_pe(const Params &p, const Sweep &sw, long long lo, int S, un
         const int n = C.n, len = C.len;                   // level at the pass start
         const int s0 = ti.s0, s1 = ti.s0 + ti.cnt - 1;    // its first and last subdomain
         T cA = sizeof(T) == 4 ? (T)p.cA32 : (T)p.cA;
-        T cr = COMP ? (T)p.cB32 : sizeof(T) == 4 ? (T)p.cr32 : (T)p.cr;
+        T cr = sizeof(T) == 4 ? (T)p.cr32 : (T)p.cr;
         bool bnd0 = false, bnd1 = false;
         if constexpr (BATCH) {
             const BatchSub &bf = rec_first(ti), &bl = rec_last(ti);
@@ -1502,8 +1506,16 @@ __device__ void run_pe(const Params &p, const Sweep &sw, long long lo, int S, un
 // ---------------------------------------------------------------------------
 // the persistent kernel
 // ---------------------------------------------------------------------------
+// (a compensated state in short runs: three CTAs an SM in 168 registers, which are a
+// few short of what two groups a lane would take: 4800 subdomains of 256 points 5.0
+// us a seeded level, 6.1 with two)
+constexpr int stepper_min_ctas(int prec, int gw)
+{
+    return prec == 2 && gw <= 2 && AT_MIN_CTAS_PER_SM < 3 ? 3 : AT_MIN_CTAS_PER_SM;
+}
+
 template <typename T, int ORDER, int GW, bool FORCED, bool FULL, bool BATCH, int PREC, bool BS>
-__global__ void __launch_bounds__(kThreads, AT_MIN_CTAS_PER_SM) at_stepper(const Params p)
+__global__ void __launch_bounds__(kThreads, stepper_min_ctas(PREC, GW)) at_stepper(const Params p)
 {
     extern __shared__ __align__(128) unsigned char smem[];
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
