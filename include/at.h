@@ -145,7 +145,11 @@ typedef struct at_grid {
                             /* multiple of sub[a]; P = product of n[a] / sub[a]   */
 } at_grid;
 
-/* Launch facts of a solver, for tests and benchmarks. */
+/* Launch facts of a solver, for tests and benchmarks.  ctas, threads, stages and
+ * smem_bytes are those of the general stepper.  Plain 1D runs with prescribed
+ * delays (AT_SEEDED, AT_REPLAY; max_ctas 0) whose subdomains each find a resident
+ * CTA take a kernel of P CTAs of M / 8 to M threads without tile buffers, unless a
+ * forced call is short or at_tune found it slower; the results are the same. */
 typedef struct at_info {
   int64_t N, P, M;          /* points, subdomains, points per subdomain            */
   int32_t order, L;         /* stencil order, maximal delay                        */
@@ -329,9 +333,14 @@ int at_create_batch(const at_grid *grid, int64_t n_inst, const at_instance *inst
  * 1 .. L + 1 (in an ensemble each processing element then takes at most its
  * own smallest delay bound + 1); for AT_SYNC 1 .. L + 1 only if the solver
  * was created with steps_per_pass > 1 (the blocked synchronous mode), else 1.
+ * For AT_SEEDED also the kernel of one subdomain per CTA that runs with
+ * prescribed delays take where every subdomain finds a resident CTA (at_info):
+ * it has no shape to choose and is timed as one more.
  * --------------------------------------------------------------------------- */
 typedef struct at_tune_result {
-  int32_t ctas, stages, steps_per_pass;   /* the fastest shape                     */
+  int32_t ctas, stages, steps_per_pass;   /* the fastest shape (if the kernel of   */
+                                          /* one subdomain per CTA was: the shape   */
+                                          /* that the other modes keep)            */
   int32_t n_tried;                        /* shapes timed                          */
   double  best_ms;                        /* its time for at_step(n_steps)          */
   double  first_ms;                       /* time of the shape the solver had      */

@@ -507,6 +507,7 @@ struct at_solver {
     int G_b3, stages_b3, smem_b3;   // 3D: its CTAs, plane stages and shared memory
     void *kernel_res;          // 1D: the one-subdomain-per-CTA kernel of prescribed delays (NULL: none)
     bool res_cluster = false;  // ... whose CTAs are one cluster
+    bool general_only = false; // at_tune found the general kernel faster than it
     bool bs_ok;                // it can run in the launch shape chosen for `kernel`
     void *init_kernel;
 };
@@ -532,13 +533,13 @@ cudaLaunchAttribute cluster_attr(int n)
 // 112.9; 300 of 1024: 24.8 and 76.2, 17.3 and 92.1; 600 of 64: 10.5 and 58.0, 8.6 and
 // 84.8.  FP64, 600 of 1024: 53.5 and 864, 31.0 and 845; 300 of 256: 14.4 and 161, 13.3
 // and 264.  (Both kernels give the same bits and may take turns.)
-bool takes_resident(const at_solver *h, const atk::Params *p)
+bool takes_resident(const at_solver *h, int mode, int sb, int64_t n_steps)
 {
-    if (!h->kernel_res || p->sb != 1 || (p->mode != AT_SEEDED && p->mode != AT_REPLAY)) return false;
+    if (!h->kernel_res || h->general_only || sb != 1 || (mode != AT_SEEDED && mode != AT_REPLAY)) return false;
     if (h->g.forcing_amp == 0.0) return true;
     const int64_t sms = h->sm_count, filled = (h->P + atk::kWarps - 1) / atk::kWarps;
     const int64_t R = (h->P + sms - 1) / sms, general = ((filled < h->G ? filled : h->G) + sms - 1) / sms;
-    return p->n_steps >= (h->w == 4 ? h->M * (R - general) / 37 : h->M * (R - 2) / 176);
+    return n_steps >= (h->w == 4 ? h->M * (R - general) / 37 : h->M * (R - 2) / 176);
 }
 
 // One launch of the persistent stepper: cooperative, so that every CTA is
@@ -547,7 +548,7 @@ bool takes_resident(const at_solver *h, const atk::Params *p)
 // may partition the subdomains into PEs differently from the one before.)
 cudaError_t launch_stepper(at_solver *h, atk::Params *p, void *kernel)
 {
-    const bool res = takes_resident(h, p);
+    const bool res = takes_resident(h, p->mode, p->sb, p->n_steps);
     p->G = h->G;
     if (res) {
         kernel = h->kernel_res;
@@ -1598,7 +1599,7 @@ int at_tune(at_solver *h, int64_t n_steps, int delay_mode, at_tune_result *res)
         const int r = launch_shape((int64_t)kt * h->M, h->w, h->P, tsz, sh.G, sh.stages, true, h->sm_count,
                                    h->smem_optin, h->kernel, &G, &st, &sl, &smem, &smax);
         if (r != AT_OK) return r;
-        if (st != sh.stages) return AT_ERR_RESIDENCY;   // did not fit as asked
+        if (st != sh.stages || G < (sh.G < h->P ? sh.G : h->P)) return AT_ERR_RESIDENCY;   // did not fit as asked
         h->G = G; h->stages = st; h->sl = sl; h->smem = smem; h->smax = smax; h->sb = sh.sb;
         int64_t most = 0;
         h->split = split_tiles(groups, G, &most);
@@ -1630,9 +1631,24 @@ int at_tune(at_solver *h, int64_t n_steps, int delay_mode, at_tune_result *res)
     const Shape orig{h->G, h->stages, h->sb, h->batch ? h->K : 1};
     Shape best = orig;
     double best_ms = 0.0;
+    // (prescribed delays: the resident kernel, which has no shape to choose, against
+    // the shapes of the general one; with general_only set earlier, once more)
+    const bool was_general = h->general_only, prescribed = delay_mode == AT_SEEDED && h->kernel_res;
+    bool best_res = takes_resident(h, delay_mode, 1, n_steps);
+    const bool first_res = best_res;
     int rc = time_shape(&best_ms);
     int tried = 1;
     res->first_ms = best_ms;
+    h->general_only = false;
+    bool timed_res = first_res;
+    if (rc == AT_OK && !first_res && takes_resident(h, delay_mode, 1, n_steps)) {
+        double ms = 0.0;
+        rc = time_shape(&ms);
+        ++tried;
+        timed_res = true;
+        if (rc == AT_OK && ms < best_ms) { best_ms = ms; best_res = true; }
+    }
+    h->general_only = prescribed;
     // levels per pass: up to the largest delay bound + 1 (an ensemble's PEs
     // clamp it to their own smallest bound + 1); the synchronous mode keeps
     // one level per pass unless the solver was made for blocked passes
@@ -1652,20 +1668,22 @@ int at_tune(at_solver *h, int64_t n_steps, int delay_mode, at_tune_result *res)
                 lastG = G;
                 for (int sb = 1; rc == AT_OK && sb <= sb_hi; ++sb) {
                     const Shape sh{G, st, sb, h->batch ? K : 1};
-                    if (sh.G == orig.G && sh.stages == orig.stages && sh.sb == orig.sb && sh.K == orig.K) continue;
+                    if (sh.G == orig.G && sh.stages == orig.stages && sh.sb == orig.sb && sh.K == orig.K && !first_res)
+                        continue;
                     const int ra = apply(sh);
                     if (ra == AT_ERR_CUDA) { rc = ra; break; }
                     if (ra != AT_OK) { g_err[0] = 0; continue; }   // not resident: skip
                     double ms = 0.0;
                     rc = time_shape(&ms);
                     ++tried;
-                    if (rc == AT_OK && ms < best_ms) { best_ms = ms; best = sh; }
+                    if (rc == AT_OK && ms < best_ms) { best_ms = ms; best = sh; best_res = false; }
                 }
             }
         }
     }
     for (int i = 0; i < 3; ++i) cudaEventDestroy(ev[i]);
-    const int rc_apply = apply(rc == AT_OK ? best : orig);
+    h->general_only = rc != AT_OK || !timed_res ? was_general : !best_res;
+    const int rc_apply = apply(rc == AT_OK && !best_res ? best : orig);
     if (rc != AT_OK) return rc;
     if (rc_apply != AT_OK) return rc_apply;
     res->ctas = h->G;
