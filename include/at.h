@@ -66,6 +66,8 @@ extern "C" {
                      /* with steps_per_pass > 1: every pass (ghost cells)     */
 #define AT_SEEDED 1  /* k prescribed by SplitMix64(seed) per (n, p, face)      */
 #define AT_FREE   2  /* k = how far the neighbour lags, waiting only if > L    */
+                     /* (3D, FP32, one level per pass: at most 20 us a face   */
+                     /* for a neighbour that lags less, see the 3D section)   */
 #define AT_REPLAY 3  /* k read from a caller array                             */
 
 /* at_grid.flags */
@@ -246,7 +248,11 @@ const char *at_last_error(void);
  * levels n-k, n-k-1 of the neighbouring subdomain (Eq. AT1/AT2) with a delay
  * per (level, subdomain, face); AT_SEEDED draws it at counter (n P + p) 6 +
  * face.  at_create's P must equal the number of subdomains; scheme_order must
- * be 2.  The delay arrays of at_step are [n_steps][P][6].  Stability limit
+ * be 2.  The delay arrays of at_step are [n_steps][P][6].  AT_FREE with FP32
+ * state, sub[0] a power of two and one level per pass gives a neighbour that
+ * lags by at most L up to 20 us to bring level n itself before it takes the
+ * delay: delays and their error are smaller, a neighbour later than that
+ * still holds nobody up.  FP64 and other rows never wait within L.  Stability limit
  * for at_create: nu dt (1/dx^2 + 1/dy^2 + 1/dz^2) <= 1/2.
  * Temporal blocking (scalar equation, AT_FREE): grid->steps_per_pass b in
  * 2 .. min(L+1, 4) with sub[0] a power of two in 4..128 advances each

@@ -44,12 +44,17 @@ namespace atk {
 // the system, whose threads hold every field's window, 256
 constexpr int v4_min_ctas(int nf, int nt) { return nf == 1 ? 512 / nt : nt <= 64 ? 256 / nt : nt == 128 ? 2 : 1; }
 
-// Free running, a face whose neighbour lags (by at most L) gets this long to
-// bring level n itself before the delay is taken.  A team that is ahead of its
-// neighbours loses nothing by it, since they set the pace, and stays nearer to
-// them: 16 levels of the 5-field system on 256^3 points take 4.49 ms with 0, 4,
-// 10 and 30 us, at mean delays of 0.08, 0.040, 0.022 and 0.010 (the kernel
-// before, 8.0 ms and 0.029) and errors of 14, 7.3, 4.8 and 3.2e-7 (4.9e-7).
+// Free running, a face whose neighbour lags (by at most L) gets this long to bring
+// level n itself before the delay is taken (at.h says so; at_stepper3d and the
+// blocked kernel take what is there at once).  A team ahead of its neighbours stays
+// nearer to them by it.  Mean delay, relative error against delay 0 and time a level,
+// without the wait, with 10 and with 20 us (in brackets the kernel before this one,
+// which had none):
+//   5 fields of 256^3 in 16^3, 16 levels  0.091 2.8e-6 263 us  0.019 1.3e-6 248  0.011 8.5e-7 250  (0.030 1.2e-6 458)
+//   256^3 in 16^3, 24 levels              0.104 4.5e-6  55     0.041 2.6e-6  59  0.003 5.1e-7  58  (0.102 2.9e-6 211)
+//   512^3 in 32^3, 24 levels              0.053 3.0e-7 262     0.025 2.8e-7 266  0.013 2.2e-7 266  (0.097 3.9e-7 333)
+// (barrier per level: 268, 58 and 249 us).  So it pays in time for several fields and
+// costs the scalar equation 2 to 6 %, for delays a tenth to a quarter as large.
 constexpr long long kGraceNs = 20000;
 
 // grid barrier before level `step` (1-based within the launch), one arrival per
