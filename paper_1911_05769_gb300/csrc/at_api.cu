@@ -339,6 +339,10 @@ TabSize tab_size(int64_t M, int w, bool forced, bool batch, bool comp = false, i
     return {0, 0, comp, 0, 0, 1};
 }
 
+// x / cA in FP32, the factor beside cA in the update (0 where the time step is so
+// short that cA is 0 in FP32: nothing moves, as cA times anything finite is 0).
+float factor32(double x, float cA) { return cA != 0.0f ? (float)(x / (double)cA) : 0.0f; }
+
 // Lets a kernel take all the dynamic shared memory its static one leaves.
 // (The limit belongs to the kernel, not to a solver: a smaller one set for one
 // solver would fail another's launches.)
@@ -1092,8 +1096,8 @@ static atk::Params make_params(const at_solver *h)
     p.cA32 = (float)p.cA;
     p.cB32 = (float)p.cB;
     // (the factors of the rounded cA: their products with it are rounded once)
-    p.cr32 = (float)(p.cB / (double)p.cA32);
-    p.fX32 = (float)(h->v64 ? p.fX : h->dt * h->g.forcing_amp / (double)p.cA32);
+    p.cr32 = factor32(p.cB, p.cA32);
+    p.fX32 = h->v64 ? (float)p.fX : factor32(h->dt * h->g.forcing_amp, p.cA32);
     p.gpl = h->gpl;
     const atk::Swizzle swz = atk::Swizzle::of(h->gpl * h->w / 4);
     p.swz_shift = swz.shift;
@@ -1499,7 +1503,7 @@ int at_create_batch(const at_grid *grid, int64_t n_inst, const at_instance *inst
             b.cA = a.dt / ((scheme_order == 2 ? 2.0 : 12.0) * dx);
             b.cr = (scheme_order == 2 ? 2.0 : 1.0) * a.nu / dx;
             b.cA32 = (float)b.cA;
-            b.cr32 = (float)(cB / (double)b.cA32);
+            b.cr32 = factor32(cB, b.cA32);
             b.seed = a.seed;
             b.L = a.L;
             b.lp = (int)lp;
