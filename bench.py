@@ -38,6 +38,7 @@ METRIC = "grid-point updates/sec (GPts/s), AT vs synchronous, 1D forced Burgers 
 UNIT = "GPts/s"
 FALLBACK_HBM = 6800.0
 KERNEL_SOURCES = ["paper_1911_05769_gb300/csrc/at_kernels.cuh", "paper_1911_05769_gb300/csrc/at_device.cuh",
+                  "paper_1911_05769_gb300/csrc/at_items.cuh",
                   "paper_1911_05769_gb300/csrc/at_kernels_f32.cu"]
 PROFILE = os.path.join(ROOT, "profiles", "at_stepper_f32_o4_n2p26.md")
 

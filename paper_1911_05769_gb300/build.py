@@ -1,6 +1,6 @@
 """Builds the CUDA library ``libat.so`` in-tree for sm_103a with nvcc.
 
-Fifteen translation units (host ABI; FP32 and FP64 single-domain kernels;
+Twenty translation units (host ABI; FP32 and FP64 single-domain kernels;
 FP32 and FP64 ensemble kernels; adjoint kernels; FP32 kernels with FP64
 viscous accumulation; single-domain and ensemble FP32 kernels with a
 compensated state; blocked synchronous kernels for FP32, FP32 with FP64

@@ -400,7 +400,7 @@ __global__ void __launch_bounds__(kAdjThreads, ORDER == 2 ? 7 : 3) at_adjoint_in
 // hears from its neighbours is one message per face and level:
 //   * the adjoint of its halo values at level n (src: R words, from lambda^{n+1}
 //     and u^n at its own edge points) goes out at the start of the level, as one
-//     16-byte access with the level's tag (see EntryTag in at_kernels.cuh);
+//     16-byte access with the level's tag (see st_entry in at_kernels.cuh);
 //   * a warp that receives the message of level n adds w_m(k) src to its own
 //     pending words of level n - k - m, k the neighbour's delay (prescribed, so
 //     known to both sides): the pending ring is private, in shared memory;

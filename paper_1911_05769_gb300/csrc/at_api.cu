@@ -1072,11 +1072,9 @@ static atk::Params make_params(const at_solver *h)
     if (h->comp) p.ur = h->ws + h->lay.ur;
     p.strip = h->ws + h->lay.strip;
     p.ntiles = h->P;
-    p.ktile = 1;
     if (h->batch) {
         p.tiles = reinterpret_cast<const int4 *>(h->ws + h->lay.tiles);   // one subdomain per tile
         p.sub_order = reinterpret_cast<const int *>(h->ws + h->lay.order);
-        p.ktile = h->K;
         p.bsub = reinterpret_cast<const atk::BatchSub *>(h->ws + h->lay.bsub);
         p.binst = reinterpret_cast<const atk::BatchInst *>(h->ws + h->lay.binst);
     }
@@ -1105,7 +1103,6 @@ static atk::Params make_params(const at_solver *h)
     p.x0 = h->g.origin[0];
     p.dx = h->dx;
     p.G = h->G;
-    p.E = h->G * atk::kWarps;
     p.stages = h->stages;
     p.smax = h->smax;
     p.raw_off = h->sl.raw_off;
@@ -1135,7 +1132,7 @@ int at_set_state(at_solver *h, const void *u)
         e = cudaLaunchKernel(h->init_kernel, dim3(blocks), dim3(atk::kThreads3), args, 0, h->stream);
         if (e != cudaSuccess) return cuda_fail(e, "launch at_init3d");
         h->step = 0;
-            h->has_state = true;
+        h->has_state = true;
         return AT_OK;
     }
     e = cudaMemsetAsync(h->ws + h->lay.ring, 0, h->lay.ctrl - h->lay.ring, h->stream);

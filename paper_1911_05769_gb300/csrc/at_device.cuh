@@ -1,11 +1,11 @@
 // at_device.cuh -- device primitives of the persistent AT stepper (sm_103a).
 //
-// Inline PTX for the pieces the kernel needs: shared-memory mbarriers
-// (pipeline full/empty signalling), cp.async 16-byte copies whose completion
-// arrives on an mbarrier, gpu-scope release/acquire on the progress flags
-// (the device counterpart of the notified put / notification test of
-// Algorithm 2), the global nanosecond timer that bounds every wait, and the
-// SplitMix64 generator for prescribed delays.
+// Inline PTX for the pieces the kernels need: 16-byte asynchronous copies, words
+// with their level tag as one 16-byte access (the device counterpart of Algorithm
+// 2's notified put: data and notification arrive together), shared-memory mbarriers
+// and tensor copies with gpu-scope release/acquire on the progress flags (3D), the
+// global nanosecond timer that bounds every wait, and the SplitMix64 generator for
+// prescribed delays.
 #pragma once
 
 #include <cstdint>
@@ -24,7 +24,7 @@ enum : int {
     kCtrlStatus = 0, kCtrlAbort = 1, kCtrlCta = 2, kCtrlWhere = 3, kCtrlNb = 4, kCtrlStep = 5,
     kCtrlN0 = 8, kCtrlDone = 10, kCtrlWords = 16
 };
-enum : int { kWhereTile = 1, kWhereRing = 2, kWhereFlag = 3, kWhereGrid = 4, kWhereAdjoint = 5 };
+enum : int { kWhereTile = 1, kWhereFlag = 3, kWhereGrid = 4, kWhereAdjoint = 5 };
 constexpr int kStatusTimeout = -5;
 
 __device__ __forceinline__ unsigned smem_addr(const void *p)
@@ -51,13 +51,6 @@ __device__ __forceinline__ void mbar_arrive(uint64_t *bar)
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_addr(bar)) : "memory");
 }
 
-// Arrival triggered when all cp.async copies issued so far by this thread
-// have landed; counts as one of the barrier's expected arrivals.
-__device__ __forceinline__ void mbar_arrive_on_copies(uint64_t *bar)
-{
-    asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(smem_addr(bar)) : "memory");
-}
-
 // One bounded probe of the phase with the given parity (acquire at CTA scope).
 __device__ __forceinline__ bool mbar_try_wait(uint64_t *bar, unsigned parity)
 {
@@ -79,7 +72,7 @@ __device__ __forceinline__ void cp_async16(void *dst_smem, const void *src_gmem)
                  : "memory");
 }
 
-// ---- bulk copy (TMA engine, async proxy) -----------------------------------
+// ---- tensor copy (TMA engine, async proxy) ---------------------------------
 // Arrival that also announces `bytes` of asynchronous transactions.
 __device__ __forceinline__ void mbar_arrive_expect_tx(uint64_t *bar, unsigned bytes)
 {
@@ -87,27 +80,9 @@ __device__ __forceinline__ void mbar_arrive_expect_tx(uint64_t *bar, unsigned by
                  : "memory");
 }
 
-// Contiguous global -> shared copy of `bytes` (multiple of 16, both ends
-// 16-byte aligned) whose completion is counted on `bar`.
-__device__ __forceinline__ void bulk_load(void *dst_smem, const void *src_gmem, unsigned bytes, uint64_t *bar)
-{
-    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-                 ::"r"(smem_addr(dst_smem)), "l"(src_gmem), "r"(bytes), "r"(smem_addr(bar))
-                 : "memory");
-}
-
-// Tiled tensor copy (TMA): the box of a 3D tensor map at element coordinates
-// (x, y, z) into shared memory, completion counted on `bar`.  x times the
+// Tiled tensor copy (TMA): the box of a 4D tensor map at element coordinates
+// (x, y, z, w) into shared memory, completion counted on `bar`.  x times the
 // element size must be a multiple of 16 bytes.
-__device__ __forceinline__ void tensor_load_3d(void *dst_smem, const void *tmap, int x, int y, int z, uint64_t *bar)
-{
-    asm volatile(
-        "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];"
-        ::"r"(smem_addr(dst_smem)), "l"(tmap), "r"(x), "r"(y), "r"(z), "r"(smem_addr(bar))
-        : "memory");
-}
-
-// The same for a 4D tensor map (element coordinates x, y, z, w).
 __device__ __forceinline__ void tensor_load_4d(void *dst_smem, const void *tmap, int x, int y, int z, int w,
                                                uint64_t *bar)
 {
@@ -143,11 +118,6 @@ __device__ __forceinline__ void cp_async_wait(int n)
     case 6: asm volatile("cp.async.wait_group 6;" ::: "memory"); break;
     default: asm volatile("cp.async.wait_group 7;" ::: "memory"); break;
     }
-}
-
-__device__ __forceinline__ void cp_async_wait_all()
-{
-    asm volatile("cp.async.wait_all;" ::: "memory");
 }
 
 // ---- gpu-scope release / acquire ------------------------------------------

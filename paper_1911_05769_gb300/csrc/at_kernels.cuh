@@ -153,7 +153,7 @@ struct BatchInst {
 };
 static_assert(sizeof(BatchInst) == 64, "BatchInst is 64 bytes");
 
-// A tile of an ensemble launch: cnt (1..ktile) consecutive subdomains s0 ..
+// A tile of an ensemble launch: cnt consecutive subdomains s0 ..
 // s0+cnt-1 of one instance, advanced together (the faces between them at
 // delay 0: the neighbour's level itself).  Tiles are listed in the order the
 // processing elements sweep them (instances grouped by delay bound); rec is
@@ -189,7 +189,6 @@ struct Params {
     const int *sub_order;      // ensembles: subdomain at each place of the tile lists' enumeration [P]
     TileSplit split;
     long long ntiles;          // tiles of the launch (single domain: P, tile j = subdomain j)
-    int ktile;                 // most subdomains per tile
     void *ur;                  // compensated state: the rounding error of every point (N words)
     unsigned char *strip;      // blocked synchronous mode: edge strips [2][P][2] of kStripBytes (pass parity)
     int strip_words;           // words per strip (R x levels per pass, rounded up to a multiple of 4)
@@ -206,7 +205,6 @@ struct Params {
     float cA32, cB32, cr32, fX32;   // the same in FP32 (no conversion per tile)
     double x0, dx;
     int G;                     // CTAs
-    int E;                     // PEs = G * kWarps
     int stages;                // tile buffers per PE
     int gpl;                   // groups of 4 points per lane
     int swz_shift, swz_mask;   // place of a tile's chunks in its stage (see Swizzle)
@@ -215,7 +213,7 @@ struct Params {
     int tab_words;             // words of a forcing table (M, padded)
     long long raw_off, stage_off, tab_off;
     long long timeout_ns;
-    int skip_publish;          // test knob: PE 0 stops releasing flags
+    int skip_publish;          // test knob: the first tile's PE stops publishing
     long long skip_step;
 };
 
@@ -595,7 +593,7 @@ static __device__ __noinline__ bool cta_grid_sync(const Params &p, int *s_count,
 // of one level while the level is below s-1, then of sb levels (the last one
 // shorter).  sb may differ between PEs (in an ensemble each PE takes the
 // smallest delay bound of its subdomains): a PE's halo waits only need its
-// neighbours' per-level flags, whatever their pass boundaries.
+// neighbours' ring entries level by level, whatever their pass boundaries.
 //
 // The sweep direction alternates from pass to pass (lo..hi-1, then
 // hi-1..lo, ...).  A pass of L+1 levels must start from its edge neighbours'
@@ -709,7 +707,7 @@ __device__ __forceinline__ T exact_ghost2(const BatchInst *binst, const BatchSub
 // A PE with one subdomain keeps it in registers for the whole launch.
 //
 // Halo values come from the ring entries of the neighbour's boundary words;
-// an entry's halves carry the level they belong to (see EntryTag), written and
+// an entry's halves carry the level they belong to (see st_entry), written and
 // read as single 16-byte accesses, so an entry is its own notification: one
 // read tells whether the level is there and brings it (a flag released after
 // the entry costs the writer a fence and the reader a second trip to the L2
@@ -955,8 +953,6 @@ __device__ void run_pe(const Params &p, const Sweep &sw, long long lo, int S, un
     // level n - k among the face's entries.  Returns false on abort.
     auto wait_entries = [&](const Cursor &c, int &k, int &first) -> bool {
         const int cnt = (h_k + h_kmax == 0 && c.len == 1) ? 1 : h_kmax + S_LEV;
-        const bool any = __any_sync(kAll, h_act);
-        (void)any;
         const bool face = ((__ballot_sync(kAll, h_act) >> (lane & 16)) & 0xffffu) != 0u;   // (no exact boundary)
         int base = 0;                  // offset of this lane's first entry
         const unsigned long long t0 = global_ns();

@@ -581,7 +581,7 @@ __device__ __forceinline__ void init_rows(const T *row_a, const T *row_b, unsign
 }
 
 // A block takes one field of one subdomain at a time and copies its faces in
-// pairs, x faces word by word, y and z faces in 16-byte groups where rows allow.
+// pairs, x faces word by word, y and z faces in 16-byte groups.
 // Bound by memory: the x faces touch half the state's sectors.  (One thread per
 // word with its place from 64-bit divisions was bound by those: 512^3 FP32 points
 // in 32^3 subdomains took 313 us; set_state, 24 levels and the state back 5.87 ms
@@ -592,7 +592,7 @@ __global__ void __launch_bounds__(kThreads3) at_init3d(const Params3 p)
     const unsigned m0 = p.m0, m1 = p.m1, m2 = p.m2, nf = p.nf;
     const size_t row = (size_t)p.n0, plane = (size_t)(p.n0 * p.n1);
     const unsigned uP0 = (unsigned)p.P0, uP1 = (unsigned)p.P1;
-    const bool groups = m0 % 4 == 0;                         // (then n0 and every array's words are multiples of 4)
+    // (m0 is a multiple of 4, and so n0 and every array's words)
     for (long long item = blockIdx.x; item < p.P * (int)nf; item += gridDim.x) {
         const unsigned sub = (unsigned)(item / nf), fld = (unsigned)(item - (long long)sub * nf);
         const unsigned q1 = sub / uP0, s0 = sub - q1 * uP0, s2 = q1 / uP1, s1 = q1 - s2 * uP1;
@@ -607,13 +607,8 @@ __global__ void __launch_bounds__(kThreads3) at_init3d(const Params3 p)
             x0[e] = r[0];
             x1[e] = r[m0 - 1];
         }
-        if (groups) {
-            init_rows<T, 4>(u, u + (m1 - 1) * row, m0, m2, plane, face(2), face(3));
-            init_rows<T, 4>(u, u + (m2 - 1) * plane, m0, m1, row, face(4), face(5));
-        } else {
-            init_rows<T, 1>(u, u + (m1 - 1) * row, m0, m2, plane, face(2), face(3));
-            init_rows<T, 1>(u, u + (m2 - 1) * plane, m0, m1, row, face(4), face(5));
-        }
+        init_rows<T, 4>(u, u + (m1 - 1) * row, m0, m2, plane, face(2), face(3));
+        init_rows<T, 4>(u, u + (m2 - 1) * plane, m0, m1, row, face(4), face(5));
         if (fld == 0 && threadIdx.x < 6) p.flag[(size_t)sub * 6 + threadIdx.x] = 0ull;
     }
     if (blockIdx.x == 0) {
