@@ -178,7 +178,6 @@ struct TileSplit {
 struct Params {
     void *u;                   // state, N words, updated in place
     unsigned char *ring;       // [T][P][2] entries (see entry_halves)
-    int nh;                    // halves of an entry
     int *ctrl;                 // control block (status, abort, diagnostics)
     unsigned long long *hist;  // [L+1] delay counts
     unsigned long long *gbar;  // grid-barrier arrival counter (AT_SYNC)
@@ -205,6 +204,7 @@ struct Params {
     float cA32, cB32, cr32, fX32;   // the same in FP32 (no conversion per tile)
     double x0, dx;
     int G;                     // CTAs
+    int nh;                    // halves of an entry
     int stages;                // tile buffers per PE
     int gpl;                   // groups of 4 points per lane
     int swz_shift, swz_mask;   // place of a tile's chunks in its stage (see Swizzle)
@@ -403,8 +403,8 @@ __device__ __forceinline__ T forcing_point(T fs, T fc, T sv, T cv)
 // RMS error up to 1.7 times this one at order 4 and steps of 3e-8 to 1e-7).  The
 // increment is formed apart from lo and meets it in one rounding, by the last factor's
 // multiply-add: increments are often smaller than lo there, and added to it term by
-// term they were rounded at its magnitude two or three times (1.02 to 2 times the
-// error at steps of 1e-8 and less).
+// term they were rounded at its magnitude two or three times (up to 3 times the
+// error at steps of 1e-9, 1.2 to 1.6 at 1e-8).
 //
 // Every operation is written as the one instruction it is, so that a point
 // computed twice -- by its owner in group(), by a neighbour as a ghost cell in
@@ -812,7 +812,10 @@ __device__ void run_pe(const Params &p, const Sweep &sw, long long lo, int S, un
     const unsigned tmask = (unsigned)p.T - 1u;
     const unsigned n0lo = (unsigned)sw.n0;
     const unsigned long long tag0 = entry_tag(sw.n0);    // tag of relative level 0
-    const bool stop_pub = p.skip_publish && lo == 0;   // (test knob: the first tile's owner)
+    // (test knob: the first tile's owner; in FP64 the first warp, which has a tile)
+    bool stop_pub;
+    if constexpr (sizeof(T) == 8) stop_pub = p.skip_publish && blockIdx.x == 0 && threadIdx.x < 32;
+    else stop_pub = p.skip_publish && lo == 0;
     const T fX = sizeof(T) == 4 ? (T)p.fX32 : (T)p.fX;
     const int err_off = p.stage_bytes / 2;               // (compensated state: the error words of a tile)
     const Swizzle swz = FULL ? Swizzle::of(NCH) : Swizzle{p.swz_shift, p.swz_mask};
@@ -1502,16 +1505,18 @@ __device__ void run_pe(const Params &p, const Sweep &sw, long long lo, int S, un
 // ---------------------------------------------------------------------------
 // the persistent kernel
 // ---------------------------------------------------------------------------
-// (a compensated state in short runs: three CTAs an SM in 168 registers, which are a
-// few short of what two groups a lane would take: 4800 subdomains of 256 points 5.0
-// us a seeded level, 6.1 with two)
-constexpr int stepper_min_ctas(int prec, int gw)
+// (a compensated state in runs of one and two groups a lane, and of four at order 2
+// unforced: the registers that three CTAs an SM leave, or four, are a few short of
+// what the compiler would take: 4800 subdomains of 256 points, order 4, 5.0 us a
+// seeded level, 6.1 with a CTA less)
+constexpr int stepper_min_ctas(int order, int gw, bool forced, bool batch, int prec)
 {
-    return prec == 2 && gw <= 2 && AT_MIN_CTAS_PER_SM < 3 ? 3 : AT_MIN_CTAS_PER_SM;
+    if (prec != 2) return AT_MIN_CTAS_PER_SM;
+    return gw == 1 && !forced && !batch ? 4 : gw <= 2 || (gw == 4 && order == 2 && !forced && !batch) ? 3 : AT_MIN_CTAS_PER_SM;
 }
 
 template <typename T, int ORDER, int GW, bool FORCED, bool FULL, bool BATCH, int PREC, bool BS>
-__global__ void __launch_bounds__(kThreads, stepper_min_ctas(PREC, GW)) at_stepper(const Params p)
+__global__ void __launch_bounds__(kThreads, stepper_min_ctas(ORDER, GW, FORCED, BATCH, PREC)) at_stepper(const Params p)
 {
     extern __shared__ __align__(128) unsigned char smem[];
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
