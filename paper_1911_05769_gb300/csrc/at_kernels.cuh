@@ -696,8 +696,8 @@ __device__ __forceinline__ T exact_ghost2(const BatchInst *binst, const BatchSub
 // of 4 levels, 10 of them arithmetic.  (Interleaved runs of two groups per lane
 // take four times the shuffles and a select per exchanged word, 23.8.  2^26
 // points, FP32, 100 levels: 5.91 ms then, 4.27 ms so; the compensated state on
-// 2^24 points 3.62 and 2.03 ms; FP64 on 2^22 points, 40 levels, bound by its
-// FP64 pipe, 4.48 and 3.63 ms.)
+// 2^24 points 3.62 and 2.03 ms (2.06 with its exact differences kept apart); FP64
+// on 2^22 points, 40 levels, bound by its FP64 pipe, 4.48 and 3.63 ms.)
 //
 // The tile travels through a shared-memory stage: 16-byte asynchronous copies
 // in, coalesced in global memory and swizzled in the stage (see swizzle()), so
